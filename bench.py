@@ -102,8 +102,8 @@ def measured_peaks() -> dict:
 _COMMON = ["cg_device.cuh", "layout.h"]
 KERNEL_SOURCES = {
     "cg_solve_kernel": ["gbcg.cu", "plan.h"] + _COMMON,
-    "cg_sell_kernel": ["gbcg.cu", "sell.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
-    "cg_sellmem_kernel": ["gbcg.cu", "sell.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
+    "cg_sell_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
+    "cg_sellmem_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "sell_spmv_kernel": ["gbcg.cu", "sell.cuh", "plan.h"],
     "cg_ir_kernel": ["gbcg.cu", "plan.h", "lowprec.h"] + _COMMON,
     "cg_irsell_kernel": ["gbcg.cu", "sell.cuh", "sellsolve.cuh", "plan.h", "lowprec.h"] + _COMMON,

@@ -95,10 +95,11 @@ typedef struct {
                                 wait for this many CTAs that never arrive, so
                                 every wait runs out and the solve returns
                                 CG_ETIMEOUT without hanging the device            */
-    int32_t vectors_in_memory; /* 0 (default): when every thread owns at most 4
-                                rows, the solver keeps x, r, z, p, q and 1/diag of
-                                those rows in registers for the whole solve;
-                                1: always keep every vector in device memory     */
+    int32_t vectors_in_memory; /* 0 (default): FP64 solves run the SELL-32 kernels,
+                                which keep the vectors of systems with at most one
+                                32-row slice per warp in registers for the whole
+                                solve; 1: the tiled kernel, every vector in device
+                                memory                                            */
     int32_t inner_values;    /* CG_VALUES_*; default CG_VALUES_FP64.  FP32/BF16
                                 turn the solve into iterative refinement: the
                                 outer loop keeps x and r = b - A x in FP64 with
@@ -143,15 +144,17 @@ typedef struct {
     int32_t smem_bytes;      /* dynamic shared memory per CTA                     */
     int32_t lanes_per_row;   /* threads that share one row in the SpMV            */
     int32_t l2_evict_first;  /* 1 when the matrix stream is marked evict-first    */
-    int32_t reg_rows;        /* rows per thread held in registers (0: none)       */
+    int32_t reg_rows;        /* rows per thread if each thread of the tiled plan
+                                held its rows in registers: 1, 2 or 4; 0: more, or
+                                vectors_in_memory                                 */
     int32_t window_tiles;    /* tiles whose gathers read a staged x-window        */
     int64_t device_bytes;    /* device memory the handle owns                     */
     int32_t slice_solve;     /* FP64 solves run: 1 the SELL-32 kernel with one
                                 32-row slice per warp and rows in registers; 2
                                 the SELL-32 kernel with the vectors in memory
-                                (systems too large for 1 and for register rows
-                                in the tiled kernel); 0 the tiled kernel
-                                described by the fields above                    */
+                                (reg_rows 0); 0 that kernel too when reg_rows is
+                                not 0, else the tiled kernel described by the
+                                fields above                                     */
     int32_t inner_solve;     /* handles with inner_values FP32/BF16: 1 when the
                                 refinement runs on SELL-32 copies (one 32-row
                                 slice per warp), 0 when it runs on the staged

@@ -46,19 +46,6 @@ static_assert(sizeof(I4) == sizeof(int4), "tile descriptor layout");
 
 namespace {
 
-// ------------------------------------------------------------ row state
-// With RPT > 0 every thread keeps the vector entries of the rows it owns
-// (lane l of warp w owns row r0 + l of each of the warp's tiles) in
-// registers for the whole solve: x, r, z, p, q and 1/diag never round-trip
-// through memory; only p is published (the SpMV gathers it) and x is written
-// at the end.  RPT = 0 keeps every vector in global memory.
-template <int RPT>
-struct RegRows {
-    int row[RPT > 0 ? RPT : 1];
-    double x[RPT > 0 ? RPT : 1], r[RPT > 0 ? RPT : 1], z[RPT > 0 ? RPT : 1];
-    double p[RPT > 0 ? RPT : 1], q[RPT > 0 ? RPT : 1], dinv[RPT > 0 ? RPT : 1];
-};
-
 // ------------------------------------------------------------ epilogues
 struct EpiSetup {       // r = b - A x0, z = M^-1 r (gathered), p = z, q = 0; sums r.r, r.z, b.b
     const double *b;
@@ -88,28 +75,6 @@ struct EpiSetup {       // r = b - A x0, z = M^-1 r (gathered), p = z, q = 0; su
     }
 };
 
-template <int RPT>
-struct RegSetup {       // the same, into registers (p is also published)
-    RegRows<RPT> &R;
-    const double *b;
-    double *p;
-    int precond;
-    double rr = 0.0, rz = 0.0, bb = 0.0;
-    __device__ __forceinline__ void row(int i, double ax, int j) {
-        const double bi = b[i];
-        const double ri = bi - ax;
-        const double zi = precond ? R.dinv[j] * ri : ri;
-        R.r[j] = ri;
-        R.z[j] = zi;
-        R.p[j] = zi;
-        R.q[j] = 0.0;
-        p[i] = zi;
-        rr = fma(ri, ri, rr);
-        rz = fma(ri, zi, rz);
-        bb = fma(bi, bi, bb);
-    }
-};
-
 struct EpiIter {        // p = z + beta p, q = A z + beta q; sum p . q
     double *q;
     double *pd;
@@ -127,20 +92,6 @@ struct EpiIter {        // p = z + beta p, q = A z + beta q; sum p . q
         const double pi = fma(beta, pi_, zi_);
         q[i] = qi;
         pd[i] = pi;
-        pq = fma(pi, qi, pq);
-    }
-};
-
-template <int RPT>
-struct RegIter {
-    RegRows<RPT> &R;
-    double beta;
-    double pq = 0.0;
-    __device__ __forceinline__ void row(int, double az, int j) {
-        const double qi = fma(beta, R.q[j], az);
-        const double pi = fma(beta, R.p[j], R.z[j]);
-        R.q[j] = qi;
-        R.p[j] = pi;
         pq = fma(pi, qi, pq);
     }
 };
@@ -165,12 +116,12 @@ struct EpiStore {       // y = A x
 constexpr int kCtlRun = 0;       // 1: continue iterating
 constexpr int kCtlZeroB = 2;     // 1: b = 0, so x = 0
 constexpr int kCtlTrue = 3;      // 1: compute the true residual
+constexpr int kCtlShift = 4;     // fixed-point shift of the published z
 
 // ------------------------------------------------------- the solve kernel
 // Scalar recurrences (alpha, beta, the stop test) run in thread 0 only: on
 // GB300 an FP64 divide or square root executed by every warp would cost the
 // FP64 pipe as much as a tile of the SpMV.
-template <int RPT>
 __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const Smem S = carve_smem(smem_raw);
@@ -186,41 +137,13 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
     // thread 0's scalar state
     int status = CG_OK, iters = 0;
     double rr = 0.0, bb = 0.0, true_rr = -1.0, rho = 0.0, bnorm = 0.0;
-    RegRows<RPT> R;
-    if constexpr (RPT > 0) {
-        const int t0 = P.cta_tile[blockIdx.x], nt = P.cta_tile[blockIdx.x + 1] - t0;
-        const int w = tid >> 5, lane = tid & 31;
-#pragma unroll
-        for (int j = 0; j < RPT; ++j) {
-            R.row[j] = -1;
-            R.x[j] = 0.0;
-            R.dinv[j] = 1.0;
-            const int t = w + kWarps * j;
-            if (t < nt) {
-                const TileDesc d = load_desc(P, t0 + t);
-                const int row = d.r0 + lane;
-                if (row < d.r1) {
-                    R.row[j] = row;
-                    R.x[j] = P.x[row];
-                    if (P.precond) R.dinv[j] = P.dinv[row];
-                }
-            }
-        }
-    }
-
     // ---- setup: r0 = b - A x0, z0 = M^-1 r0, p0 = z0; r.r, r.z, b.b
     bool run;
     {
         double v[3];
-        if constexpr (RPT > 0) {
-            RegSetup<RPT> epi{R, P.b, p, P.precond};
-            if (!spmv_tiles<RPT, double, double, double>(P, S, pipe, P.vals, P.x, epi)) goto out;
-            v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
-        } else {
-            EpiSetup epi{P.b, P.r, P.z, p, P.pd, P.q, P.dinv, P.precond};
-            if (!spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, P.x, epi)) goto out;
-            v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
-        }
+        EpiSetup epi{P.b, P.r, P.z, p, P.pd, P.q, P.dinv, P.precond};
+        if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, epi)) goto out;
+        v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
         block_sum<3>(v, S);
         publish_partials<3>(P, set, v);
         if (!grid_barrier(P, epoch, S)) goto out;
@@ -252,14 +175,8 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         }
         __syncthreads();
         run = S.ctl[kCtlRun] != 0;
-        if (S.ctl[kCtlZeroB]) {  // b = 0: the solution is x = 0
-            if constexpr (RPT > 0) {
-#pragma unroll
-                for (int j = 0; j < RPT; ++j) R.x[j] = 0.0;
-            } else {
-                for (int i = row_lo + tid; i < row_hi; i += kThreads) P.x[i] = 0.0;
-            }
-        }
+        if (S.ctl[kCtlZeroB])  // b = 0: the solution is x = 0
+            for (int i = row_lo + tid; i < row_hi; i += kThreads) P.x[i] = 0.0;
     }
 
     // ---- the CG loop
@@ -268,17 +185,9 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         double beta = 0.0;  // p_1 = z_0 and q_1 = A z_0
         for (int k = 1; k <= P.maxit; ++k) {
             // phase A: p = z + beta p, q = A z + beta q (= A p), p . q
-            double pq;
-            if constexpr (RPT > 0) {
-                RegIter<RPT> ei{R, beta};
-                if (!spmv_tiles<RPT, double, double, double>(P, S, pipe, P.vals, p, ei)) goto out;
-                pq = ei.pq;
-            } else {
-                EpiIter ei{P.q, P.pd, p, beta};
-                if (!spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, p, ei)) goto out;
-                pq = ei.pq;
-            }
-            double v1[1] = {pq};
+            EpiIter ei{P.q, P.pd, p, beta};
+            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, p, ei)) goto out;
+            double v1[1] = {ei.pq};
             block_sum<1>(v1, S);
             publish_partials<1>(P, set, v1);
             if (!grid_barrier(P, epoch, S)) goto out;
@@ -301,37 +210,18 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
             // phase B: x += alpha p, r -= alpha q, z = dinv r (published for
             // the next SpMV: every gather of phase A is over); r.r, r.z
             double prr = 0.0, prz = 0.0;
-            if constexpr (RPT > 0) {
-#pragma unroll
-                for (int j = 0; j < RPT; ++j) {
-                    if (R.row[j] >= 0) {
-                        R.x[j] = fma(alpha, R.p[j], R.x[j]);
-                        const double ri = fma(-alpha, R.q[j], R.r[j]);
-                        R.r[j] = ri;
-                        prr = fma(ri, ri, prr);
-                        double zi = ri;
-                        if (P.precond) {
-                            zi = R.dinv[j] * ri;
-                            prz = fma(ri, zi, prz);
-                        }
-                        R.z[j] = zi;
-                        p[R.row[j]] = zi;
-                    }
+            for (int i = row_lo + tid; i < row_hi; i += kThreads) {
+                const double pi = P.pd[i], qi = P.q[i], xi = P.x[i], ri0 = P.r[i];
+                P.x[i] = fma(alpha, pi, xi);
+                const double ri = fma(-alpha, qi, ri0);
+                P.r[i] = ri;
+                prr = fma(ri, ri, prr);
+                double zi = ri;
+                if (P.precond) {
+                    zi = P.dinv[i] * ri;
+                    prz = fma(ri, zi, prz);
                 }
-            } else {
-                for (int i = row_lo + tid; i < row_hi; i += kThreads) {
-                    const double pi = P.pd[i], qi = P.q[i], xi = P.x[i], ri0 = P.r[i];
-                    P.x[i] = fma(alpha, pi, xi);
-                    const double ri = fma(-alpha, qi, ri0);
-                    P.r[i] = ri;
-                    prr = fma(ri, ri, prr);
-                    double zi = ri;
-                    if (P.precond) {
-                        zi = P.dinv[i] * ri;
-                        prz = fma(ri, zi, prz);
-                    }
-                    p[i] = zi;
-                }
+                p[i] = zi;
             }
             double t2[2];
             if (P.precond) {
@@ -373,23 +263,15 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         }
     }
 
-    // ---- publish x (register mode), then the true residual ||b - A x||
-    if constexpr (RPT > 0) {
-#pragma unroll
-        for (int j = 0; j < RPT; ++j)
-            if (R.row[j] >= 0) P.x[R.row[j]] = R.x[j];
-    }
+    // ---- the true residual ||b - A x||
     {
         if (tid == 0) S.ctl[kCtlTrue] = (P.true_res && status != CG_ENAN && bb != 0.0) ? 1 : 0;
         __syncthreads();
         const bool want_true = S.ctl[kCtlTrue] != 0;
         if (tid == 0 && P.true_res && status != CG_ENAN && bb == 0.0) true_rr = 0.0;
         if (want_true) {
-            if constexpr (RPT > 0) {
-                if (!grid_barrier(P, epoch, S)) goto out;  // every x entry is written
-            }
             EpiTrue et{P.b};
-            if (!spmv_tiles<RPT, double, double, double>(P, S, pipe, P.vals, P.x, et)) goto out;
+            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, et)) goto out;
             double v[1] = {et.acc};
             block_sum<1>(v, S);
             publish_partials<1>(P, set, v);
@@ -427,21 +309,25 @@ out:
 // beta = rho'/rho.  The warps then finish q = A z + beta q and p = z + beta p
 // (the last iteration's SpMV is computed and dropped).
 constexpr int kSliceMaxPerCta = kSellSolveThreads / 32 - 1;   // warps 1..31
+constexpr int kFixedUnroll = 9;    // entries in flight per row of the integer product (6: 11.3 against
+                                   // 10.9 us per iteration at 50^3)
 constexpr int kSliceVecCost = 8;   // FP64 vector operations per row, in SpMV-width units
 
-template <bool PRE>
+template <bool PRE, bool FX>
 __global__ void __launch_bounds__(kSellSolveThreads, 1)
-    cg_sell_kernel(Params P, SellMatrix M, const int32_t *__restrict__ cut) {
+    cg_sell_kernel(Params P, SellMatrix M, FixedMatrix F, const int32_t *__restrict__ cut) {
     __shared__ double red[3 * kSellSolveThreads];
     __shared__ double quarter[12];
     __shared__ double bcast[8];
     __shared__ int ctl[16];
     __shared__ long long slice_a[kSellSolveThreads / 32];
     __shared__ int slice_w[kSellSolveThreads / 32];
-    Smem S{};
-    S.red = red;
-    S.bcast = bcast;
-    S.ctl = ctl;
+    __shared__ unsigned int wmax_s[FX ? kMaxSlots : 1];
+    unsigned int *const wmax = FX ? wmax_s : nullptr;
+    Smem SM{};
+    SM.red = red;
+    SM.bcast = bcast;
+    SM.ctl = ctl;
     unsigned int epoch = 0;
     int set = 0;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -450,6 +336,11 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
     const int row = t * 32 + lane;
     const bool own = has_slice && row < P.n;
     double *const zg = P.p0;   // z, gathered by the SpMV
+    int2 *const zx = reinterpret_cast<int2 *>(P.p0);   // FX: its integers instead (fixed.cuh)
+    const int ce = FX && own ? F.c[row] : 0;
+    int S = 0;               // FX: z's shift (every thread)
+    unsigned int mz = 0;     // FX: the bound on z (thread 0)
+    auto bound = [&](double v) { return own ? fixed_ub(v, ce) : 0u; };
 
     // thread 0's scalar state
     int status = CG_OK, iters = 0;
@@ -470,16 +361,17 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             r = bi - ax;
             z = PRE ? __ldg(dinv_g + row) * r : r;
             p = z;
-            zg[row] = z;
+            if constexpr (!FX) zg[row] = z;
             v[0] = r * r;
             v[1] = r * z;
             v[2] = bi * bi;
         }
-        block_sum_1k<3>(v, red, quarter);
+        block_sum_1k<3>(v, red, quarter, wmax, FX ? bound(z) : 0u);
         publish_partials<3>(P, set, v);
-        if (!grid_barrier<false>(P, epoch, S)) goto out;
+        if constexpr (FX) publish_max(P, set, wmax[32]);
+        if (!grid_barrier<false>(P, epoch, SM)) goto out;
         double tot[3];
-        grid_totals_1k<3>(P, set, tot, quarter);
+        grid_totals_1k<3>(P, set, tot, quarter, wmax);
         set ^= 1;
         if (tid == 0) {
             rr = tot[0];
@@ -504,10 +396,21 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             ctl[kCtlRun] = go;
             ctl[kCtlZeroB] = zero_b;
+            if constexpr (FX) {
+                mz = wmax[33];
+                ctl[kCtlShift] = fixed_shift(mz, 0u);
+            }
         }
         __syncthreads();
         run = ctl[kCtlRun] != 0;
         if (ctl[kCtlZeroB]) x = 0.0;  // b = 0: the solution is x = 0
+        if constexpr (FX) {
+            if (run) {   // z_0's integers, now that their shift is known
+                S = ctl[kCtlShift];
+                if (own) zx[row] = fixed_publish(z, ce, S);
+                if (!grid_barrier<false>(P, epoch, SM)) goto out;
+            }
+        }
     }
 
     // ---- the CG loop
@@ -543,14 +446,33 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             slice_w[w] = (int)((M.ptr[t + 1] - slice_a[w]) >> 5);
         }
         __syncwarp();
-        double azl = has_slice ? sell_slice_sum_at(M, t, slice_a[w], slice_w[w], zg, 0.0, 0, wl) : 0.0;
+        double azl = 0.0;
+        FixedAcc acc;
+        auto local_part = [&]() {
+            if constexpr (FX) {
+                acc = FixedAcc{};
+                fixed_slice_sum<kFixedUnroll>(F, P.n, t, slice_a[w], zx, acc, 0, wl);
+            } else {
+                azl = sell_slice_sum_at(M, t, slice_a[w], slice_w[w], zg, 0.0, 0, wl);
+            }
+        };
+        if (has_slice) local_part();
         for (int k = 1;; ++k) {
             // phase A: az = A z on warps 1..31 (the rest of each row, from
             // azl); the control warp decides on iteration k-1 meanwhile
-            const double az = has_slice ? sell_slice_sum_at(M, t, slice_a[w], slice_w[w], zg, azl, wl) : 0.0;
+            double az = 0.0;
+            if (has_slice) {
+                if constexpr (FX) {
+                    fixed_slice_sum<kFixedUnroll>(F, P.n, t, slice_a[w], zx, acc, wl, slice_w[w]);
+                    az = fixed_value(acc, ce - F.u - S);
+                } else {
+                    az = sell_slice_sum_at(M, t, slice_a[w], slice_w[w], zg, azl, wl);
+                }
+            }
             if (k > 1 && w == 0) {
                 double t2[NB];
                 grid_totals<NB>(P, set ^ 1, t2);
+                if constexpr (FX) mz = grid_max(P, set ^ 1);
                 if (tid == 0) decide(k - 1, t2);
             }
             __syncthreads();
@@ -563,11 +485,19 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 p = fma(beta, p, z);
                 v1[0] = p * q;
             }
-            block_sum_1k<1>(v1, red, quarter);
+            // FX: the next z is z - alpha M q, so the bounds on z and on M q
+            // give the bound its shift needs before it is formed
+            unsigned int mq = 0;
+            if constexpr (FX) {
+                mq = bound(q);
+                if (PRE && own) mq = fixed_ub_mul(mq, __ldg(dinv_g + row));
+            }
+            block_sum_1k<1>(v1, red, quarter, wmax, mq);
             publish_partials<1>(P, set, v1);
-            if (!grid_barrier<false>(P, epoch, S)) goto out;
+            if constexpr (FX) publish_max(P, set, wmax[32]);
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;
             double sg[1];
-            grid_totals_1k<1>(P, set, sg, quarter);
+            grid_totals_1k<1>(P, set, sg, quarter, wmax);
             set ^= 1;
             if (tid == 0) {
                 const double sigma = sg[0];
@@ -575,12 +505,15 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                bcast[0] = go ? rho / sigma : 0.0;
+                const double al = go ? rho / sigma : 0.0;
+                bcast[0] = al;
                 ctl[kCtlRun] = go;
+                if constexpr (FX) ctl[kCtlShift] = fixed_shift(mz, fixed_ub_mul(wmax[33], al));
             }
             __syncthreads();
             if (!ctl[kCtlRun]) break;
             const double alpha = bcast[0];
+            if constexpr (FX) S = ctl[kCtlShift];
 
             // phase B: r -= alpha q, z = dinv r (published); r.r, r.z (plain
             // CG: z = r and r.z = r.r, one sum); x += alpha p below
@@ -590,12 +523,14 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             if (own) {
                 r = fma(-alpha, q, r);
                 z = PRE ? __ldg(dinv_g + row) * r : r;
-                zg[row] = z;
+                if constexpr (FX) zx[row] = fixed_publish(z, ce, S);
+                else zg[row] = z;
                 v2[0] = r * r;
                 if constexpr (PRE) v2[NB - 1] = r * z;
             }
-            block_sum_1k<NB>(v2, red, quarter);
+            block_sum_1k<NB>(v2, red, quarter, wmax, FX ? bound(z) : 0u);
             publish_partials<NB>(P, set, v2);
+            if constexpr (FX) publish_max(P, set, wmax[32]);
             // the barrier that publishes z: the warps with a slice add its
             // entries in this CTA's own rows (z written before grid_arrive's
             // __syncthreads) while thread 0 waits for the other CTAs
@@ -604,7 +539,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 // x is read by nothing before the end: x += alpha p leaves
                 // the critical path (p changes only in the next phase A)
                 if (own) x = fma(alpha, p, x);
-                azl = sell_slice_sum_at(M, t, slice_a[w], slice_w[w], zg, 0.0, 0, wl);
+                local_part();
             } else if (tid == 0) {
                 ctl[15] = grid_wait<false>(P, epoch);
             }
@@ -631,7 +566,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
         const bool want_true = ctl[kCtlTrue] != 0;
         if (tid == 0 && P.true_res && status != CG_ENAN && bb == 0.0) true_rr = 0.0;
         if (want_true) {
-            if (!grid_barrier<false>(P, epoch, S)) goto out;  // every x entry is written
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;  // every x entry is written
             const double ax = has_slice ? sell_slice_sum(M, t, P.x, 0.0) : 0.0;
             double v[1] = {0.0};
             if (own) {
@@ -640,7 +575,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             block_sum_1k<1>(v, red, quarter);
             publish_partials<1>(P, set, v);
-            if (!grid_barrier<false>(P, epoch, S)) goto out;
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;
             double tt[1];
             grid_totals_1k<1>(P, set, tt, quarter);
             if (tid == 0) true_rr = tt[0];
@@ -668,17 +603,19 @@ out:
 // the same thread.  Two grid barriers per iteration; each decision is taken
 // before the next phase starts.
 
-template <bool PRE>
+template <bool PRE, bool FX>
 __global__ void __launch_bounds__(kSellSolveThreads, 1)
-    cg_sellmem_kernel(Params P, SellMatrix M, const int32_t *__restrict__ cut) {
+    cg_sellmem_kernel(Params P, SellMatrix M, FixedMatrix F, const int32_t *__restrict__ cut) {
     __shared__ double red[3 * kSellSolveThreads];
     __shared__ double quarter[12];
     __shared__ double bcast[8];
     __shared__ int ctl[16];
-    Smem S{};
-    S.red = red;
-    S.bcast = bcast;
-    S.ctl = ctl;
+    __shared__ unsigned int wmax_s[FX ? kMaxSlots : 1];
+    unsigned int *const wmax = FX ? wmax_s : nullptr;
+    Smem SM{};
+    SM.red = red;
+    SM.bcast = bcast;
+    SM.ctl = ctl;
     unsigned int epoch = 0;
     int set = 0;
     constexpr int kW = kSellSolveThreads / 32;
@@ -686,6 +623,9 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
     const int t0 = cut[blockIdx.x] + (tid >> 5), t1 = cut[blockIdx.x + 1];
     double *const zg = P.p0;   // z: the vector the SpMV gathers
     double *const pv = P.pd;   // p
+    int2 *const zx = reinterpret_cast<int2 *>(P.p0);   // FX: z's integers instead (fixed.cuh)
+    int S = 0;               // FX: z's shift (every thread)
+    unsigned int mz = 0;     // FX: the bound on z (thread 0; every thread's own in phase B)
 
     // thread 0's scalar state
     int status = CG_OK, iters = 0;
@@ -695,6 +635,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
     bool run;
     {
         double v[3] = {0.0, 0.0, 0.0};
+        unsigned int mx = 0;
         for (int t = t0; t < t1; t += kW) {
             const double ax = sell_slice_sum<kSellUnrollMem>(M, t, P.x, 0.0);
             const int row = t * 32 + lane;
@@ -703,7 +644,8 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 const double ri = bi - ax;
                 const double zi = PRE ? __ldg(P.dinv + row) * ri : ri;
                 P.r[row] = ri;
-                zg[row] = zi;
+                if constexpr (FX) mx = max(mx, fixed_ub(zi, F.c[row]));
+                else zg[row] = zi;
                 pv[row] = zi;
                 P.q[row] = 0.0;
                 v[0] = fma(ri, ri, v[0]);
@@ -711,11 +653,12 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 v[2] = fma(bi, bi, v[2]);
             }
         }
-        block_sum_1k<3>(v, red, quarter);
+        block_sum_1k<3>(v, red, quarter, wmax, mx);
         publish_partials<3>(P, set, v);
-        if (!grid_barrier<false>(P, epoch, S)) goto out;
+        if constexpr (FX) publish_max(P, set, wmax[32]);
+        if (!grid_barrier<false>(P, epoch, SM)) goto out;
         double tot[3];
-        grid_totals_1k<3>(P, set, tot, quarter);
+        grid_totals_1k<3>(P, set, tot, quarter, wmax);
         set ^= 1;
         if (tid == 0) {
             rr = tot[0];
@@ -740,12 +683,26 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             ctl[kCtlRun] = go;
             ctl[kCtlZeroB] = zero_b;
+            if constexpr (FX) {
+                mz = wmax[33];
+                ctl[kCtlShift] = fixed_shift(mz, 0u);
+            }
         }
         __syncthreads();
         run = ctl[kCtlRun] != 0;
         if (ctl[kCtlZeroB])   // b = 0: the solution is x = 0
             for (int t = t0; t < t1; t += kW)
                 if (t * 32 + lane < P.n) P.x[t * 32 + lane] = 0.0;
+        if constexpr (FX) {
+            if (run) {   // z_0's integers, now that their shift is known (p_0 = z_0)
+                S = ctl[kCtlShift];
+                for (int t = t0; t < t1; t += kW) {
+                    const int row = t * 32 + lane;
+                    if (row < P.n) zx[row] = fixed_publish(pv[row], F.c[row], S);
+                }
+                if (!grid_barrier<false>(P, epoch, SM)) goto out;
+            }
+        }
     }
 
     // ---- the CG loop
@@ -756,22 +713,39 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
         for (int k = 1; k <= P.maxit; ++k) {
             // phase A: q = A z + beta q (= A p), p = z + beta p; p . q
             double v1[1] = {0.0};
+            unsigned int mq = 0;   // FX: bound on M q, from which the next z's shift follows
             for (int t = t0; t < t1; t += kW) {
-                const double az = sell_slice_sum<kSellUnrollMem>(M, t, zg, 0.0);
                 const int row = t * 32 + lane;
+                double az;
+                if constexpr (FX) {
+                    FixedAcc acc;
+                    const long long a = M.ptr[t];
+                    fixed_slice_sum<kFixedUnroll>(F, P.n, t, a, zx, acc, 0, (int)((M.ptr[t + 1] - a) >> 5));
+                    az = row < P.n ? fixed_value(acc, F.c[row] - F.u - S) : 0.0;
+                } else {
+                    az = sell_slice_sum<kSellUnrollMem>(M, t, zg, 0.0);
+                }
                 if (row < P.n) {
+                    double zi;
+                    if constexpr (FX) zi = PRE ? __ldg(P.dinv + row) * P.r[row] : P.r[row];
+                    else zi = zg[row];
                     const double qi = fma(beta, P.q[row], az);
-                    const double pi = fma(beta, pv[row], zg[row]);
+                    const double pi = fma(beta, pv[row], zi);
                     P.q[row] = qi;
                     pv[row] = pi;
                     v1[0] = fma(pi, qi, v1[0]);
+                    if constexpr (FX) {
+                        const unsigned int ub = fixed_ub(qi, F.c[row]);
+                        mq = max(mq, PRE ? fixed_ub_mul(ub, __ldg(P.dinv + row)) : ub);
+                    }
                 }
             }
-            block_sum_1k<1>(v1, red, quarter);
+            block_sum_1k<1>(v1, red, quarter, wmax, mq);
             publish_partials<1>(P, set, v1);
-            if (!grid_barrier<false>(P, epoch, S)) goto out;
+            if constexpr (FX) publish_max(P, set, wmax[32]);
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;
             double sg[1];
-            grid_totals_1k<1>(P, set, sg, quarter);
+            grid_totals_1k<1>(P, set, sg, quarter, wmax);
             set ^= 1;
             if (tid == 0) {
                 const double sigma = sg[0];
@@ -779,12 +753,16 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                bcast[0] = go ? rho / sigma : 0.0;
+                const double al = go ? rho / sigma : 0.0;
+                bcast[0] = al;
                 ctl[kCtlRun] = go;
+                if constexpr (FX) ctl[kCtlShift] = fixed_shift(mz, fixed_ub_mul(wmax[33], al));
             }
             __syncthreads();
             if (!ctl[kCtlRun]) break;
             const double alpha = bcast[0];
+            if constexpr (FX) S = ctl[kCtlShift];
+            mz = 0;
 
             // phase B: x += alpha p, r -= alpha q, z = dinv r (published); r.r, r.z
             double v2[NB];
@@ -797,18 +775,26 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                     P.x[row] = fma(alpha, pv[row], P.x[row]);
                     P.r[row] = ri;
                     const double zi = PRE ? __ldg(P.dinv + row) * ri : ri;
-                    zg[row] = zi;
+                    if constexpr (FX) {
+                        const int c = F.c[row];
+                        zx[row] = fixed_publish(zi, c, S);
+                        mz = max(mz, fixed_ub(zi, c));
+                    } else {
+                        zg[row] = zi;
+                    }
                     v2[0] = fma(ri, ri, v2[0]);
                     if constexpr (PRE) v2[NB - 1] = fma(ri, zi, v2[NB - 1]);
                 }
             }
-            block_sum_1k<NB>(v2, red, quarter);
+            block_sum_1k<NB>(v2, red, quarter, wmax, mz);
             publish_partials<NB>(P, set, v2);
-            if (!grid_barrier<false>(P, epoch, S)) goto out;
+            if constexpr (FX) publish_max(P, set, wmax[32]);
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;
             double t2[NB];
-            grid_totals_1k<NB>(P, set, t2, quarter);
+            grid_totals_1k<NB>(P, set, t2, quarter, wmax);
             set ^= 1;
             if (tid == 0) {
+                if constexpr (FX) mz = wmax[33];
                 iters = k;
                 rr = t2[0];
                 const double rho_new = t2[NB - 1];
@@ -837,7 +823,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
         const bool want_true = ctl[kCtlTrue] != 0;
         if (tid == 0 && P.true_res && status != CG_ENAN && bb == 0.0) true_rr = 0.0;
         if (want_true) {
-            if (!grid_barrier<false>(P, epoch, S)) goto out;  // every x entry is written
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;  // every x entry is written
             double v[1] = {0.0};
             for (int t = t0; t < t1; t += kW) {
                 const double ax = sell_slice_sum<kSellUnrollMem>(M, t, P.x, 0.0);
@@ -849,7 +835,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             block_sum_1k<1>(v, red, quarter);
             publish_partials<1>(P, set, v);
-            if (!grid_barrier<false>(P, epoch, S)) goto out;
+            if (!grid_barrier<false>(P, epoch, SM)) goto out;
             double tt[1];
             grid_totals_1k<1>(P, set, tt, quarter);
             if (tid == 0) true_rr = tt[0];
@@ -945,7 +931,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_ir_kernel(Params P) {
         double rho;
         {
             EpiOuter eo{P.b, P.r32, P.p32, P.pd32, P.q32, P.d32, P.dinv32, P.precond};
-            if (!spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, P.x, eo, true)) goto out;
+            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, eo, true)) goto out;
             double v[3] = {eo.rr, eo.bb, (double)eo.rz};
             block_sum<3>(v, S);
             publish_partials<3>(P, set, v);
@@ -983,7 +969,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_ir_kernel(Params P) {
         float beta = 0.0f;
         for (int k = 1;; ++k) {
             EpiInner ei{P.q32, P.pd32, P.p32, P.diag_lo, beta};
-            if (!spmv_tiles<0, VT, float, float>(P, S, pipe, vlo, P.p32, ei, true)) goto out;
+            if (!spmv_tiles<VT, float, float>(P, S, pipe, vlo, P.p32, ei, true)) goto out;
             double v1[1] = {(double)ei.pq};
             block_sum<1>(v1, S);
             publish_partials<1>(P, set, v1);
@@ -1348,7 +1334,7 @@ __global__ void __launch_bounds__(kThreads, 1) lo_spmv_tiles_kernel(Params P, fl
     if constexpr (sizeof(VT) == 4) vlo = reinterpret_cast<const VT *>(P.vals32);
     else vlo = reinterpret_cast<const VT *>(P.vals16);
     EpiLoStore epi{y, P.p32, P.diag_lo};
-    spmv_tiles<0, VT, float, float>(P, S, pipe, vlo, P.p32, epi, true);
+    spmv_tiles<VT, float, float>(P, S, pipe, vlo, P.p32, epi, true);
     drain<float, float>(P, S, pipe, P.p32);
 }
 
@@ -1387,21 +1373,66 @@ __global__ void __launch_bounds__(512) fp64_fma_probe_kernel(int iters, double s
     if (s == -12345.0) g_fp64_probe_sink = s;
 }
 
-constexpr int kRptChoices[] = {0, 1, 2, 4};
-SolveKernel solve_kernel_for(int rpt) {
-    switch (rpt) {
-        case 1: return cg_solve_kernel<1>;
-        case 2: return cg_solve_kernel<2>;
-        case 4: return cg_solve_kernel<4>;
-        default: return cg_solve_kernel<0>;
-    }
+const void *sell_kernel_for(bool pre, bool fx) {
+    if (fx) return pre ? (const void *)cg_sell_kernel<true, true> : (const void *)cg_sell_kernel<false, true>;
+    return pre ? (const void *)cg_sell_kernel<true, false> : (const void *)cg_sell_kernel<false, false>;
 }
+const void *sellmem_kernel_for(bool pre, bool fx) {
+    if (fx) return pre ? (const void *)cg_sellmem_kernel<true, true> : (const void *)cg_sellmem_kernel<false, true>;
+    return pre ? (const void *)cg_sellmem_kernel<true, false> : (const void *)cg_sellmem_kernel<false, false>;
+}
+
+// The instantiations of a SELL-32 solve kernel prefer L1 to shared memory
+// and must be resident, one CTA per SM.
+bool prepare_solve_kernels(const void *(*kernel_for)(bool, bool), bool *resident) {
+    *resident = true;
+    for (int i = 0; i < 4; ++i) {
+        const void *k = kernel_for((i & 1) != 0, (i & 2) != 0);
+        int occ = 0;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxL1) !=
+                cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kSellSolveThreads, 0) != cudaSuccess)
+            return false;
+        *resident = *resident && occ >= 1;
+    }
+    return true;
+}
+
+constexpr int kRptChoices[] = {1, 2, 4};   // cg_plan.reg_rows
 
 }  // namespace
 
 // =================================================================== host
 
 namespace {
+
+// The fixed-point copy of the handle's SELL-32 matrix (fixed.cuh), where the
+// matrix is eligible; otherwise the handle keeps the FP64 product.
+int build_fixed(cg_handle *h, size_t entries) {
+    if (!h->sell_c16) return CG_OK;
+    const SellMatrix M = sell_of(h);
+    const int blocks = (M.nslices + 7) / 8;
+    unsigned int *stat = nullptr, got[4] = {0, 0, 0, 0};
+    int rc = dev_alloc(h, &h->fixed_c, (size_t)h->n);
+    if (rc == CG_OK) rc = dev_alloc(h, &stat, 4);
+    if (rc != CG_OK) return rc;
+    // on the legacy default stream, behind the uploads of the matrix
+    cudaError_t e = cudaMemset(stat, 0, sizeof got);
+    fixed_scale_kernel<<<blocks, 256>>>(M, h->fixed_c, stat, stat + 2);
+    fixed_max_kernel<<<blocks, 256>>>(M, h->fixed_c, stat, stat + 1);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(got, stat, sizeof got, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e);
+    const int top = (int)got[1] - kFixedExpOffset;   // every scaled entry is below 2^top
+    const int spread = (int)got[2] + (int)got[3] - 256;   // largest c_i - c_j
+    if (got[0] != 0 || top > 3 || spread > kFixedSpreadC) return CG_OK;   // 2^(3 + 3) bounds a row's sum
+    h->fixed_u = kFixedBitsA - top;
+    if ((rc = dev_alloc(h, &h->fixed_vals, entries)) != CG_OK) return rc;
+    fixed_build_kernel<<<blocks, 256>>>(M, h->fixed_c, h->fixed_u, h->fixed_vals);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    return e == cudaSuccess ? CG_OK : cuda_fail(e);
+}
 
 void free_handle(cg_handle *h) {
     if (!h) return;
@@ -1479,12 +1510,11 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
     if (e == cudaSuccess) {
         if ((h->sell_solve || h->sell_mem) && h->opts.inner_values == CG_VALUES_FP64) {
             SellMatrix M = sell_of(h);
+            FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
             const int32_t *cut = h->sell_cut;
-            void *args[] = {&P, &M, &cut};
-            const void *kern =
-                h->sell_solve ? (precond ? (const void *)cg_sell_kernel<true> : (const void *)cg_sell_kernel<false>)
-                              : (precond ? (const void *)cg_sellmem_kernel<true>
-                                         : (const void *)cg_sellmem_kernel<false>);
+            void *args[] = {&P, &M, &F, &cut};
+            const bool pre = precond != 0, fx = h->fixed_vals != nullptr;
+            const void *kern = h->sell_solve ? sell_kernel_for(pre, fx) : sellmem_kernel_for(pre, fx);
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), args, 0, h->stream);
         } else if (h->sell_lo && h->opts.inner_values != CG_VALUES_FP64) {
             SellMatrix M = sell_of(h);
@@ -1496,7 +1526,7 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), args, 0, h->stream);
         } else {
             void *args[] = {&P};
-            const void *kern = (const void *)h->kernel;
+            const void *kern = (const void *)cg_solve_kernel;
             if (h->opts.inner_values == CG_VALUES_FP32) kern = (const void *)cg_ir_kernel<float>;
             if (h->opts.inner_values == CG_VALUES_BF16) kern = (const void *)cg_ir_kernel<__nv_bfloat16>;
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kThreads),
@@ -1685,12 +1715,9 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
     h->max_tile_nnz = max_tile;
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(CG_ECUDA);
-    for (int rpt : kRptChoices) {
-        if (cudaFuncSetAttribute((const void *)solve_kernel_for(rpt),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
-            return fail(CG_ECUDA);
-    }
-    if (cudaFuncSetAttribute((const void *)sell_spmv_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+    if (cudaFuncSetAttribute((const void *)cg_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute((const void *)sell_spmv_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxL1) != cudaSuccess ||
         cudaFuncSetAttribute((const void *)cg_ir_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kSmemBytes) != cudaSuccess ||
@@ -1701,7 +1728,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         cudaFuncSetAttribute((const void *)lo_spmv_tiles_kernel<__nv_bfloat16>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
         return fail(CG_ECUDA);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_kernel_for(4), kThreads, kSmemBytes) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_solve_kernel, kThreads, kSmemBytes) !=
             cudaSuccess ||
         per_sm < 1)
         return fail(CG_ECUDA);
@@ -1717,12 +1744,11 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
     h->rpt = 0;
     if (!opts.vectors_in_memory) {
         for (int rpt : kRptChoices)
-            if (rpt > 0 && per_warp <= rpt) {
+            if (per_warp <= rpt) {
                 h->rpt = rpt;
                 break;
             }
     }
-    h->kernel = solve_kernel_for(h->rpt);
     TilePlan tp = plan_windows(n, rowptr, colidx, tiles);
     h->window_tiles = tp.windowed;
     std::vector<int32_t> cta_row(ctas + 1);
@@ -1793,20 +1819,9 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                                              : split_slices(sh.ptr, ctas, kSliceMaxPerCta, kSliceVecCost);
         h->sell_solve = 0;
         if (!cut.empty()) {
-            int occ_plain = 0, occ_pre = 0;
-            const bool ok =
-                cudaFuncSetAttribute((const void *)cg_sell_kernel<false>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxL1) == cudaSuccess &&
-                cudaFuncSetAttribute((const void *)cg_sell_kernel<true>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxL1) == cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_plain, cg_sell_kernel<false>,
-                                                              kSellSolveThreads, 0) == cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_pre, cg_sell_kernel<true>,
-                                                              kSellSolveThreads, 0) == cudaSuccess;
-            if (!ok) return fail(CG_ECUDA);
-            if (occ_plain >= 1 && occ_pre >= 1) {
+            bool resident = false;
+            if (!prepare_solve_kernels(sell_kernel_for, &resident)) return fail(CG_ECUDA);
+            if (resident) {
                 // each row's entries in the CTA's own rows first (read while the
                 // grid barrier that publishes z completes)
                 sh = build_sell(n, rowptr, colidx, vals, &cut);
@@ -1821,24 +1836,14 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                 h->sell_solve = 1;
             }
         }
-        // larger systems (no register rows in the tiled kernel): the SELL-32
-        // kernel with the vectors in memory, slices in contiguous ranges per CTA
-        if (!h->sell_solve && !opts.vectors_in_memory && h->rpt == 0 && n > 0) {
+        // larger systems: the SELL-32 kernel with the vectors in memory, slices
+        // in contiguous ranges per CTA (at n = 161820, Jacobi-PCG: 22.2 us per
+        // iteration, 18.6 with the fixed-point product, where the tiled kernel
+        // with its rows in registers took 26.0)
+        if (!h->sell_solve && !opts.vectors_in_memory && n > 0) {
             const std::vector<int32_t> mcut = split_slices(sh.ptr, ctas, h->sell_slices, kSliceVecCost);
-            int occ_plain = 0, occ_pre = 0;
-            const bool ok =
-                !mcut.empty() &&
-                cudaFuncSetAttribute((const void *)cg_sellmem_kernel<false>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxL1) == cudaSuccess &&
-                cudaFuncSetAttribute((const void *)cg_sellmem_kernel<true>,
-                                     cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxL1) == cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_plain, cg_sellmem_kernel<false>,
-                                                              kSellSolveThreads, 0) == cudaSuccess &&
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_pre, cg_sellmem_kernel<true>,
-                                                              kSellSolveThreads, 0) == cudaSuccess;
-            if (ok && occ_plain >= 1 && occ_pre >= 1) {
+            bool resident = false;
+            if (!mcut.empty() && prepare_solve_kernels(sellmem_kernel_for, &resident) && resident) {
                 if ((rc = dev_alloc(h, &h->sell_cut, mcut.size()))) return fail(rc);
                 if (cudaMemcpy(h->sell_cut, mcut.data(), sizeof(int32_t) * mcut.size(), cudaMemcpyHostToDevice) !=
                     cudaSuccess)
@@ -1905,6 +1910,11 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
             es = sh.rel16 ? cudaMemcpy(h->sell_c16, sh.cols16.data(), 2 * tot, cudaMemcpyHostToDevice)
                           : cudaMemcpy(h->sell_c32, sh.cols32.data(), 4 * tot, cudaMemcpyHostToDevice);
         if (es != cudaSuccess) return fail(cuda_fail(es));
+        // the fixed-point product: where the FP64 pipe, not HBM, sets the pace
+        // of the FP64 one (at 100^3, streaming the matrix, 73.8 against 73.1 us
+        // per iteration: no gain)
+        if ((h->sell_solve || (h->sell_mem && !h->evict_first)) && !mixed && (rc = build_fixed(h, tot)) != CG_OK)
+            return fail(rc);
     }
     if (cudaMallocHost(&h->st_host, sizeof(DevStatus)) != cudaSuccess) return fail(CG_ENOMEM);
     if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess)
@@ -2094,7 +2104,7 @@ int cg_get_plan(const cg_handle *h, cg_plan *plan) {
     p.reg_rows = h->rpt;
     p.window_tiles = h->window_tiles;
     p.device_bytes = h->device_bytes;
-    p.slice_solve = h->sell_solve ? 1 : (h->sell_mem ? 2 : 0);
+    p.slice_solve = h->sell_solve ? 1 : (h->sell_mem && h->rpt == 0 ? 2 : 0);
     p.inner_solve = h->sell_lo ? 1 : 0;
     *plan = p;
     return CG_OK;

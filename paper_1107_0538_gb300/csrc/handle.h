@@ -14,7 +14,6 @@
 #include "sell.cuh"
 
 namespace gbcg {
-using SolveKernel = void (*)(Params);
 struct LearnCtx;  // learned-preconditioner workspace (learn.cu)
 }  // namespace gbcg
 
@@ -26,8 +25,7 @@ struct cg_handle {
     int64_t nnz = 0;
     int ctas = 0;
     int ntiles = 0;
-    int rpt = 0;                      // rows per thread kept in registers (0: none)
-    gbcg::SolveKernel kernel = nullptr;
+    int rpt = 0;                      // cg_plan.reg_rows
     int max_tile_nnz = 0;
     int evict_first = 0;
     int64_t device_bytes = 0;
@@ -60,6 +58,9 @@ struct cg_handle {
     int sell_grid = 0;                // CTAs of a SELL SpMV launch
     int sell_solve = 0;               // 1: FP64 solves run cg_sell_kernel
     int sell_mem = 0;                 // 1: FP64 solves run cg_sellmem_kernel (vectors in memory)
+    int2 *fixed_vals = nullptr;       // fixed-point copy of the SELL values (fixed.cuh), or nullptr
+    int8_t *fixed_c = nullptr;        // its exponent per row
+    int fixed_u = 0;                  // and of the whole matrix
     int32_t *sell_cut = nullptr;      // ctas + 1 slice boundaries of the slice kernel's CTAs
     int32_t *sell_split = nullptr;    // per slice: local block width (split layout), or nullptr
     void *sell_lo = nullptr;          // low-precision off-diagonals in the SELL layout (float or

@@ -48,7 +48,6 @@ struct StageLayout {
 constexpr int kRedSlots = 4;                   // partial sums per CTA per barrier
 constexpr int kSmemBytes = kWarps * kStageBytes + kWarps * 8 /*mbarriers*/ +
                            kThreads * 8 /*block-sum transpose*/ + 64 /*broadcast*/ + 64 /*control*/;
-constexpr int kMaxRegRows = 4;                 // largest rows-per-thread kept in registers
 static_assert(kStageBytes % 16 == 0, "stage alignment");
 static_assert(kTileNnz + 6 <= kColsStage && kTileNnz + 2 <= kValsStage, "stage slack");
 static_assert(kTileRows + 1 + 6 <= kRptrStage, "row pointer slack");

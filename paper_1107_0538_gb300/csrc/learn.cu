@@ -1144,17 +1144,17 @@ __global__ void __launch_bounds__(kThreads, 1) fcg_spmv_kernel(Params P, FcgStat
     double v[3] = {0.0, 0.0, 0.0};
     if (MODE == S_SETUP) {
         EpiSetupL e{st->b, P.dinv, V.dsq, V.pidx, V.s_in, P.r};
-        (void)spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, vec, e, true);
+        (void)spmv_tiles<double, double, double>(P, S, pipe, P.vals, vec, e, true);
         v[0] = e.rr;
         v[1] = e.bb;
         v[2] = e.rdr;
     } else if (MODE == S_Q) {
         EpiQ e{vec, V.p, P.q, st->restart ? 0.0 : st->beta};
-        (void)spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, vec, e, true);
+        (void)spmv_tiles<double, double, double>(P, S, pipe, P.vals, vec, e, true);
         v[0] = e.pq;
     } else {
         EpiTrueL e{st->b};
-        (void)spmv_tiles<0, double, double, double>(P, S, pipe, P.vals, vec, e, true);
+        (void)spmv_tiles<double, double, double>(P, S, pipe, P.vals, vec, e, true);
         v[0] = e.acc;
     }
     drain<double, double>(P, S, pipe, vec);

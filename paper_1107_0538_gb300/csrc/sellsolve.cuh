@@ -4,6 +4,7 @@
 #pragma once
 
 #include "cg_device.cuh"
+#include "fixed.cuh"
 #include "sell.cuh"
 
 namespace gbcg {
@@ -54,9 +55,18 @@ __device__ __forceinline__ void add_quarters(double (&v)[NV], const double *quar
     for (int j = 0; j < NV; ++j) v[j] = __shfl_sync(0xffffffffu, t, j);
 }
 
+//
+// With wmax (kMaxSlots words of shared memory) the largest mx of the CTA is
+// formed on the way, on warps the sums leave idle, in wmax[32].
+constexpr int kMaxSlots = 34;
 template <int NV>
-__device__ __forceinline__ void block_sum_1k(double (&v)[NV], double *red, double *quarter) {
+__device__ __forceinline__ void block_sum_1k(double (&v)[NV], double *red, double *quarter, unsigned int *wmax = nullptr,
+                                             unsigned int mx = 0) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (wmax) {
+        const unsigned int m = __reduce_max_sync(0xffffffffu, mx);
+        if (lane == 0) wmax[w] = m;
+    }
 #pragma unroll
     for (int j = 0; j < NV; ++j) red[j * kSellSolveThreads + threadIdx.x] = v[j];
     __syncthreads();
@@ -70,16 +80,35 @@ __device__ __forceinline__ void block_sum_1k(double (&v)[NV], double *red, doubl
             t[j] = ((src[0] + src[128]) + (src[256] + src[384])) + ((src[512] + src[640]) + (src[768] + src[896]));
         }
         fold_quarter<NV>(t, quarter, w);
+    } else if (wmax && w == 4) {
+        const unsigned int m = __reduce_max_sync(0xffffffffu, wmax[lane]);
+        if (lane == 0) wmax[32] = m;
     }
     __syncthreads();
     if (w == 0) add_quarters<NV>(v, quarter);
+}
+
+// The CTA's maximum travels in the last slot of its partial-sum record.
+__device__ __forceinline__ void publish_max(const Params &P, int set, unsigned int mx) {
+    if (threadIdx.x == 0)
+        reinterpret_cast<long long *>(P.partials)[((size_t)set * gridDim.x + blockIdx.x) * kRedSlots + kRedSlots - 1] = mx;
+}
+
+// Largest maximum of every CTA's record (one warp; all its lanes get it).
+__device__ __forceinline__ unsigned int grid_max(const Params &P, int set) {
+    const int G = (int)gridDim.x;
+    const long long *src = reinterpret_cast<const long long *>(P.partials) + (size_t)set * G * kRedSlots + kRedSlots - 1;
+    unsigned int m = 0;
+    for (int c = threadIdx.x & 31; c < G; c += 32) m = max(m, (unsigned int)__ldcg(src + (size_t)c * kRedSlots));
+    return __reduce_max_sync(0xffffffffu, m);
 }
 
 // Grid totals of the partials of barrier set `set`: warp g < 4 adds the
 // partials of CTAs g*32 + lane + 128 u, then as above.  Every CTA computes
 // the same bits.
 template <int NV>
-__device__ __forceinline__ void grid_totals_1k(const Params &P, int set, double (&out)[NV], double *quarter) {
+__device__ __forceinline__ void grid_totals_1k(const Params &P, int set, double (&out)[NV], double *quarter,
+                                               unsigned int *wmax = nullptr) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int G = (int)gridDim.x;
     if (w < 4) {
@@ -93,6 +122,9 @@ __device__ __forceinline__ void grid_totals_1k(const Params &P, int set, double 
             for (int j = 0; j < NV; ++j) t[j] += m < G ? __ldcg(src + (size_t)m * kRedSlots + j) : 0.0;
         }
         fold_quarter<NV>(t, quarter, w);
+    } else if (wmax && w == 4) {
+        const unsigned int m = grid_max(P, set);
+        if (lane == 0) wmax[33] = m;   // with wmax: the largest maximum, for thread 0
     }
     __syncthreads();
     if (w == 0) add_quarters<NV>(out, quarter);
