@@ -34,10 +34,10 @@
 #include <vector>
 
 #include "cg_device.cuh"
+#include "cluster.cuh"
 #include "gbcg.h"
 #include "handle.h"
 #include "lowprec.h"
-#include "plan.h"
 #include "sellsolve.cuh"
 
 using namespace gbcg;
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                S.bcast[0] = go ? rho / sigma : 0.0;
+                S.bcast[0] = go ? scalar_quotient(rho, sigma) : 0.0;
                 S.ctl[kCtlRun] = go;
             }
             __syncthreads();
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
                 else if (!(rho_new > 0.0)) status = CG_EBREAKDOWN;
                 else if (k < P.maxit) go = 1;  // else ENOCONV: no further direction needed
                 if (go) {
-                    S.bcast[1] = rho_new / rho;
+                    S.bcast[1] = scalar_quotient(rho_new, rho);
                     rho = rho_new;
                 }
                 S.ctl[kCtlRun] = go;
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             else if (!(rho_new > 0.0)) status = CG_EBREAKDOWN;
             else if (kk < P.maxit) go = 1;  // else ENOCONV
             if (go) {
-                bcast[1] = rho_new / rho;
+                bcast[1] = scalar_quotient(rho_new, rho);
                 rho = rho_new;
             }
             ctl[kCtlRun] = go;
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                const double al = go ? rho / sigma : 0.0;
+                const double al = go ? scalar_quotient(rho, sigma) : 0.0;
                 bcast[0] = al;
                 ctl[kCtlRun] = go;
                 if constexpr (FX) ctl[kCtlShift] = fixed_shift(mz, fixed_ub_mul(wmax[33], al));
@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                const double al = go ? rho / sigma : 0.0;
+                const double al = go ? scalar_quotient(rho, sigma) : 0.0;
                 bcast[0] = al;
                 ctl[kCtlRun] = go;
                 if constexpr (FX) ctl[kCtlShift] = fixed_shift(mz, fixed_ub_mul(wmax[33], al));
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 else if (!(rho_new > 0.0)) status = CG_EBREAKDOWN;
                 else if (k < P.maxit) go = 1;  // else ENOCONV
                 if (go) {
-                    bcast[1] = rho_new / rho;
+                    bcast[1] = scalar_quotient(rho_new, rho);
                     rho = rho_new;
                 }
                 ctl[kCtlRun] = go;
@@ -980,7 +980,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_ir_kernel(Params P) {
             if (tid == 0) {
                 int go = 1;
                 if (!finite_bits(sg[0]) || !(sg[0] > 0.0)) go = 0;  // inner breakdown: keep d
-                S.bcast[2] = go ? rho / sg[0] : 0.0;
+                S.bcast[2] = go ? scalar_quotient(rho, sg[0]) : 0.0;
                 S.ctl[kCtlRun] = go;
                 if (!go && k == 1) status = finite_bits(sg[0]) ? CG_EBREAKDOWN : CG_ENAN;
             }
@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_ir_kernel(Params P) {
                 else if (k >= P.max_inner || inner_total >= P.maxit) go = 0;
                 else go = 1;
                 if (go) {
-                    S.bcast[3] = rho_new / rho;
+                    S.bcast[3] = scalar_quotient(rho_new, rho);
                     rho = rho_new;
                 }
                 S.ctl[kCtlRun] = go;
@@ -1236,7 +1236,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             if (tid == 0) {
                 int go = 1;
                 if (!finite_bits(sg[0]) || !(sg[0] > 0.0)) go = 0;  // inner breakdown: keep d
-                bcast[2] = go ? rho / sg[0] : 0.0;
+                bcast[2] = go ? scalar_quotient(rho, sg[0]) : 0.0;
                 ctl[kCtlRun] = go;
                 if (!go && k == 1) status = finite_bits(sg[0]) ? CG_EBREAKDOWN : CG_ENAN;
             }
@@ -1276,7 +1276,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 else if (k >= P.max_inner || inner_total >= P.maxit) go = 0;
                 else go = 1;
                 if (go) {
-                    bcast[3] = rho_new / rho;
+                    bcast[3] = scalar_quotient(rho_new, rho);
                     rho = rho_new;
                 }
                 ctl[kCtlRun] = go;
@@ -1495,6 +1495,21 @@ Params gbcg::base_params(const cg_handle *h) {
 
 namespace {
 
+// Launch configuration of the one-cluster solve (one cluster is the grid).
+cudaLaunchConfig_t cluster_config(const cg_handle *h, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(h->cluster_ctas);
+    cfg.blockDim = dim3(h->cluster_threads);
+    cfg.dynamicSmemBytes = h->cluster_smem;
+    cfg.stream = h->stream;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)h->cluster_ctas;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 // Enqueues one solve on the handle's stream (no synchronization).
 int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t maxit, int precond) {
     Params P = base_params(h);
@@ -1508,7 +1523,15 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
     if (e == cudaSuccess) e = cudaMemsetAsync(h->st, 0, sizeof(DevStatus), h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev0, h->stream);
     if (e == cudaSuccess) {
-        if ((h->sell_solve || h->sell_mem) && h->opts.inner_values == CG_VALUES_FP64) {
+        if (h->cluster_ctas > 0) {
+            const SellMatrix M = sell_of(h);
+            const FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
+            const ClusterArgs L{h->cluster_cut, h->cluster_win, h->cluster_entries, h->cluster_window};
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = cluster_config(h, &at);
+            e = precond ? cudaLaunchKernelEx(&cfg, cg_cluster_kernel<true>, P, M, F, L)
+                        : cudaLaunchKernelEx(&cfg, cg_cluster_kernel<false>, P, M, F, L);
+        } else if ((h->sell_solve || h->sell_mem) && h->opts.inner_values == CG_VALUES_FP64) {
             SellMatrix M = sell_of(h);
             FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
             const int32_t *cut = h->sell_cut;
@@ -1557,6 +1580,47 @@ int finish_solve(cg_handle *h, cg_info *info) {
     out.reverted_at = -1;
     if (info) *info = out;
     return s.status;
+}
+
+// Sets up the one-cluster solve where the system fits it and the device can
+// run a cluster of that size.
+int plan_cluster_solve(cg_handle *h, const SellHost &sh) {
+    const void *kern[] = {(const void *)cg_cluster_kernel<false>, (const void *)cg_cluster_kernel<true>};
+    cudaFuncAttributes fa{};
+    int optin = 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kern[1]) != cudaSuccess)
+        return CG_ECUDA;
+    const size_t room = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    const ClusterPlan cp = plan_cluster(sh, kClusterMaxCtas, kSellSolveThreads / 32 - 1, room);
+    if (cp.ctas == 0) return CG_OK;
+    h->cluster_ctas = cp.ctas;
+    h->cluster_threads = cp.threads;
+    h->cluster_entries = (int)cp.entries;
+    h->cluster_window = cp.window;
+    h->cluster_smem = cp.smem;
+    for (const void *k : kern) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = cluster_config(h, &at);
+        int clusters = 0;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) != cudaSuccess)
+            return CG_ECUDA;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            h->cluster_ctas = 0;   // the grid kernel then
+            return CG_OK;
+        }
+    }
+    int rc;
+    if ((rc = dev_alloc(h, &h->cluster_cut, cp.cut.size())) || (rc = dev_alloc(h, &h->cluster_win, cp.win.size() / 2)))
+        return rc;
+    if (cudaMemcpy(h->cluster_cut, cp.cut.data(), sizeof(int32_t) * cp.cut.size(), cudaMemcpyHostToDevice) !=
+            cudaSuccess ||
+        cudaMemcpy(h->cluster_win, cp.win.data(), sizeof(int32_t) * cp.win.size(), cudaMemcpyHostToDevice) !=
+            cudaSuccess)
+        return CG_ECUDA;
+    return CG_OK;
 }
 
 int check_solve_args(const cg_handle *h, const double *b, const double *x, double tol) {
@@ -1914,6 +1978,11 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         // of the FP64 one (at 100^3, streaming the matrix, 73.8 against 73.1 us
         // per iteration: no gain)
         if ((h->sell_solve || (h->sell_mem && !h->evict_first)) && !mixed && (rc = build_fixed(h, tot)) != CG_OK)
+            return fail(rc);
+        // small systems: the whole solve inside one cluster (a caller that sets
+        // the CTA count, or tests the grid barrier, gets the grid)
+        if (h->sell_solve && h->fixed_vals && opts.grid_ctas == 0 && opts.debug_phantom_arrivals == 0 &&
+            (rc = plan_cluster_solve(h, sh)) != CG_OK)
             return fail(rc);
     }
     if (cudaMallocHost(&h->st_host, sizeof(DevStatus)) != cudaSuccess) return fail(CG_ENOMEM);

@@ -61,6 +61,11 @@ struct cg_handle {
     int2 *fixed_vals = nullptr;       // fixed-point copy of the SELL values (fixed.cuh), or nullptr
     int8_t *fixed_c = nullptr;        // its exponent per row
     int fixed_u = 0;                  // and of the whole matrix
+    int cluster_ctas = 0;             // CTAs of the one-cluster solve (cluster.cuh), 0: not used
+    int cluster_threads = 0, cluster_entries = 0, cluster_window = 0;
+    size_t cluster_smem = 0;
+    int32_t *cluster_cut = nullptr;
+    int2 *cluster_win = nullptr;
     int32_t *sell_cut = nullptr;      // ctas + 1 slice boundaries of the slice kernel's CTAs
     int32_t *sell_split = nullptr;    // per slice: local block width (split layout), or nullptr
     void *sell_lo = nullptr;          // low-precision off-diagonals in the SELL layout (float or

@@ -477,4 +477,49 @@ inline SellHost build_sell(int32_t n, const std::vector<int32_t> &rowptr, const 
     return S;
 }
 
+// Plan of the one-cluster solve (cluster.cuh): contiguous slice ranges for up
+// to kClusterMaxCtas CTAs, a warp per slice and one control warp each, and the
+// window of rows every CTA's columns lie in.  Shared memory per CTA: 8 + 2
+// bytes per padded entry, 8 per window row and 16 per thread.  No CTAs when it does not fit.
+constexpr int kClusterMaxCtas = 16;
+
+struct ClusterPlan {
+    int ctas = 0, threads = 0;
+    long long entries = 0;        // largest padded entry count of a CTA
+    int window = 0;               // largest window
+    size_t smem = 0;
+    std::vector<int32_t> cut;     // ctas + 1
+    std::vector<int32_t> win;     // first and past-the-last row per CTA
+};
+
+inline ClusterPlan plan_cluster(const SellHost &S, int max_ctas, int max_slices, size_t max_smem) {
+    ClusterPlan cp;
+    const int ns = (int)S.ptr.size() - 1;
+    if (ns < 1 || !S.rel16 || max_ctas < 1) return cp;
+    const int ctas = std::min(max_ctas, ns);
+    if ((ns + ctas - 1) / ctas > max_slices) return cp;
+    int slices = 0;
+    for (int c = 0; c <= ctas; ++c) cp.cut.push_back((int32_t)((long long)c * ns / ctas));
+    for (int c = 0; c < ctas; ++c) {
+        const int t0 = cp.cut[c], t1 = cp.cut[c + 1];
+        slices = std::max(slices, t1 - t0);
+        cp.entries = std::max(cp.entries, S.ptr[t1] - S.ptr[t0]);
+        int lo = t0 * 32, hi = t0 * 32 + 1;
+        for (int t = t0; t < t1; ++t)
+            for (long long i = S.ptr[t]; i < S.ptr[t + 1]; ++i) {
+                const int col = t * 32 + (int)((i - S.ptr[t]) & 31) + S.cols16[(size_t)i];
+                lo = std::min(lo, col);
+                hi = std::max(hi, col + 1);
+            }
+        cp.win.push_back(lo);
+        cp.win.push_back(hi);
+        cp.window = std::max(cp.window, hi - lo);
+    }
+    cp.smem = (size_t)cp.entries * 10 + (size_t)cp.window * 8 + 16 * 32 * ((size_t)slices + 1);
+    if (cp.smem > max_smem || cp.window > 65535) return cp;
+    cp.ctas = ctas;
+    cp.threads = 32 * (slices + 1);
+    return cp;
+}
+
 }  // namespace gbcg

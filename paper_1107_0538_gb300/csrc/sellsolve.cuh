@@ -12,6 +12,30 @@ namespace gbcg {
 constexpr int kSellSolveThreads = 1024;
 constexpr int kSellUnrollMem = 18;   // loads in flight per row where rows are not held in registers
 
+// a / b to the last bit or two, for the scalars of an iteration: Newton's step
+// for the reciprocal from a single-precision seed y (error 2^-22), folded into
+// the quotient, and one correction with the exact remainder (Markstein, "Computation
+// of elementary functions on the IBM RISC System/6000", 1990): five FP64
+// operations of 64 clocks, where a call of the division takes 580.
+__device__ __forceinline__ double scalar_quotient(double a, double b) {
+    const unsigned int ha = (unsigned int)__double2hiint(a), hb = (unsigned int)__double2hiint(b);
+    const int ea = (int)(ha >> 20) & 0x7ff, eb = (int)(hb >> 20) & 0x7ff;
+    if (ea < 64 || ea > 1982 || eb < 64 || eb > 1982 || abs(ea - eb) > 900) return a / b;
+    // b = 2^(eb - 1023) m, m in [1, 2) with b's sign
+    const double m = __hiloint2double((int)((hb & 0x800fffffu) | 0x3ff00000u), __double2loint(b));
+    const unsigned int mf = ((hb & 0xfffffu) << 3) | ((unsigned int)__double2loint(b) >> 29);
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(0x3f800000u | mf)));
+    const unsigned int yb = __float_as_uint(yf);   // in (1/2, 1]
+    const double y = __hiloint2double((int)(((yb >> 3) + ((1023u - 127u) << 20)) | (hb & 0x80000000u)), (int)(yb << 29));
+    const double q0 = a * y;
+    const double e = fma(-m, y, 1.0);
+    const double q1 = fma(q0, e, q0);
+    const double q = fma(fma(-m, q1, a), y, q1);
+    // times 2^(1023 - eb): the exponents stay inside the normal range
+    return __hiloint2double(__double2hiint(q) + ((1023 - eb) << 20), __double2loint(q));
+}
+
 // Sums over the CTA in a fixed order with the FP64 work spread over the four
 // SM sub-partitions (warp w issues on sub-partition w mod 4; one warp-wide
 // FP64 add occupies a sub-partition's FP64 pipe for ~64 cycles, so the number
