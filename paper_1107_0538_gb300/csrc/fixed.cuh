@@ -39,7 +39,7 @@
 // than 64 in the scaled units, or a diagonal outside 2^+-200 or spread over
 // more than a factor of 2^24 (where the one shift of the whole vector would
 // leave the small rows of an unpreconditioned residual few bits) keeps the
-// FP64 product (fixed_scale_kernel, fixed_max_kernel).
+// FP64 product (fixed_build.cuh).
 #pragma once
 
 #include <cstdint>
@@ -205,87 +205,6 @@ __device__ __forceinline__ void fixed_slice_sum(const FixedMatrix &F, int n, int
     if constexpr (U > 3)
         for (; m >= 3; m -= 3, vv += 96, cc += 96) fixed_batch<3>(vv, cc, Z + row, row, n, s);
     for (; m > 0; --m, vv += 32, cc += 32) fixed_batch<1>(vv, cc, Z + row, row, n, s);
-}
-
-// ---- the matrix's fixed-point copy, built once per handle from its SELL-32
-// copy (one warp per slice, lane per row).  flags: bit 0 set when the matrix
-// is not eligible.
-
-// c_i from the diagonal.
-static __global__ void __launch_bounds__(256) fixed_scale_kernel(SellMatrix M, int8_t *c, unsigned int *flags, unsigned int *maxc) {
-    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (t >= M.nslices) return;
-    const int row = t * 32 + lane;
-    if (row >= M.n) return;
-    const long long a = M.ptr[t];
-    const int w = (int)((M.ptr[t + 1] - a) >> 5);
-    double d = 0.0;
-    for (int k = 0; k < w; ++k) {
-        const long long i = a + 32LL * k + lane;
-        const int col = M.cols16 ? row + M.cols16[i] : M.cols32[i];
-        if (col == row) d += M.vals[i];   // padding adds zeros
-    }
-    const int e = (int)((unsigned long long)__double_as_longlong(d) >> 52);   // with the sign bit
-    const int ci = (e - 1023 + 1) >> 1;
-    if (w > kFixedMaxWidth || e == 0 || e >= 2047 || ci > kFixedMaxC || ci < -kFixedMaxC) {
-        atomicOr(flags, 1u);
-        c[row] = 0;
-        return;
-    }
-    c[row] = (int8_t)ci;
-    atomicMax(maxc, (unsigned int)(128 + ci));       // maxc[0] - 128 = max c_i,
-    atomicMax(maxc + 1, (unsigned int)(128 - ci));   // 128 - maxc[1] = min c_i
-}
-
-// The smallest x (plus kFixedExpOffset) with every |a_ij| 2^(-c_i - c_j) < 2^x
-// and every row's sum of them < 2^(x + 3); entries that are not finite raise
-// the flag.
-constexpr int kFixedExpOffset = 4096;
-static __global__ void __launch_bounds__(256)
-    fixed_max_kernel(SellMatrix M, const int8_t *c, unsigned int *flags, unsigned int *maxexp) {
-    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (t >= M.nslices) return;
-    const int row = t * 32 + lane;
-    int x = 0;
-    if (row < M.n) {
-        const long long a = M.ptr[t];
-        const int w = (int)((M.ptr[t + 1] - a) >> 5);
-        const int cr = c[row];
-        double sum = 0.0;
-        for (int k = 0; k < w; ++k) {
-            const long long i = a + 32LL * k + lane;
-            const int col = M.cols16 ? row + M.cols16[i] : M.cols32[i];
-            const double v = M.vals[i];
-            const int e = (__double2hiint(v) >> 20) & 0x7ff;
-            if (e == 0x7ff) atomicOr(flags, 1u);
-            if (e != 0) {
-                x = max(x, e - 1022 - cr - c[col] + kFixedExpOffset);
-                sum += ldexp(fabs(v), -cr - c[col]);
-            }
-        }
-        if (sum > 0.0) x = max(x, ((__double2hiint(sum) >> 20) & 0x7ff) - 1022 - 3 + kFixedExpOffset);
-    }
-    const unsigned int m = __reduce_max_sync(0xffffffffu, (unsigned int)x);
-    if (lane == 0 && m) atomicMax(maxexp, m);
-}
-
-static __global__ void __launch_bounds__(256)
-    fixed_build_kernel(SellMatrix M, const int8_t *c, int u, int2 *vals) {
-    const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (t >= M.nslices) return;
-    const int row = t * 32 + lane;
-    const long long a = M.ptr[t];
-    const int w = (int)((M.ptr[t + 1] - a) >> 5);
-    for (int k = 0; k < w; ++k) {
-        const long long i = a + 32LL * k + lane;
-        int2 v = make_int2(0, 0);
-        if (row < M.n) {
-            const int col = M.cols16 ? row + M.cols16[i] : M.cols32[i];
-            v = fixed_split(fixed_of((unsigned long long)__double_as_longlong(M.vals[i]), u - c[row] - c[col]),
-                            kFixedLoBits);
-        }
-        vals[i] = v;
-    }
 }
 
 }  // namespace gbcg

@@ -35,6 +35,7 @@
 
 #include "cg_device.cuh"
 #include "cluster.cuh"
+#include "fixed_build.cuh"
 #include "gbcg.h"
 #include "handle.h"
 #include "lowprec.h"

@@ -30,10 +30,13 @@
 // it: a process that resets a device must not call this entry point on it
 // again.
 //
-// It is a variant of cg_solve_kernel: the same recurrence, fixed-order
-// reductions, thread-0 scalars and bounded grid barriers, with a plain
-// row-per-thread SpMV straight from the caller's CSR arrays instead of the
-// TMA-staged tiles (whose plan cg_create builds on the host).
+// It is the recurrence of the SELL-32 solve kernels (two grid barriers per
+// iteration: q = A r + beta q, p = r + beta p, then x and r), with their
+// fixed-order sums, thread-0 scalars and bounded barriers, and a row-per-thread
+// SpMV straight from the caller's CSR arrays instead of the SELL-32 copy that
+// cg_create builds.  Per iteration, against the three-barrier form with two
+// entries in flight per row: 50^3 17.1 us (22.6), 60x61x59 25.1 (29.5),
+// 37x41x29 13.0 (15.4), 20^3 11.7 (14.0).
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -41,8 +44,8 @@
 #include <cstdint>
 #include <mutex>
 
-#include "cg_device.cuh"
 #include "gbcg.h"
+#include "sellsolve.cuh"
 
 using namespace gbcg;
 
@@ -58,7 +61,9 @@ constexpr size_t kOffPartials = kOffQ + kVecBytes;
 constexpr size_t kOffBar = kOffPartials + kPartialBytes;
 constexpr size_t kOffStatus = kOffBar + 256;
 constexpr size_t kScratchBytes = kOffStatus + 256;
-constexpr int kNoallocSmem = kThreads * 8 + 64 + 64;
+constexpr int kNoallocUnroll = 9;    // entries of a row in flight
+constexpr int kNoallocUnroll2 = 7;   // of a lane, two lanes to a row (5: 17.8 us at 50^3, 14: 22.6)
+constexpr int kNoallocRows2 = 512;   // rows per CTA from which two lanes share a row
 
 }  // namespace
 
@@ -79,151 +84,223 @@ struct NoallocArgs {
     int32_t maxit;
 };
 
-// y_i = sum_k vals[k] * v[colidx[k]] for one row; false if the row's range or
-// a column is out of bounds (the entry is then skipped).
+// Row i's range of entries; false if it is out of bounds.
+__device__ __forceinline__ bool noalloc_range(const NoallocArgs &A, int i, int64_t nnz, int &k0, int &k1) {
+    k0 = __ldg(A.rowptr + i);
+    k1 = __ldg(A.rowptr + i + 1);
+    return k0 >= 0 && k1 >= k0 && (int64_t)k1 <= nnz;
+}
+
+// sum_k vals[k] v[colidx[k]] over the row's entries, kNoallocUnroll of
+// them in flight.  CHECK (the first pass over the matrix): a row range or a
+// column out of bounds sets bad and its entries are not read; the passes
+// after it run only if there was none.  v is written by this kernel between
+// grid barriers: coherent loads.
+template <bool CHECK>
 __device__ __forceinline__ double noalloc_row(const NoallocArgs &A, int i, const double *v, int64_t nnz,
                                               bool &bad) {
-    const int k0 = A.rowptr[i], k1 = A.rowptr[i + 1];
-    if (k0 < 0 || k1 < k0 || (int64_t)k1 > nnz) {
+    int k0, k1;
+    if (!noalloc_range(A, i, nnz, k0, k1)) {
         bad = true;
         return 0.0;
     }
-    double s0 = 0.0, s1 = 0.0;
-    int k = k0;
-    for (; k + 1 < k1; k += 2) {
-        const int c0 = A.colidx[k], c1 = A.colidx[k + 1];
-        const bool ok0 = (unsigned)c0 < (unsigned)A.n, ok1 = (unsigned)c1 < (unsigned)A.n;
-        bad |= !ok0 || !ok1;
-        const double x0 = ok0 ? v[c0] : 0.0, x1 = ok1 ? v[c1] : 0.0;
-        s0 = fma(A.vals[k], x0, s0);
-        s1 = fma(A.vals[k + 1], x1, s1);
+    double s = 0.0;
+    for (int k = k0; k < k1; k += kNoallocUnroll) {
+        double vr[kNoallocUnroll], xr[kNoallocUnroll];
+#pragma unroll
+        for (int u = 0; u < kNoallocUnroll; ++u) {
+            const bool in = k + u < k1;
+            vr[u] = in ? __ldg(A.vals + k + u) : 0.0;
+            const int c = in ? __ldg(A.colidx + k + u) : i;
+            if (CHECK) {
+                const bool ok = (unsigned)c < (unsigned)A.n;
+                bad |= !ok;
+                xr[u] = ok && in ? __ldca(v + c) : 0.0;
+            } else {
+                xr[u] = in ? __ldca(v + c) : 0.0;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kNoallocUnroll; ++u)
+            if (k + u < k1) s = fma(vr[u], xr[u], s);
     }
-    if (k < k1) {
-        const int c0 = A.colidx[k];
-        const bool ok0 = (unsigned)c0 < (unsigned)A.n;
-        bad |= !ok0;
-        s0 = fma(A.vals[k], ok0 ? v[c0] : 0.0, s0);
-    }
-    return s0 + s1;
+    return s;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) cg_noalloc_kernel(NoallocArgs A, Params P, int64_t nnz) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    Smem S;
-    S.stage = nullptr;
-    S.mbar = nullptr;
-    S.red = reinterpret_cast<double *>(smem_raw);
-    S.bcast = S.red + kThreads;
-    S.ctl = reinterpret_cast<int *>(S.bcast + 8);
+// Row sums of the warp's 32 rows base .. base + 31 (below row_hi), lane l's
+// row's in lane l, two lanes to a row and 16 rows at a time; the partial sums
+// are brought together at the end (28 FMAs and an add for 32 rows of 27
+// entries instead of 27 FMAs).
+//
+// Why: with a lane per row a load of the caller's CSR arrays touches 32 lines,
+// and the L1 data pipe, not the FP64 pipe, sets the pace once an SM has many
+// rows (50^3: it is busy 46% of an iteration, nearly all of the product).  At
+// 132651 rows an iteration takes 17.3 us with two lanes and 18.5 with one; at
+// 48000 (316 per CTA), where latency counts, 14.0 and 12.6.
+__device__ __forceinline__ double noalloc_rows2(const NoallocArgs &A, int base, int row_hi, const double *v) {
+    const int lane = threadIdx.x & 31;
+    int k[2], k1[2];
+    double s[2] = {0.0, 0.0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int row = base + 16 * h + (lane >> 1);
+        const bool in = row < row_hi;
+        k[h] = in ? __ldg(A.rowptr + row) + (lane & 1) : 0;
+        k1[h] = in ? __ldg(A.rowptr + row + 1) : 0;
+    }
+    while (__any_sync(0xffffffffu, k[0] < k1[0] || k[1] < k1[1])) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            double vr[kNoallocUnroll2], xr[kNoallocUnroll2];
+#pragma unroll
+            for (int u = 0; u < kNoallocUnroll2; ++u) {
+                const int e = k[h] + 2 * u;
+                vr[u] = xr[u] = 0.0;
+                if (e < k1[h]) {
+                    vr[u] = __ldg(A.vals + e);
+                    xr[u] = __ldca(v + __ldg(A.colidx + e));
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kNoallocUnroll2; ++u)
+                if (k[h] + 2 * u < k1[h]) s[h] = fma(vr[u], xr[u], s[h]);
+            k[h] += 2 * kNoallocUnroll2;
+        }
+    }
+    const int src = 2 * (lane & 15);
+    const double a0 = __shfl_sync(0xffffffffu, s[0], src), b0 = __shfl_sync(0xffffffffu, s[0], src + 1);
+    const double a1 = __shfl_sync(0xffffffffu, s[1], src), b1 = __shfl_sync(0xffffffffu, s[1], src + 1);
+    return (lane < 16 ? a0 : a1) + (lane < 16 ? b0 : b1);
+}
+
+__global__ void __launch_bounds__(kSellSolveThreads, 1) cg_noalloc_kernel(NoallocArgs A, Params P, int64_t nnz) {
+    __shared__ double red[3 * kSellSolveThreads];
+    __shared__ double quarter[12];
+    __shared__ double bcast[8];
+    __shared__ int ctl[16];
+    Smem S{};
+    S.red = red;
+    S.bcast = bcast;
+    S.ctl = ctl;
+    constexpr int kT = kSellSolveThreads;
     const int tid = threadIdx.x;
     const int G = (int)gridDim.x;
     const int row_lo = (int)((int64_t)A.n * blockIdx.x / G);
     const int row_hi = (int)((int64_t)A.n * (blockIdx.x + 1) / G);
+    const bool two = A.n > kNoallocRows2 * G;
     unsigned int epoch = 0;
     int set = 0;
     bool bad = false;
     int status = CG_OK, iters = 0;
-    double rr = 0.0, bb = 0.0, rho = 0.0, bnorm = 0.0;
+    double rr = 0.0, bb = 0.0, rho = 0.0, bnorm = 0.0, tol2bb = 0.0;
 
-    // setup: r = b - A x, p = r; r.r, b.b (and any malformed row)
+    // setup: r = b - A x, p = r, q = 0; r.r, b.b (and any malformed row)
     double v[3] = {0.0, 0.0, 0.0};
-    for (int i = row_lo + tid; i < row_hi; i += kThreads) {
+    for (int i = row_lo + tid; i < row_hi; i += kT) {
         const double bi = A.b[i];
-        const double ri = bi - noalloc_row(A, i, A.x, nnz, bad);
+        const double ri = bi - noalloc_row<true>(A, i, A.x, nnz, bad);
         P.r[i] = ri;
-        P.p0[i] = ri;
+        P.pd[i] = ri;
+        P.q[i] = 0.0;
         v[0] = fma(ri, ri, v[0]);
         v[1] = fma(bi, bi, v[1]);
     }
     v[2] = __syncthreads_or(bad) ? 1.0 : 0.0;
-    block_sum<3>(v, S);
+    block_sum_1k<3>(v, red, quarter);
+    // every thread of a CTA has the same v[2]: the CTA's sum is 1024 or 0
     publish_partials<3>(P, set, v);
-    if (!grid_barrier(P, epoch, S)) return;
+    if (!grid_barrier<false>(P, epoch, S)) return;
     {
         double t[3];
-        grid_totals<3>(P, set, t);
+        grid_totals_1k<3>(P, set, t, quarter);
         set ^= 1;
         if (tid == 0) {
             rr = t[0];
             bb = t[1];
             rho = t[0];
             bnorm = sqrt(bb);
+            tol2bb = (P.tol * bnorm) * (P.tol * bnorm);
             int go = 0, zero_b = 0;
             if (t[2] != 0.0) status = CG_EINVAL;
             else if (!finite_bits(bb) || !finite_bits(rr)) status = CG_ENAN;
             else if (bnorm == 0.0) { zero_b = 1; rr = 0.0; }
-            else if (sqrt(rr) <= P.tol * bnorm) status = CG_OK;
+            else if (rr <= tol2bb) status = CG_OK;
             else go = 1;
-            S.ctl[0] = go;
-            S.ctl[2] = zero_b;
+            ctl[0] = go;
+            ctl[2] = zero_b;
         }
         __syncthreads();
-        if (S.ctl[2])
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) A.x[i] = 0.0;
+        if (ctl[2])
+            for (int i = row_lo + tid; i < row_hi; i += kT) A.x[i] = 0.0;
     }
-    if (S.ctl[0]) {
+    if (ctl[0]) {
         if (tid == 0) status = CG_ENOCONV;
+        double beta = 0.0;   // p_1 = r_0, q_1 = A r_0
         for (int k = 1; k <= P.maxit; ++k) {
-            // q = A p, p . q
-            double pq = 0.0;
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) {
-                const double qi = noalloc_row(A, i, P.p0, nnz, bad);
+            // q = A r + beta q (= A p), p = r + beta p; p . q
+            double v1[1] = {0.0};
+            for (int i = row_lo + tid; i - (tid & 31) < row_hi; i += kT) {
+                const double az = two ? noalloc_rows2(A, i - (tid & 31), row_hi, P.r)
+                                      : (i < row_hi ? noalloc_row<false>(A, i, P.r, nnz, bad) : 0.0);
+                if (i >= row_hi) break;
+                const double qi = fma(beta, P.q[i], az);
+                const double pi = fma(beta, P.pd[i], P.r[i]);
                 P.q[i] = qi;
-                pq = fma(P.p0[i], qi, pq);
+                P.pd[i] = pi;
+                v1[0] = fma(pi, qi, v1[0]);
             }
-            double v1[1] = {pq};
-            block_sum<1>(v1, S);
+            block_sum_1k<1>(v1, red, quarter);
             publish_partials<1>(P, set, v1);
-            if (!grid_barrier(P, epoch, S)) return;
+            if (!grid_barrier<false>(P, epoch, S)) return;
             double sg[1];
-            grid_totals<1>(P, set, sg);
+            grid_totals_1k<1>(P, set, sg, quarter);
             set ^= 1;
             if (tid == 0) {
                 int go = 0;
                 if (!finite_bits(sg[0])) status = CG_ENAN;
                 else if (!(sg[0] > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                S.bcast[0] = go ? rho / sg[0] : 0.0;
-                S.ctl[0] = go;
+                bcast[0] = go ? scalar_quotient(rho, sg[0]) : 0.0;
+                ctl[0] = go;
             }
             __syncthreads();
-            if (!S.ctl[0]) break;
-            const double alpha = S.bcast[0];
-            // x += alpha p, r -= alpha q; r.r
-            double prr = 0.0;
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) {
-                A.x[i] = fma(alpha, P.p0[i], A.x[i]);
+            if (!ctl[0]) break;
+            const double alpha = bcast[0];
+            // r -= alpha q (every gather of it is over); r.r
+            double v2[1] = {0.0};
+            for (int i = row_lo + tid; i < row_hi; i += kT) {
                 const double ri = fma(-alpha, P.q[i], P.r[i]);
                 P.r[i] = ri;
-                prr = fma(ri, ri, prr);
+                v2[0] = fma(ri, ri, v2[0]);
             }
-            double v2[1] = {prr};
-            block_sum<1>(v2, S);
+            block_sum_1k<1>(v2, red, quarter);
             publish_partials<1>(P, set, v2);
-            if (!grid_barrier(P, epoch, S)) return;
+            // x += alpha p, read by nothing before the end, while thread 0 waits
+            grid_arrive(P, epoch);
+            if (tid == 0) ctl[15] = grid_wait<false>(P, epoch);
+            for (int i = row_lo + tid; i < row_hi; i += kT) A.x[i] = fma(alpha, P.pd[i], A.x[i]);
+            __syncthreads();
+            if (!ctl[15]) return;
             double t2[1];
-            grid_totals<1>(P, set, t2);
+            grid_totals_1k<1>(P, set, t2, quarter);
             set ^= 1;
             if (tid == 0) {
                 iters = k;
                 rr = t2[0];
                 int go = 0;
                 if (!finite_bits(rr)) status = CG_ENAN;
-                else if (sqrt(rr) <= P.tol * bnorm) status = CG_OK;
+                else if (rr <= tol2bb) status = CG_OK;
                 else if (!(rr > 0.0)) status = CG_EBREAKDOWN;
                 else if (k < P.maxit) go = 1;
                 if (go) {
-                    S.bcast[1] = rr / rho;
+                    bcast[1] = scalar_quotient(rr, rho);
                     rho = rr;
                 }
-                S.ctl[0] = go;
+                ctl[0] = go;
             }
             __syncthreads();
-            if (!S.ctl[0]) break;
-            const double beta = S.bcast[1];
-            // p = r + beta p
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) P.p0[i] = fma(beta, P.p0[i], P.r[i]);
-            if (!grid_barrier(P, epoch, S)) return;
+            if (!ctl[0]) break;
+            beta = bcast[1];
         }
     }
     if (blockIdx.x == 0 && tid == 0) {
@@ -247,13 +324,13 @@ int noalloc_setup(int dev, unsigned char **scratch, int *grid) {
     if (!g_scratch_ptr[dev]) {
         void *ptr = nullptr;
         if (cudaGetSymbolAddress(&ptr, g_cg_noalloc_scratch) != cudaSuccess || !ptr) return CG_ECUDA;
-        if (cudaFuncSetAttribute((const void *)cg_noalloc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kNoallocSmem) != cudaSuccess)
+        if (cudaFuncSetAttribute((const void *)cg_noalloc_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxL1) != cudaSuccess)
             return CG_ECUDA;
         int sms = 0, per_sm = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_noalloc_kernel, kThreads,
-                                                          kNoallocSmem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_noalloc_kernel,
+                                                          kSellSolveThreads, 0) != cudaSuccess ||
             per_sm < 1)
             return CG_ECUDA;
         int g = sms < kNoallocMaxCtas ? sms : kNoallocMaxCtas;
@@ -330,7 +407,7 @@ int solve_noalloc(const cg_csr *A, const double *b, double *x, double tol, int32
     Params P{};
     P.n = A->n;
     P.r = reinterpret_cast<double *>(scratch + kOffR);
-    P.p0 = reinterpret_cast<double *>(scratch + kOffP);
+    P.pd = reinterpret_cast<double *>(scratch + kOffP);
     P.q = reinterpret_cast<double *>(scratch + kOffQ);
     P.partials = reinterpret_cast<double *>(scratch + kOffPartials);
     P.bar = reinterpret_cast<unsigned int *>(scratch + kOffBar);
@@ -345,8 +422,8 @@ int solve_noalloc(const cg_csr *A, const double *b, double *x, double tol, int32
     cudaError_t e = cudaMemsetAsync(scratch + kOffBar, 0, 256 + 256, st);
     if (e == cudaSuccess) {
         void *kargs[] = {&args, &P, &nnz};
-        e = cudaLaunchCooperativeKernel((const void *)cg_noalloc_kernel, dim3(grid), dim3(kThreads), kargs,
-                                        (size_t)kNoallocSmem, st);
+        e = cudaLaunchCooperativeKernel((const void *)cg_noalloc_kernel, dim3(grid), dim3(kSellSolveThreads), kargs, 0,
+                                        st);
     }
     DevStatus s{};
     if (e == cudaSuccess) e = cudaMemcpyAsync(&s, scratch + kOffStatus, sizeof(DevStatus), cudaMemcpyDeviceToHost, st);
