@@ -105,6 +105,8 @@ KERNEL_SOURCES = {
     "cg_sell_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "cg_sellmem_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "sell_spmv_kernel": ["gbcg.cu", "sell.cuh", "plan.h"],
+    "cg_ring_kernel": ["gbcg.cu", "ring.cuh", "fixed.cuh", "sell.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
+    "cg_irring_kernel": ["gbcg.cu", "ring.cuh", "sell.cuh", "sellsolve.cuh", "plan.h", "lowprec.h"] + _COMMON,
     "cg_ir_kernel": ["gbcg.cu", "plan.h", "lowprec.h"] + _COMMON,
     "cg_irsell_kernel": ["gbcg.cu", "sell.cuh", "sellsolve.cuh", "plan.h", "lowprec.h"] + _COMMON,
     "cg_batch_kernel": ["batch.cu", "plan.h", "lowprec.h"] + _COMMON,
@@ -591,7 +593,7 @@ def measure_forms_100cube(flush, fp64_tflops: float, count: int = 2) -> dict:
         if name == "fp64_cg":
             x_fp64, ms_fp64 = xv.copy(), v_ms
             # FP64-ALU roofline of the solve kernel (Table I's flop count)
-            kern = "cg_sellmem_kernel" if plan_v["slice_solve"] == 2 else "cg_solve_kernel"
+            kern = "cg_ring_kernel" if plan_v["slice_solve"] == 2 else "cg_solve_kernel"
             kern_s = statistics.mean(i.kernel_ms for _, i in res_v) / 1e3
             flops = info_v.iters * flops_per_iteration(big.A.n, big.A.nnz, False)
             tr = ncu_traffic(kern)

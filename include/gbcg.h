@@ -156,8 +156,8 @@ typedef struct {
                                 not 0, else the tiled kernel described by the
                                 fields above                                     */
     int32_t inner_solve;     /* handles with inner_values FP32/BF16: 1 when the
-                                refinement runs on SELL-32 copies (one 32-row
-                                slice per warp), 0 when it runs on the staged
+                                refinement runs with one 32-row slice per warp;
+                                0 for larger systems and when it runs on the staged
                                 tiles described above; 0 for FP64 handles       */
 } cg_plan;
 

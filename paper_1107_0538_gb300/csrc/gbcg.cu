@@ -39,6 +39,8 @@
 #include "gbcg.h"
 #include "handle.h"
 #include "lowprec.h"
+#include "ring.cuh"
+#include "ring_build.cuh"
 #include "sellsolve.cuh"
 
 using namespace gbcg;
@@ -604,19 +606,17 @@ out:
 // the same thread.  Two grid barriers per iteration; each decision is taken
 // before the next phase starts.
 
-template <bool PRE, bool FX>
+template <bool PRE>
 __global__ void __launch_bounds__(kSellSolveThreads, 1)
-    cg_sellmem_kernel(Params P, SellMatrix M, FixedMatrix F, const int32_t *__restrict__ cut) {
+    cg_sellmem_kernel(Params P, SellMatrix M, const int32_t *__restrict__ cut) {
     __shared__ double red[3 * kSellSolveThreads];
     __shared__ double quarter[12];
     __shared__ double bcast[8];
     __shared__ int ctl[16];
-    __shared__ unsigned int wmax_s[FX ? kMaxSlots : 1];
-    unsigned int *const wmax = FX ? wmax_s : nullptr;
-    Smem SM{};
-    SM.red = red;
-    SM.bcast = bcast;
-    SM.ctl = ctl;
+    Smem S{};
+    S.red = red;
+    S.bcast = bcast;
+    S.ctl = ctl;
     unsigned int epoch = 0;
     int set = 0;
     constexpr int kW = kSellSolveThreads / 32;
@@ -624,9 +624,6 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
     const int t0 = cut[blockIdx.x] + (tid >> 5), t1 = cut[blockIdx.x + 1];
     double *const zg = P.p0;   // z: the vector the SpMV gathers
     double *const pv = P.pd;   // p
-    int2 *const zx = reinterpret_cast<int2 *>(P.p0);   // FX: z's integers instead (fixed.cuh)
-    int S = 0;               // FX: z's shift (every thread)
-    unsigned int mz = 0;     // FX: the bound on z (thread 0; every thread's own in phase B)
 
     // thread 0's scalar state
     int status = CG_OK, iters = 0;
@@ -636,7 +633,6 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
     bool run;
     {
         double v[3] = {0.0, 0.0, 0.0};
-        unsigned int mx = 0;
         for (int t = t0; t < t1; t += kW) {
             const double ax = sell_slice_sum<kSellUnrollMem>(M, t, P.x, 0.0);
             const int row = t * 32 + lane;
@@ -645,8 +641,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 const double ri = bi - ax;
                 const double zi = PRE ? __ldg(P.dinv + row) * ri : ri;
                 P.r[row] = ri;
-                if constexpr (FX) mx = max(mx, fixed_ub(zi, F.c[row]));
-                else zg[row] = zi;
+                zg[row] = zi;
                 pv[row] = zi;
                 P.q[row] = 0.0;
                 v[0] = fma(ri, ri, v[0]);
@@ -654,12 +649,11 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 v[2] = fma(bi, bi, v[2]);
             }
         }
-        block_sum_1k<3>(v, red, quarter, wmax, mx);
+        block_sum_1k<3>(v, red, quarter);
         publish_partials<3>(P, set, v);
-        if constexpr (FX) publish_max(P, set, wmax[32]);
-        if (!grid_barrier<false>(P, epoch, SM)) goto out;
+        if (!grid_barrier<false>(P, epoch, S)) goto out;
         double tot[3];
-        grid_totals_1k<3>(P, set, tot, quarter, wmax);
+        grid_totals_1k<3>(P, set, tot, quarter);
         set ^= 1;
         if (tid == 0) {
             rr = tot[0];
@@ -684,26 +678,12 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             ctl[kCtlRun] = go;
             ctl[kCtlZeroB] = zero_b;
-            if constexpr (FX) {
-                mz = wmax[33];
-                ctl[kCtlShift] = fixed_shift(mz, 0u);
-            }
         }
         __syncthreads();
         run = ctl[kCtlRun] != 0;
         if (ctl[kCtlZeroB])   // b = 0: the solution is x = 0
             for (int t = t0; t < t1; t += kW)
                 if (t * 32 + lane < P.n) P.x[t * 32 + lane] = 0.0;
-        if constexpr (FX) {
-            if (run) {   // z_0's integers, now that their shift is known (p_0 = z_0)
-                S = ctl[kCtlShift];
-                for (int t = t0; t < t1; t += kW) {
-                    const int row = t * 32 + lane;
-                    if (row < P.n) zx[row] = fixed_publish(pv[row], F.c[row], S);
-                }
-                if (!grid_barrier<false>(P, epoch, SM)) goto out;
-            }
-        }
     }
 
     // ---- the CG loop
@@ -714,39 +694,22 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
         for (int k = 1; k <= P.maxit; ++k) {
             // phase A: q = A z + beta q (= A p), p = z + beta p; p . q
             double v1[1] = {0.0};
-            unsigned int mq = 0;   // FX: bound on M q, from which the next z's shift follows
             for (int t = t0; t < t1; t += kW) {
+                const double az = sell_slice_sum<kSellUnrollMem>(M, t, zg, 0.0);
                 const int row = t * 32 + lane;
-                double az;
-                if constexpr (FX) {
-                    FixedAcc acc;
-                    const long long a = M.ptr[t];
-                    fixed_slice_sum<kFixedUnroll>(F, P.n, t, a, zx, acc, 0, (int)((M.ptr[t + 1] - a) >> 5));
-                    az = row < P.n ? fixed_value(acc, F.c[row] - F.u - S) : 0.0;
-                } else {
-                    az = sell_slice_sum<kSellUnrollMem>(M, t, zg, 0.0);
-                }
                 if (row < P.n) {
-                    double zi;
-                    if constexpr (FX) zi = PRE ? __ldg(P.dinv + row) * P.r[row] : P.r[row];
-                    else zi = zg[row];
                     const double qi = fma(beta, P.q[row], az);
-                    const double pi = fma(beta, pv[row], zi);
+                    const double pi = fma(beta, pv[row], zg[row]);
                     P.q[row] = qi;
                     pv[row] = pi;
                     v1[0] = fma(pi, qi, v1[0]);
-                    if constexpr (FX) {
-                        const unsigned int ub = fixed_ub(qi, F.c[row]);
-                        mq = max(mq, PRE ? fixed_ub_mul(ub, __ldg(P.dinv + row)) : ub);
-                    }
                 }
             }
-            block_sum_1k<1>(v1, red, quarter, wmax, mq);
+            block_sum_1k<1>(v1, red, quarter);
             publish_partials<1>(P, set, v1);
-            if constexpr (FX) publish_max(P, set, wmax[32]);
-            if (!grid_barrier<false>(P, epoch, SM)) goto out;
+            if (!grid_barrier<false>(P, epoch, S)) goto out;
             double sg[1];
-            grid_totals_1k<1>(P, set, sg, quarter, wmax);
+            grid_totals_1k<1>(P, set, sg, quarter);
             set ^= 1;
             if (tid == 0) {
                 const double sigma = sg[0];
@@ -754,16 +717,12 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                 if (!finite_bits(sigma)) status = CG_ENAN;
                 else if (!(sigma > 0.0)) status = CG_EBREAKDOWN;
                 else go = 1;
-                const double al = go ? scalar_quotient(rho, sigma) : 0.0;
-                bcast[0] = al;
+                bcast[0] = go ? scalar_quotient(rho, sigma) : 0.0;
                 ctl[kCtlRun] = go;
-                if constexpr (FX) ctl[kCtlShift] = fixed_shift(mz, fixed_ub_mul(wmax[33], al));
             }
             __syncthreads();
             if (!ctl[kCtlRun]) break;
             const double alpha = bcast[0];
-            if constexpr (FX) S = ctl[kCtlShift];
-            mz = 0;
 
             // phase B: x += alpha p, r -= alpha q, z = dinv r (published); r.r, r.z
             double v2[NB];
@@ -776,26 +735,18 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
                     P.x[row] = fma(alpha, pv[row], P.x[row]);
                     P.r[row] = ri;
                     const double zi = PRE ? __ldg(P.dinv + row) * ri : ri;
-                    if constexpr (FX) {
-                        const int c = F.c[row];
-                        zx[row] = fixed_publish(zi, c, S);
-                        mz = max(mz, fixed_ub(zi, c));
-                    } else {
-                        zg[row] = zi;
-                    }
+                    zg[row] = zi;
                     v2[0] = fma(ri, ri, v2[0]);
                     if constexpr (PRE) v2[NB - 1] = fma(ri, zi, v2[NB - 1]);
                 }
             }
-            block_sum_1k<NB>(v2, red, quarter, wmax, mz);
+            block_sum_1k<NB>(v2, red, quarter);
             publish_partials<NB>(P, set, v2);
-            if constexpr (FX) publish_max(P, set, wmax[32]);
-            if (!grid_barrier<false>(P, epoch, SM)) goto out;
+            if (!grid_barrier<false>(P, epoch, S)) goto out;
             double t2[NB];
-            grid_totals_1k<NB>(P, set, t2, quarter, wmax);
+            grid_totals_1k<NB>(P, set, t2, quarter);
             set ^= 1;
             if (tid == 0) {
-                if constexpr (FX) mz = wmax[33];
                 iters = k;
                 rr = t2[0];
                 const double rho_new = t2[NB - 1];
@@ -824,7 +775,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
         const bool want_true = ctl[kCtlTrue] != 0;
         if (tid == 0 && P.true_res && status != CG_ENAN && bb == 0.0) true_rr = 0.0;
         if (want_true) {
-            if (!grid_barrier<false>(P, epoch, SM)) goto out;  // every x entry is written
+            if (!grid_barrier<false>(P, epoch, S)) goto out;  // every x entry is written
             double v[1] = {0.0};
             for (int t = t0; t < t1; t += kW) {
                 const double ax = sell_slice_sum<kSellUnrollMem>(M, t, P.x, 0.0);
@@ -836,7 +787,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             }
             block_sum_1k<1>(v, red, quarter);
             publish_partials<1>(P, set, v);
-            if (!grid_barrier<false>(P, epoch, SM)) goto out;
+            if (!grid_barrier<false>(P, epoch, S)) goto out;
             double tt[1];
             grid_totals_1k<1>(P, set, tt, quarter);
             if (tid == 0) true_rr = tt[0];
@@ -1378,9 +1329,8 @@ const void *sell_kernel_for(bool pre, bool fx) {
     if (fx) return pre ? (const void *)cg_sell_kernel<true, true> : (const void *)cg_sell_kernel<false, true>;
     return pre ? (const void *)cg_sell_kernel<true, false> : (const void *)cg_sell_kernel<false, false>;
 }
-const void *sellmem_kernel_for(bool pre, bool fx) {
-    if (fx) return pre ? (const void *)cg_sellmem_kernel<true, true> : (const void *)cg_sellmem_kernel<false, true>;
-    return pre ? (const void *)cg_sellmem_kernel<true, false> : (const void *)cg_sellmem_kernel<false, false>;
+const void *sellmem_kernel_for(bool pre, bool) {
+    return pre ? (const void *)cg_sellmem_kernel<true> : (const void *)cg_sellmem_kernel<false>;
 }
 
 // The instantiations of a SELL-32 solve kernel prefer L1 to shared memory
@@ -1407,10 +1357,10 @@ constexpr int kRptChoices[] = {1, 2, 4};   // cg_plan.reg_rows
 
 namespace {
 
-// The fixed-point copy of the handle's SELL-32 matrix (fixed.cuh), where the
-// matrix is eligible; otherwise the handle keeps the FP64 product.
-int build_fixed(cg_handle *h, size_t entries) {
-    if (!h->sell_c16) return CG_OK;
+// The row exponents and the scale of the handle's fixed-point matrix
+// (fixed.cuh); *ok tells whether the matrix is eligible.
+int fixed_scales(cg_handle *h, bool *ok) {
+    *ok = false;
     const SellMatrix M = sell_of(h);
     const int blocks = (M.nslices + 7) / 8;
     unsigned int *stat = nullptr, got[4] = {0, 0, 0, 0};
@@ -1424,16 +1374,109 @@ int build_fixed(cg_handle *h, size_t entries) {
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(got, stat, sizeof got, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e);
-    const int top = (int)got[1] - kFixedExpOffset;   // every scaled entry is below 2^top
+    const int top = (int)got[1] - kFixedExpOffset;        // every scaled entry is below 2^top
     const int spread = (int)got[2] + (int)got[3] - 256;   // largest c_i - c_j
-    if (got[0] != 0 || top > 3 || spread > kFixedSpreadC) return CG_OK;   // 2^(3 + 3) bounds a row's sum
+    *ok = got[0] == 0 && top <= 3 && spread <= kFixedSpreadC;   // 2^(3 + 3) bounds a row's sum
     h->fixed_u = kFixedBitsA - top;
+    return CG_OK;
+}
+
+// The fixed-point copy of the handle's SELL-32 matrix, for the slice and
+// cluster kernels.
+int build_fixed(cg_handle *h, size_t entries) {
+    bool ok = false;
+    int rc = h->sell_c16 ? fixed_scales(h, &ok) : CG_OK;
+    if (rc != CG_OK || !ok) return rc;
+    const SellMatrix M = sell_of(h);
     if ((rc = dev_alloc(h, &h->fixed_vals, entries)) != CG_OK) return rc;
-    fixed_build_kernel<<<blocks, 256>>>(M, h->fixed_c, h->fixed_u, h->fixed_vals);
-    e = cudaGetLastError();
+    fixed_build_kernel<<<(M.nslices + 7) / 8, 256>>>(M, h->fixed_c, h->fixed_u, h->fixed_vals);
+    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     return e == cudaSuccess ? CG_OK : cuda_fail(e);
 }
+
+RingMatrix ring_of(const cg_handle *h) {
+    return RingMatrix{h->n,        h->sell_slices, h->ring_slots, h->ring_slot_bytes,
+                      h->ring_pad, h->ring_stream, h->ring_meta,  h->ring_blob};
+}
+
+// The ring's copy of the matrix with values of type VT, where the rows' offsets
+// have enough in common: at most kRingMaxWidth per slice and at most a quarter
+// more entries than SELL-32 stores.
+template <class VT>
+int build_ring(cg_handle *h, const void *const *kernels, int nkernels, size_t sell_entries, int max_slices, int l2) {
+    constexpr int VB = (int)sizeof(VT);
+    const SellMatrix M = sell_of(h);
+    const int blocks = (M.nslices + 7) / 8;
+    int32_t *width = nullptr;
+    unsigned int *flags = nullptr, got[2] = {0, 0};
+    int optin = 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess)
+        return CG_ECUDA;
+    int rc;
+    if ((rc = dev_alloc(h, &width, (size_t)M.nslices)) || (rc = dev_alloc(h, &flags, 2))) return rc;
+    std::vector<int32_t> wid((size_t)M.nslices);
+    cudaError_t e = cudaMemset(flags, 0, sizeof got);
+    ring_count_kernel<<<blocks, 256>>>(M, width, flags);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(got, flags, sizeof got, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(wid.data(), width, sizeof(int32_t) * wid.size(), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return cuda_fail(e);
+    std::vector<int2> meta((size_t)M.nslices);
+    size_t at = 0, entries = 0;
+    int wmax = 0;
+    for (int t = 0; t < M.nslices; ++t) {
+        meta[t] = make_int2((int)at, wid[t]);
+        at += (size_t)ring_bytes<VB>(wid[t]) / 16;
+        entries += 32 * (size_t)wid[t];
+        wmax = std::max(wmax, wid[t]);
+    }
+    if (got[0] || 4 * entries > 5 * sell_entries || got[1] > (unsigned)h->n || at > (size_t)INT32_MAX) return CG_OK;
+    if (((size_t)h->n + 2 * (size_t)got[1] + 128) * 8 > (size_t)INT32_MAX) return CG_OK;   // 32-bit byte offsets
+    // slots: as many as the CTA with the most slices needs, within the room that
+    // leaves L1 enough for the gathered vector
+    const size_t room = kRingBytes;
+    const int slot_bytes = std::max(16, ring_bytes<VB>(wmax));
+    const int slots = std::min({kRingMaxSlots, std::max(1, max_slices), (int)(room / slot_bytes)});
+    for (int i = 0; i < nkernels; ++i) {
+        int occ = 0;
+        cudaFuncAttributes fa{};
+        // the limit is the kernel's, not the handle's: always the largest
+        if (cudaFuncGetAttributes(&fa, kernels[i]) != cudaSuccess ||
+            cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 optin - (int)fa.sharedSizeBytes) != cudaSuccess)
+            return CG_ECUDA;
+        if (slots * slot_bytes > optin - (int)fa.sharedSizeBytes) return CG_OK;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernels[i], kSellSolveThreads,
+                                                          (size_t)slots * slot_bytes) != cudaSuccess)
+            return CG_ECUDA;
+        if (occ < 1) return CG_OK;
+    }
+    h->ring_slots = slots;
+    h->ring_slot_bytes = slot_bytes;
+    h->ring_pad = ((int)got[1] + 32 + 15) / 16 * 16;
+    h->ring_stream = 16.0 * (double)at + 64.0 * (double)h->n > 0.6 * l2;
+    double *z = nullptr;   // int2 or float entries
+    const size_t zlen = (size_t)h->n + 2 * (size_t)h->ring_pad;
+    unsigned char *blob = nullptr;
+    if ((rc = dev_alloc(h, &h->ring_meta, meta.size())) || (rc = dev_alloc(h, &blob, at * 16)) ||
+        (rc = dev_alloc(h, &z, VB == 8 ? zlen : (zlen + 1) / 2)))
+        return rc;
+    e = cudaMemcpy(h->ring_meta, meta.data(), sizeof(int2) * meta.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(z, 0, (VB == 8 ? 8 : 4) * zlen);
+    if (e == cudaSuccess) {
+        ring_fill_kernel<VT><<<blocks, 256>>>(M, h->ring_meta, blob, h->fixed_c, h->fixed_u);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess) return cuda_fail(e);
+    h->ring_z = z;
+    h->ring_blob = blob;
+    return CG_OK;
+}
+
+// Shared memory of the ring.
+size_t ring_smem(const cg_handle *h) { return (size_t)h->ring_slots * h->ring_slot_bytes; }
 
 void free_handle(cg_handle *h) {
     if (!h) return;
@@ -1532,11 +1575,27 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
             const cudaLaunchConfig_t cfg = cluster_config(h, &at);
             e = precond ? cudaLaunchKernelEx(&cfg, cg_cluster_kernel<true>, P, M, F, L)
                         : cudaLaunchKernelEx(&cfg, cg_cluster_kernel<false>, P, M, F, L);
+        } else if (h->ring_blob) {
+            SellMatrix M = sell_of(h);
+            RingMatrix R = ring_of(h);
+            const int32_t *cut = h->sell_cut;
+            const int8_t *c = h->fixed_c;
+            int u = h->fixed_u;
+            void *z = h->ring_z;
+            void *args64[] = {&P, &M, &R, &c, &u, &z, &cut}, *args_ir[] = {&P, &M, &R, &z, &cut};
+            const bool fp64 = h->opts.inner_values == CG_VALUES_FP64;
+            const void *kern = fp64 ? (precond ? (const void *)cg_ring_kernel<true> : (const void *)cg_ring_kernel<false>)
+                               : h->opts.inner_values == CG_VALUES_FP32
+                                   ? (const void *)cg_irring_kernel<float>
+                                   : (const void *)cg_irring_kernel<__nv_bfloat16>;
+            e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), fp64 ? args64 : args_ir,
+                                            ring_smem(h), h->stream);
         } else if ((h->sell_solve || h->sell_mem) && h->opts.inner_values == CG_VALUES_FP64) {
             SellMatrix M = sell_of(h);
             FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
             const int32_t *cut = h->sell_cut;
-            void *args[] = {&P, &M, &F, &cut};
+            void *args_slice[] = {&P, &M, &F, &cut}, *args_mem[] = {&P, &M, &cut};
+            void **args = h->sell_solve ? args_slice : args_mem;
             const bool pre = precond != 0, fx = h->fixed_vals != nullptr;
             const void *kern = h->sell_solve ? sell_kernel_for(pre, fx) : sellmem_kernel_for(pre, fx);
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), args, 0, h->stream);
@@ -1882,6 +1941,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         const std::vector<int32_t> cut =
             opts.vectors_in_memory || n == 0 ? std::vector<int32_t>{}
                                              : split_slices(sh.ptr, ctas, kSliceMaxPerCta, kSliceVecCost);
+        std::vector<int32_t> scut;   // the slice ranges of the solve kernels' CTAs
         h->sell_solve = 0;
         if (!cut.empty()) {
             bool resident = false;
@@ -1899,6 +1959,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                                cudaMemcpyHostToDevice) != cudaSuccess)
                     return fail(CG_ECUDA);
                 h->sell_solve = 1;
+                scut = cut;
             }
         }
         // larger systems: the SELL-32 kernel with the vectors in memory, slices
@@ -1914,15 +1975,52 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                     cudaSuccess)
                     return fail(CG_ECUDA);
                 h->sell_mem = 1;
+                scut = mcut;
             }
         }
-        // refinement on the SELL copies, for the systems of the slice kernel:
-        // the low-precision off-diagonals in the same layout (the builder on
-        // the low values widened to double: FP32 and BF16 values are exact in
-        // double, diagonal slots stay 0).  Larger systems keep the tiled
-        // refinement kernel, whose inner iteration hides more memory latency
-        // (measured at 100^3: 59 against 77 us per FP32 inner iteration).
-        if (mixed && h->sell_solve) {
+        const size_t tot = sh.vals.size();
+        if ((rc = dev_alloc(h, &h->sell_ptr, sh.ptr.size())) || (rc = dev_alloc(h, &h->sell_vals, tot)))
+            return fail(rc);
+        if (sh.rel16) rc = dev_alloc(h, &h->sell_c16, tot);
+        else rc = dev_alloc(h, &h->sell_c32, tot);
+        if (rc) return fail(rc);
+        cudaError_t es = cudaMemcpy(h->sell_ptr, sh.ptr.data(), sizeof(long long) * sh.ptr.size(),
+                                    cudaMemcpyHostToDevice);
+        if (es == cudaSuccess && tot)
+            es = cudaMemcpy(h->sell_vals, sh.vals.data(), sizeof(double) * tot, cudaMemcpyHostToDevice);
+        if (es == cudaSuccess && tot)
+            es = sh.rel16 ? cudaMemcpy(h->sell_c16, sh.cols16.data(), 2 * tot, cudaMemcpyHostToDevice)
+                          : cudaMemcpy(h->sell_c32, sh.cols32.data(), 4 * tot, cudaMemcpyHostToDevice);
+        if (es != cudaSuccess) return fail(cuda_fail(es));
+        // the fixed-point product in the slice and cluster kernels, and the ring
+        // for FP64 solves of larger systems and for every refinement, where the
+        // matrix allows them.  Per iteration, ring against what ran before: FP64
+        // CG 100^3 55 us (73), 65^3 19.7 (26.7), Jacobi-PCG on 161820 rows 17.8
+        // (22.2, and 18.6 with fixed-point SELL-32); FP32 refinement 100^3 28.6
+        // (48.7), 57x44x61 11.1 (18.1), 50^3 9.7 (13.8), 20^3 9.1 (13.9).
+        int max_slices = 0;
+        for (size_t c = 0; c + 1 < scut.size(); ++c) max_slices = std::max(max_slices, scut[c + 1] - scut[c]);
+        if (h->sell_solve && !mixed && (rc = build_fixed(h, tot)) != CG_OK) return fail(rc);
+        if (h->sell_mem && !mixed) {
+            bool ok = false;
+            const void *k[] = {(const void *)cg_ring_kernel<false>, (const void *)cg_ring_kernel<true>};
+            if ((rc = fixed_scales(h, &ok)) != CG_OK) return fail(rc);
+            if (ok && (rc = build_ring<int2>(h, k, 2, tot, max_slices, l2)) != CG_OK) return fail(rc);
+        } else if ((h->sell_solve || h->sell_mem) && mixed) {
+            const void *k32[] = {(const void *)cg_irring_kernel<float>, (const void *)lo_spmv_ring_kernel<float>};
+            const void *k16[] = {(const void *)cg_irring_kernel<__nv_bfloat16>,
+                                 (const void *)lo_spmv_ring_kernel<__nv_bfloat16>};
+            rc = opts.inner_values == CG_VALUES_FP32 ? build_ring<float>(h, k32, 2, tot, max_slices, l2)
+                                                     : build_ring<__nv_bfloat16>(h, k16, 2, tot, max_slices, l2);
+            if (rc != CG_OK) return fail(rc);
+        }
+        // refinement of matrices without common offsets, on the SELL copies for
+        // the systems of the slice kernel: the low-precision off-diagonals in the
+        // same layout (the builder on the low values widened to double: FP32 and
+        // BF16 values are exact in double, diagonal slots stay 0).  Larger ones
+        // keep the tiled refinement kernel, whose inner iteration hides more
+        // memory latency.
+        if (mixed && h->sell_solve && !h->ring_blob) {
             int occ32 = 0, occ16 = 0;
             const bool ok =
                 cudaFuncSetAttribute((const void *)cg_irsell_kernel<float>,
@@ -1961,25 +2059,6 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                 if (el != cudaSuccess) return fail(cuda_fail(el));
             }
         }
-        const size_t tot = sh.vals.size();
-        if ((rc = dev_alloc(h, &h->sell_ptr, sh.ptr.size())) || (rc = dev_alloc(h, &h->sell_vals, tot)))
-            return fail(rc);
-        if (sh.rel16) rc = dev_alloc(h, &h->sell_c16, tot);
-        else rc = dev_alloc(h, &h->sell_c32, tot);
-        if (rc) return fail(rc);
-        cudaError_t es = cudaMemcpy(h->sell_ptr, sh.ptr.data(), sizeof(long long) * sh.ptr.size(),
-                                    cudaMemcpyHostToDevice);
-        if (es == cudaSuccess && tot)
-            es = cudaMemcpy(h->sell_vals, sh.vals.data(), sizeof(double) * tot, cudaMemcpyHostToDevice);
-        if (es == cudaSuccess && tot)
-            es = sh.rel16 ? cudaMemcpy(h->sell_c16, sh.cols16.data(), 2 * tot, cudaMemcpyHostToDevice)
-                          : cudaMemcpy(h->sell_c32, sh.cols32.data(), 4 * tot, cudaMemcpyHostToDevice);
-        if (es != cudaSuccess) return fail(cuda_fail(es));
-        // the fixed-point product: where the FP64 pipe, not HBM, sets the pace
-        // of the FP64 one (at 100^3, streaming the matrix, 73.8 against 73.1 us
-        // per iteration: no gain)
-        if ((h->sell_solve || (h->sell_mem && !h->evict_first)) && !mixed && (rc = build_fixed(h, tot)) != CG_OK)
-            return fail(rc);
         // small systems: the whole solve inside one cluster (a caller that sets
         // the CTA count, or tests the grid barrier, gets the grid)
         if (h->sell_solve && h->fixed_vals && opts.grid_ctas == 0 && opts.debug_phantom_arrivals == 0 &&
@@ -2131,12 +2210,21 @@ int cg_spmv_inner(cg_handle *h, const float *x, float *y) {
     if (!x || !y) return CG_EINVAL;
     DeviceGuard g(h->device);
     // the inner kernels gather from the handle's padded, 16-byte aligned p32
-    cudaError_t e = cudaMemcpyAsync(h->p32, x, sizeof(float) * (size_t)h->n, cudaMemcpyDeviceToDevice, h->stream);
+    float *const gathered = h->ring_blob ? static_cast<float *>(h->ring_z) + h->ring_pad : h->p32;
+    cudaError_t e = cudaMemcpyAsync(gathered, x, sizeof(float) * (size_t)h->n, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->st, 0, sizeof(DevStatus), h->stream);
     if (e == cudaSuccess) {
         Params P = base_params(h);
         const bool fp32 = h->opts.inner_values == CG_VALUES_FP32;
-        if (h->sell_lo) {
+        if (h->ring_blob) {
+            const RingMatrix R = ring_of(h);
+            const float *zf = static_cast<const float *>(h->ring_z);
+            if (fp32)
+                lo_spmv_ring_kernel<float><<<h->ctas, kSellSolveThreads, ring_smem(h), h->stream>>>(P, R, zf, h->sell_cut, y);
+            else
+                lo_spmv_ring_kernel<__nv_bfloat16>
+                    <<<h->ctas, kSellSolveThreads, ring_smem(h), h->stream>>>(P, R, zf, h->sell_cut, y);
+        } else if (h->sell_lo) {
             const SellMatrix M = sell_of(h);
             if (fp32)
                 lo_spmv_sell_kernel<float><<<h->ctas, kSellSolveThreads, 0, h->stream>>>(
@@ -2175,7 +2263,7 @@ int cg_get_plan(const cg_handle *h, cg_plan *plan) {
     p.window_tiles = h->window_tiles;
     p.device_bytes = h->device_bytes;
     p.slice_solve = h->sell_solve ? 1 : (h->sell_mem && h->rpt == 0 ? 2 : 0);
-    p.inner_solve = h->sell_lo ? 1 : 0;
+    p.inner_solve = h->sell_lo || (h->ring_blob && h->sell_solve && h->opts.inner_values != CG_VALUES_FP64) ? 1 : 0;
     *plan = p;
     return CG_OK;
 }

@@ -61,6 +61,12 @@ struct cg_handle {
     int2 *fixed_vals = nullptr;       // fixed-point copy of the SELL values (fixed.cuh), or nullptr
     int8_t *fixed_c = nullptr;        // its exponent per row
     int fixed_u = 0;                  // and of the whole matrix
+    // slices with common offsets in a shared-memory ring (ring.cuh): the matrix of
+    // the FP64 solve's fixed-point product, or of the inner solve of refinement
+    int2 *ring_meta = nullptr;
+    unsigned char *ring_blob = nullptr;   // nullptr: not used
+    void *ring_z = nullptr;               // the gathered vector, with its margins
+    int ring_pad = 0, ring_slots = 0, ring_slot_bytes = 0, ring_stream = 0;
     int cluster_ctas = 0;             // CTAs of the one-cluster solve (cluster.cuh), 0: not used
     int cluster_threads = 0, cluster_entries = 0, cluster_window = 0;
     size_t cluster_smem = 0;
