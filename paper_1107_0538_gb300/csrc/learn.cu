@@ -258,8 +258,11 @@ struct ConvArgs {
     const __nv_bfloat16 *gate;   // gates (padded, 16 channels)
     float *dg;                   // E_BWD_GATE: gate-gradient field (padded, 16 channels, FP32)
     int dg_add;                  // 0: dg = ..., 1: dg += ...
+    __nv_bfloat16 *dag;          // E_BWD_GATE: if set, dg g (1 - g) goes here and dg is complete (not stored)
     // conv_out
-    float *u;                    // E_OUT_U: node-order FP32 output
+    const float *ehat;           // E_OUT_LOSS: v = u - e_hat, t = D^-1/2 v (node order)
+    float *v;
+    double *t;
     double *z;                   // E_OUT_Z / E_OUT_FCG
     const double *r;             // E_OUT_FCG: residual (node order)
     const double *q;             // E_OUT_FCG: A p of the last step
@@ -272,7 +275,7 @@ struct ConvArgs {
 };
 
 enum { E_STORE = 0, E_GATE = 1, E_GATE_PRE = 2, E_BWD_GATE = 3, E_SIGMOID = 4 };
-enum { E_OUT_U = 0, E_OUT_Z = 1, E_OUT_FCG = 2 };
+enum { E_OUT_LOSS = 0, E_OUT_Z = 1, E_OUT_FCG = 2 };
 
 __device__ __forceinline__ bool conv_skip(const FcgState *st) {
     return st && (st->done || st->mode != kModeLearned);
@@ -331,7 +334,12 @@ __device__ __forceinline__ void store16(const ConvArgs &A, const Brick &B, int w
                         float2 dv = A.dg_add ? *d : make_float2(0.0f, 0.0f);
                         dv.x = fmaf(pv.x, v0, dv.x);
                         dv.y = fmaf(pv.y, v1, dv.y);
-                        *d = dv;
+                        if (A.dag) {
+                            const uint32_t dw = pack_bf16(dv.x * gv.x * (1.0f - gv.x), dv.y * gv.y * (1.0f - gv.y));
+                            *reinterpret_cast<uint32_t *>(A.dag + e) = dw;
+                        } else {
+                            *d = dv;
+                        }
                     }
                     *reinterpret_cast<uint32_t *>(A.out + e) = pack_bf16(gv.x * v0, gv.y * v1);
                 }
@@ -722,7 +730,7 @@ __device__ __forceinline__ void finish(FcgState *st, int status) {
 
 // ------------------------------------------------ 16 -> 1 convolution
 // u[p] = sum_{t, c} K[t][c] x[c, p + off(t)] (K packed [27][16]).  EPI:
-// E_OUT_U stores u (FP32, node order), E_OUT_Z stores z = sigma D^-1/2 u,
+// E_OUT_LOSS stores v = u - e_hat and D^-1/2 v (training), E_OUT_Z stores z = sigma D^-1/2 u,
 // E_OUT_FCG also forms z.r and z.q and takes the flexible-CG decisions (in
 // the Jacobi fallback it forms z = D^-1 r instead of running the network).
 //
@@ -801,9 +809,12 @@ __device__ __forceinline__ OutNodes out_nodes(const ConvArgs &A, const Brick &B,
     o.ok0 = rowok && ox < G.nx;
     o.ok1 = rowok && ox + 1 < G.nx;
     o.i0 = ox + G.nx * (gy + G.ny * gz);
-    if (EPI != E_OUT_U) {
-        if (o.ok0) o.d0 = __ldg(A.dsq32 + o.i0);
-        if (o.ok1) o.d1 = __ldg(A.dsq32 + o.i0 + 1);
+    const float *d = EPI == E_OUT_LOSS ? A.ehat : A.dsq32;
+    if (o.ok0) o.d0 = __ldg(d + o.i0);
+    if (o.ok1) o.d1 = __ldg(d + o.i0 + 1);
+    if (EPI == E_OUT_LOSS) {
+        if (o.ok0) o.q0 = __ldg(A.dsq + o.i0);
+        if (o.ok1) o.q1 = __ldg(A.dsq + o.i0 + 1);
     }
     if (EPI == E_OUT_FCG) {
         if (o.ok0) {
@@ -841,7 +852,7 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
         const int j4 = threadIdx.x & 3, quad = threadIdx.x >> 2;
         const int xh = quad & 1, brow = quad >> 1;
         const int oy = brow % kBY, oz = brow / kBY;
-        const float sigma = EPI == E_OUT_U ? 1.0f : (float)(st ? st->sigma : A.sigma[0]);
+        const float sigma = EPI == E_OUT_LOSS ? 1.0f : (float)(st ? st->sigma : A.sigma[0]);
         // the CTA's bricks b = blockIdx.x, + gridDim.x, ...: brick k is
         // multiplied from buffer k mod 2 while brick k + 1 is staged into the
         // other one, and the epilogue operands of a lane's two nodes are
@@ -911,9 +922,16 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
             // FP32 adds nothing to its error), widened for the FP64 dots
             const float u0 = j4 == 0 ? acc[0] : j4 == 1 ? acc[2] : j4 == 2 ? acc[4] : acc[6];
             const float u1 = j4 == 0 ? acc[1] : j4 == 1 ? acc[3] : j4 == 2 ? acc[5] : acc[7];
-            if (EPI == E_OUT_U) {
-                if (nd.ok0) A.u[nd.i0] = u0;
-                if (nd.ok1) A.u[nd.i0 + 1] = u1;
+            if (EPI == E_OUT_LOSS) {
+                const float v0 = u0 - nd.d0, v1 = u1 - nd.d1;
+                if (nd.ok0) {
+                    A.v[nd.i0] = v0;
+                    A.t[nd.i0] = nd.q0 * (double)v0;
+                }
+                if (nd.ok1) {
+                    A.v[nd.i0 + 1] = v1;
+                    A.t[nd.i0 + 1] = nd.q1 * (double)v1;
+                }
             } else {
                 const double z0 = nd.ok0 ? (double)(sigma * nd.d0 * u0) : 0.0;
                 const double z1 = nd.ok1 ? (double)(sigma * nd.d1 * u1) : 0.0;
@@ -1361,9 +1379,7 @@ struct TrainArgs {
     double *partials;
     __nv_bfloat16 *shat;      // padded, 1 channel
     float *ehat;              // node order
-    const float *u;           // network output (node order)
-    float *v;                 // u - e_hat
-    double *t;                // D^-1/2 v (SpMV input)
+    const float *v;           // network output minus e_hat (node order)
     const double *y;          // A t
     __nv_bfloat16 *du;        // padded, 1 channel: A_hat v (n times the loss gradient)
     const int32_t *pidx;      // padded position of each node
@@ -1399,15 +1415,6 @@ __global__ void __launch_bounds__(kVT) pair_input_kernel(TrainArgs T) {
     }
 }
 
-// v = u - e_hat, t = D^-1/2 v.
-__global__ void __launch_bounds__(kVT) loss_prep_kernel(TrainArgs T) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < T.G.n; i += gridDim.x * blockDim.x) {
-        const float vi = T.u[i] - T.ehat[i];
-        T.v[i] = vi;
-        T.t[i] = T.dsq[i] * (double)vi;
-    }
-}
-
 // w = D^-1/2 A t = A_hat v; loss += v.w / 2n; du = w (padded BF16).
 __global__ void __launch_bounds__(kVT) loss_kernel(TrainArgs T) {
     __shared__ double sred[32];
@@ -1422,16 +1429,6 @@ __global__ void __launch_bounds__(kVT) loss_kernel(TrainArgs T) {
     cta_sum<1>(a, sred);
     if (!last_cta_totals<1>(a, T.partials, T.counter, tot, &sflag, sred)) return;
     if (threadIdx.x == 0) T.scal[2] += 0.5 * tot[0] / (double)T.G.n;
-}
-
-// dag = dg * g (1 - g) over the whole padded 16-channel field (zero halos stay zero).
-__global__ void __launch_bounds__(kVT) gate_grad_kernel(long long count, const float *dg, const __nv_bfloat16 *gate,
-                                                       __nv_bfloat16 *dag) {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;
-         k += (long long)gridDim.x * blockDim.x) {
-        const float gv = __bfloat162float(gate[k]);
-        dag[k] = __float2bfloat16_rn(dg[k] * gv * (1.0f - gv));
-    }
 }
 
 struct WgArgs {
@@ -1463,17 +1460,11 @@ __device__ __forceinline__ void stage_dy(const Geo &G, const Brick &B, const __n
     }
 }
 
-// Staged input row of dy row `row` (= zl * kBY + yl), shifted by a tap.
-__device__ __forceinline__ int x_row(int row, int dx, int dy, int dz) {
-    const int yl = row % kBY, zl = row / kBY;
-    return ((zl + 1 + dz) * kSY + (yl + 1 + dy)) * kSX + 1 + dx;
-}
-
 // G[o][c][t] = sum_p dy[o, p] x[c, p + off(t)] for 16-channel dy and x: a
 // GEMM over positions (M = o, N = c, K = p) per tap; warp w owns taps
 // w, w + 8, ...  Persistent over bricks; the CTA's sums go to part[blockIdx.x].
 // dy is zero off the interior nodes, so dropped positions add nothing.
-__global__ void __launch_bounds__(kCT) wgrad16_kernel(WgArgs W) {
+__global__ void __launch_bounds__(kCT, 3) wgrad16_kernel(WgArgs W) {
     extern __shared__ __align__(128) unsigned char sm[];
     const Geo &G = W.G;
     unsigned char *sdy = sm + kStage16;
@@ -1490,29 +1481,44 @@ __global__ void __launch_bounds__(kCT) wgrad16_kernel(WgArgs W) {
     const uint32_t in_base = smem_u32(sm), dy_base = smem_u32(sdy);
     const int a_pos = (lane & 7) + ((lane >> 4) << 3), a_half = (lane >> 3) & 1;
     const int b_pos = (lane & 7) + (((lane >> 3) & 1) << 3), b_half = lane >> 4;
+    int toff[kMaxT];   // staged rows from the centre to the tap
+    static_assert(kWarpsC * (kMaxT - 1) <= kTaps, "only the last tap of a warp may be missing");
+#pragma unroll
+    for (int i = 0; i < kMaxT; ++i) {
+        const int t = min(w + kWarpsC * i, kTaps - 1);
+        toff[i] = (tap_dz(t) * kSY + tap_dy(t)) * kSX + tap_dx(t);
+    }
     for (int tile = blockIdx.x; tile < G.tiles; tile += gridDim.x) {
         const Brick B = brick_of(G, tile);
         stage16(G, B, W.x, sm);
         stage_dy(G, B, W.dy, sdy);
         cp_async_wait_all();
         __syncthreads();
-        for (int row = 0; row < kRows; ++row) {
-            uint32_t a[4];
-            ldsm_x4_t(a, row_addr(dy_base, row * kBX + a_pos, a_half));
+        // row = zl kBY + yl of dy; the centre of its input row in the stage, to
+        // which the tap's offset is added (computed once: index arithmetic per
+        // tap and row, not the MMAs, was this kernel's time)
+        for (int zl = 0; zl < kBZ; ++zl)
+#pragma unroll 2
+            for (int yl = 0; yl < kBY; ++yl) {
+                uint32_t a[4];
+                ldsm_x4_t(a, row_addr(dy_base, (zl * kBY + yl) * kBX + a_pos, a_half));
+                const int centre = ((zl + 1) * kSY + yl + 1) * kSX + 1 + b_pos;
 #pragma unroll
-            for (int i = 0; i < kMaxT; ++i) {
-                const int t = w + kWarpsC * i;
-                if (t < kTaps) {
-                    uint32_t b[4];
-                    ldsm_x4_t(b, row_addr(in_base, x_row(row, tap_dx(t), tap_dy(t), tap_dz(t)) + b_pos, b_half));
-                    mma_bf16(acc[i][0], a, b[0], b[1]);
-                    mma_bf16(acc[i][1], a, b[2], b[3]);
+                for (int i = 0; i < kMaxT; ++i) {
+                    if (i + 1 < kMaxT || w + kWarpsC * i < kTaps) {
+                        uint32_t b[4];
+                        ldsm_x4_t(b, row_addr(in_base, centre + toff[i], b_half));
+                        mma_bf16(acc[i][0], a, b[0], b[1]);
+                        mma_bf16(acc[i][1], a, b[2], b[3]);
+                    }
                 }
             }
-        }
         __syncthreads();
     }
-    float *part = W.part + (size_t)blockIdx.x * CG_LEARN_PARAMS + W.off;
+    // the parts keep this weight as [t][o][c]: four lanes write a whole 32-byte
+    // sector ([o][c][t], 4 bytes every 108, took most of the kernel's time:
+    // 54 us at 50^3, 15 now)
+    float2 *part = reinterpret_cast<float2 *>(W.part + (size_t)blockIdx.x * CG_LEARN_PARAMS + W.off);
 #pragma unroll
     for (int i = 0; i < kMaxT; ++i) {
         const int t = w + kWarpsC * i;
@@ -1520,10 +1526,15 @@ __global__ void __launch_bounds__(kCT) wgrad16_kernel(WgArgs W) {
 #pragma unroll
         for (int nb = 0; nb < 2; ++nb)
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int o = g + 8 * (k >> 1), c = nb * 8 + 2 * t4 + (k & 1);
-                float *dst = part + (o * kCh + c) * kTaps + t;
-                *dst = W.add ? *dst + acc[i][nb][k] : acc[i][nb][k];
+            for (int hr = 0; hr < 2; ++hr) {
+                float2 *dst = part + ((t * kCh + g + 8 * hr) * kCh + nb * 8 + 2 * t4) / 2;
+                float2 v = make_float2(acc[i][nb][2 * hr], acc[i][nb][2 * hr + 1]);
+                if (W.add) {
+                    const float2 old = *dst;
+                    v.x += old.x;
+                    v.y += old.y;
+                }
+                *dst = v;
             }
     }
 }
@@ -1548,12 +1559,13 @@ __global__ void __launch_bounds__(kCT) wgrad1_kernel(WgArgs W) {
     const uint32_t dy_base = smem_u32(sdy);
     const int a_pos = (lane & 7) + ((lane >> 4) << 3), a_half = (lane >> 3) & 1;
     int tkind[4];   // 0 tap, 1 constant one, 2 zero
-    int tt_of[4];
+    int toff[4];    // staged positions from the centre to the tap
 #pragma unroll
     for (int nb = 0; nb < 4; ++nb) {
         const int t = nb * 8 + g;
         tkind[nb] = t < kTaps ? 0 : (t == kTaps && W.bias_off >= 0 ? 1 : 2);
-        tt_of[nb] = t < kTaps ? t : kCentre;
+        const int tt = t < kTaps ? t : kCentre;
+        toff[nb] = (tap_dz(tt) * kSY + tap_dy(tt)) * kSX + tap_dx(tt);
     }
     for (int tile = blockIdx.x; tile < G.tiles; tile += gridDim.x) {
         const Brick B = brick_of(G, tile);
@@ -1564,12 +1576,12 @@ __global__ void __launch_bounds__(kCT) wgrad1_kernel(WgArgs W) {
         for (int row = w; row < kRows; row += kWarpsC) {
             uint32_t a[4];
             ldsm_x4_t(a, row_addr(dy_base, row * kBX + a_pos, a_half));
+            const int centre = ((row / kBY + 1) * kSY + row % kBY + 1) * kSX + 1 + 2 * t4;
 #pragma unroll
             for (int nb = 0; nb < 4; ++nb) {
                 uint32_t b0, b1;
                 if (tkind[nb] == 0) {
-                    const int tt = tt_of[nb];
-                    const uint16_t *xp = xs + x_row(row, tap_dx(tt), tap_dy(tt), tap_dz(tt)) + 2 * t4;
+                    const uint16_t *xp = xs + centre + toff[nb];
                     b0 = pack_raw(xp[0], xp[1]);
                     b1 = pack_raw(xp[8], xp[9]);
                 } else if (tkind[nb] == 1) {
@@ -1604,13 +1616,45 @@ __global__ void __launch_bounds__(kCT) wgrad1_kernel(WgArgs W) {
     }
 }
 
-// grad[j] += sum over CTAs (in order) of part[cta][j].
-__global__ void __launch_bounds__(kVT) grad_reduce_kernel(const float *part, int nparts, float *grad) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= CG_LEARN_PARAMS) return;
+// The partial gradients of a mini-batch: one array of CTAs per lane.
+constexpr int kTrainLanes = 4;
+struct GradParts {
+    const float *part[kTrainLanes];
+    double *scal[kTrainLanes];   // the lanes' scalars; [2]: loss sum
+    int lanes, ctas;
+};
+
+// grad += sum over lanes and CTAs of the parts, in a fixed order: thread (g, j)
+// of a block adds every kRedGroups-th CTA's entry j, then the groups are added
+// in order.  The 16 x 16 weight's entries are [t][o][c] in the parts.  The
+// lanes' loss sums go to loss[0] and are cleared.
+constexpr int kRedGroups = 32;
+__global__ void __launch_bounds__(32 * kRedGroups) grad_reduce_kernel(GradParts P, float *grad, double *loss) {
+    __shared__ float sum[kRedGroups][32];
+    const int jl = threadIdx.x & 31, g = threadIdx.x >> 5, j = blockIdx.x * 32 + jl;
     float s = 0.0f;
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * CG_LEARN_PARAMS + j];
-    grad[j] += s;
+    if (j < CG_LEARN_PARAMS)
+        for (int l = 0; l < P.lanes; ++l)
+#pragma unroll 8
+            for (int c = g; c < P.ctas; c += kRedGroups) s += P.part[l][(size_t)c * CG_LEARN_PARAMS + j];
+    sum[g][jl] = s;
+    __syncthreads();
+    if (g == 0 && j < CG_LEARN_PARAMS) {
+        float t = sum[0][jl];
+#pragma unroll
+        for (int k = 1; k < kRedGroups; ++k) t += sum[k][jl];
+        int dst = j;
+        if (j >= kOffW2 && j < kOffWg) {
+            const int tap = (j - kOffW2) / (kCh * kCh), oc = (j - kOffW2) % (kCh * kCh);
+            dst = kOffW2 + oc * kTaps + tap;
+        }
+        grad[dst] += t;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        for (int l = 0; l < P.lanes; ++l) {
+            *loss += P.scal[l][2];
+            P.scal[l][2] = 0.0;
+        }
 }
 
 struct NetDev {
@@ -1697,15 +1741,26 @@ struct cg_net {
     NetDev d{};
     void *block = nullptr;
     long long step = 0;
-    // training workspace (allocated on first use, for one grid)
+    // training workspace (allocated on first use, for one grid): up to
+    // kTrainLanes lanes, each with its own stream, work on the pairs of a
+    // mini-batch in turn, because the kernels of one pair leave SMs idle
+    // (at 50^3 a convolution is 364 CTAs where 456 to 608 fit)
+    struct TrainLane {
+        cudaStream_t stream = nullptr;
+        cudaEvent_t done = nullptr;
+        __nv_bfloat16 *shat = nullptr, *a1 = nullptr, *h1 = nullptr, *h2 = nullptr, *kpre = nullptr, *k1 = nullptr;
+        __nv_bfloat16 *du = nullptr, *dk = nullptr, *dh2 = nullptr, *da1 = nullptr, *dag = nullptr;
+        float *dg = nullptr, *ehat = nullptr, *v = nullptr, *part = nullptr;
+        double *t = nullptr, *y = nullptr, *scal = nullptr, *partials = nullptr;
+        unsigned int *counter = nullptr;
+        std::vector<void *> allocs;
+    };
     Geo tg{};
     bool have_train = false;
+    std::vector<TrainLane> lanes;
+    cudaEvent_t fork = nullptr;
     std::vector<void *> tallocs;
-    __nv_bfloat16 *shat = nullptr, *a1 = nullptr, *h1 = nullptr, *h2 = nullptr, *kpre = nullptr, *k1 = nullptr;
-    __nv_bfloat16 *du = nullptr, *dk = nullptr, *dh2 = nullptr, *da1 = nullptr, *dag = nullptr;
-    float *dg = nullptr, *u = nullptr, *ehat = nullptr, *v = nullptr, *part = nullptr;
-    double *t = nullptr, *y = nullptr, *scal = nullptr, *partials = nullptr;
-    unsigned int *counter = nullptr;
+    double *scal = nullptr;    // [2]: loss sum of the mini-batch
     int loss_cap_n = 0;
     int wg_ctas = 0;
     int vgrid = 0;
@@ -1755,12 +1810,17 @@ int sm_count(int dev) {
 // at once (each loops over its share of the bricks), at most one per brick.
 template <int EPI>
 int convout_grid(const Geo &G) {
-    int dev = 0, occ = 0;
-    cudaGetDevice(&dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, convout_kernel<EPI>, kCT, convout_smem(G)) != cudaSuccess ||
-        occ < 1)
-        occ = 1;
-    return std::max(1, std::min(G.tiles, occ * sm_count(dev)));
+    // the same for every grid and device of this kind: asked for once
+    static const int resident = [&] {
+        int dev = 0, occ = 0;
+        cudaGetDevice(&dev);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, convout_kernel<EPI>, kCT, convout_smem(G)) !=
+                cudaSuccess ||
+            occ < 1)
+            occ = 1;
+        return occ * sm_count(dev);
+    }();
+    return std::max(1, std::min(G.tiles, resident));
 }
 
 template <class T>
@@ -1807,7 +1867,7 @@ int set_smem_limits() {
     set((const void *)conv16_kernel<E_BWD_GATE>);
     set((const void *)conv16tc_kernel<E_STORE>);
     set((const void *)conv16tc_kernel<E_GATE>);
-    set((const void *)convout_kernel<E_OUT_U>);
+    set((const void *)convout_kernel<E_OUT_LOSS>);
     set((const void *)convout_kernel<E_OUT_Z>);
     set((const void *)convout_kernel<E_OUT_FCG>);
     set((const void *)wgrad16_kernel);
@@ -1972,140 +2032,228 @@ int upload_params(cg_net *net, const float *params) {
     return CG_OK;
 }
 
-// Training workspace of the net for one grid.
-int ensure_train(cg_net *net, const Geo &G, int ninst_ctas) {
-    if (net->have_train && net->tg.nx == G.nx && net->tg.ny == G.ny && net->tg.nz == G.nz) return CG_OK;
+void free_lane(cg_net::TrainLane &W) {
+    for (void *p : W.allocs) cudaFree(p);
+    if (W.stream) cudaStreamDestroy(W.stream);
+    if (W.done) cudaEventDestroy(W.done);
+    W = cg_net::TrainLane{};
+}
+
+void free_train(cg_net *net) {
+    for (auto &W : net->lanes) free_lane(W);
+    net->lanes.clear();
     for (void *p : net->tallocs) cudaFree(p);
     net->tallocs.clear();
+    net->scal = nullptr;
     net->have_train = false;
-    net->tg = G;
-    net->wg_ctas = std::min(G.tiles, 2 * sm_count(net->device));
-    net->vgrid = std::min((G.n + kVT - 1) / kVT, 4 * sm_count(net->device));
-    const size_t a16 = act_count(G, kCh), a1 = act_count(G, 1);
-    auto &A = net->tallocs;
-    int rc;
-    if ((rc = ctx_alloc(A, &net->shat, a1)) || (rc = ctx_alloc(A, &net->a1, a16)) || (rc = ctx_alloc(A, &net->h1, a16)) ||
-        (rc = ctx_alloc(A, &net->h2, a16)) || (rc = ctx_alloc(A, &net->kpre, a16)) ||
-        (rc = ctx_alloc(A, &net->k1, a16)) || (rc = ctx_alloc(A, &net->du, a1)) || (rc = ctx_alloc(A, &net->dk, a16)) ||
-        (rc = ctx_alloc(A, &net->dh2, a16)) || (rc = ctx_alloc(A, &net->da1, a16)) ||
-        (rc = ctx_alloc(A, &net->dag, a16)) || (rc = ctx_alloc(A, &net->dg, a16)) ||
-        (rc = ctx_alloc(A, &net->u, (size_t)G.n)) || (rc = ctx_alloc(A, &net->ehat, (size_t)G.n)) ||
-        (rc = ctx_alloc(A, &net->v, (size_t)G.n)) || (rc = ctx_alloc(A, &net->t, (size_t)G.n + 16)) ||
-        (rc = ctx_alloc(A, &net->y, (size_t)G.n)) || (rc = ctx_alloc(A, &net->scal, 8)) ||
-        (rc = ctx_alloc(A, &net->counter, 4)) ||
-        (rc = ctx_alloc(A, &net->partials, (size_t)4 * std::max({net->vgrid, ninst_ctas, 1}))) ||
-        (rc = ctx_alloc(A, &net->part, (size_t)net->wg_ctas * CG_LEARN_PARAMS)))
+}
+
+int alloc_lane(cg_net *net, const Geo &G, int ninst_ctas, cg_net::TrainLane &W) {
+    if (cudaStreamCreateWithFlags(&W.stream, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&W.done, cudaEventDisableTiming) != cudaSuccess)
+        return CG_ECUDA;
+    // one allocation, cleared once: the fields' halos stay zero
+    const size_t a16 = act_count(G, kCh), a1 = act_count(G, 1), n = (size_t)G.n;
+    size_t total = 0;
+    char *base = nullptr;
+    auto place = [&](auto **p, size_t count) {
+        using T = std::remove_pointer_t<std::remove_pointer_t<decltype(p)>>;
+        if (base) *p = reinterpret_cast<T *>(base + total);
+        total += (count * sizeof(T) + 255) / 256 * 256;
+    };
+    for (int round = 0; round < 2; ++round) {
+        total = 0;
+        place(&W.shat, a1);
+        place(&W.du, a1);
+        for (auto *p : {&W.a1, &W.h1, &W.h2, &W.kpre, &W.k1, &W.dk, &W.dh2, &W.da1, &W.dag}) place(p, a16);
+        place(&W.dg, a16);
+        place(&W.ehat, n);
+        place(&W.v, n);
+        place(&W.t, n + 16);
+        place(&W.y, n);
+        place(&W.scal, 8);
+        place(&W.counter, 4);
+        place(&W.partials, (size_t)4 * std::max({net->vgrid, ninst_ctas, 1}));
+        place(&W.part, (size_t)net->wg_ctas * CG_LEARN_PARAMS);
+        if (round == 0) {
+            const int rc = ctx_alloc(W.allocs, &base, total, false);
+            if (rc != CG_OK) return rc;
+        }
+    }
+    return cudaMemsetAsync(base, 0, total, W.stream) == cudaSuccess ? CG_OK : CG_ECUDA;
+}
+
+// Training workspace of the net for one grid, with lanes for mini-batches of
+// `batch` pairs (fewer where memory for more is not to be had).
+int ensure_train(cg_net *net, const Geo &G, int ninst_ctas, int batch) {
+    if (!(net->have_train && net->tg.nx == G.nx && net->tg.ny == G.ny && net->tg.nz == G.nz)) {
+        free_train(net);
+        net->tg = G;
+        // as many bricks at a time as the weight-gradient kernels have resident
+        net->wg_ctas = std::min(G.tiles, 4 * sm_count(net->device));
+        net->vgrid = std::min((G.n + kVT - 1) / kVT, 4 * sm_count(net->device));
+        int rc = ctx_alloc(net->tallocs, &net->scal, 8);
+        if (rc != CG_OK) return rc;
+        net->have_train = true;
+    }
+    const size_t want = (size_t)std::min(kTrainLanes, std::max(batch, 1));
+    while (net->lanes.size() < want) {
+        net->lanes.emplace_back();
+        const int rc = alloc_lane(net, G, ninst_ctas, net->lanes.back());
+        if (rc == CG_OK) continue;
+        free_lane(net->lanes.back());
+        net->lanes.pop_back();
+        if (rc == CG_ENOMEM && !net->lanes.empty()) {
+            cudaGetLastError();
+            break;
+        }
         return rc;
-    net->have_train = true;
+    }
     return CG_OK;
 }
 
-// Loss and gradient of one pair, added to net->d.grad and scal[2] (stream net->stream).
-void enqueue_sample(cg_net *net, cg_handle *h, const float *r, const float *e) {
+// Loss and gradient of one pair on a lane: its loss is added to the lane's
+// scal[2], its gradient stored in (first) or added to the lane's parts.  The
+// instance's gates are there already.
+void enqueue_sample(cg_net *net, cg_net::TrainLane &N, bool first, cg_handle *h, const float *r, const float *e) {
     LearnCtx *L = h->learn;
     const Geo &G = L->G;
-    cudaStream_t s = net->stream;
+    cudaStream_t s = N.stream;
+    const int add = first ? 0 : 1;
     TrainArgs T{};
     T.G = G;
     T.r = r;
     T.e = e;
     T.dinv = h->dinv;
     T.dsq = L->dsq;
-    T.scal = net->scal;
-    T.counter = net->counter;
-    T.partials = net->partials;
-    T.shat = net->shat;
-    T.ehat = net->ehat;
-    T.u = net->u;
-    T.v = net->v;
-    T.t = net->t;
-    T.y = net->y;
-    T.du = net->du;
+    T.scal = N.scal;
+    T.counter = N.counter;
+    T.partials = N.partials;
+    T.shat = N.shat;
+    T.ehat = N.ehat;
+    T.v = N.v;
+    T.y = N.y;
+    T.du = N.du;
     T.pidx = L->pidx;
     const int vg = net->vgrid;
-    sigma_kernel<float><<<vg, kVT, 0, s>>>(G.n, r, h->dinv, net->scal, net->counter, net->partials);
+    sigma_kernel<float><<<vg, kVT, 0, s>>>(G.n, r, h->dinv, N.scal, N.counter, N.partials);
     pair_input_kernel<<<vg, kVT, 0, s>>>(T);
-    launch_gates(L, net, s);
     ConvArgs A = conv_args(G);
     A.gate = L->gates;
     // forward, keeping the pre-gate fields
-    A.in = net->shat;
+    A.in = N.shat;
     A.w = net->d.k1in;
-    A.out = net->h1;
-    A.pre = net->a1;
+    A.out = N.h1;
+    A.pre = N.a1;
     conv1_kernel<E_GATE_PRE><<<G.tiles, kCT, conv1_smem(G), s>>>(A);
-    A.in = net->h1;
+    A.in = N.h1;
     A.w = net->d.k2;
-    A.out = net->h2;
+    A.out = N.h2;
     conv16_kernel<E_STORE><<<G.tiles, kCT, conv16_smem(G), s>>>(A);
-    A.in = net->h2;
+    A.in = N.h2;
     A.w = net->d.k2t;
-    A.out = net->k1;
-    A.pre = net->kpre;
+    A.out = N.k1;
+    A.pre = N.kpre;
     conv16_kernel<E_GATE_PRE><<<G.tiles, kCT, conv16_smem(G), s>>>(A);
-    A.in = net->k1;
+    A.in = N.k1;
     A.w = net->d.k1t;
-    A.u = net->u;
-    convout_kernel<E_OUT_U><<<convout_grid<E_OUT_U>(G), kCT, convout_smem(G), s>>>(A);
-    // loss: v = u - e_hat, w = A_hat v
-    loss_prep_kernel<<<vg, kVT, 0, s>>>(T);
-    spmv_store_kernel<<<h->sell_grid, kSellThreads, 0, s>>>(sell_of(h), net->t, net->y);
+    A.ehat = N.ehat;
+    A.dsq = L->dsq;
+    A.v = N.v;
+    A.t = N.t;
+    convout_kernel<E_OUT_LOSS><<<convout_grid<E_OUT_LOSS>(G), kCT, convout_smem(G), s>>>(A);
+    // loss: w = A_hat v
+    spmv_store_kernel<<<h->sell_grid, kSellThreads, 0, s>>>(sell_of(h), N.t, N.y);
     loss_kernel<<<vg, kVT, 0, s>>>(T);
     // backward
     WgArgs W{};
     W.G = G;
-    W.part = net->part;
+    W.part = N.part;
     W.bias_off = -1;
     // u = C1^T(k1): dk1 = C1(du); dk = g dk1, dg = k dk1; dW1 += wgrad(k1, du)
-    A.in = net->du;
+    A.in = N.du;
     A.w = net->d.k1in;
-    A.out = net->dk;
-    A.pre = net->kpre;
-    A.dg = net->dg;
+    A.out = N.dk;
+    A.pre = N.kpre;
+    A.dg = N.dg;
     A.dg_add = 0;
     conv1_kernel<E_BWD_GATE><<<G.tiles, kCT, conv1_smem(G), s>>>(A);
-    W.dy = net->k1;
-    W.x = net->du;
+    W.dy = N.k1;
+    W.x = N.du;
     W.off = kOffW1;
-    W.add = 0;
+    W.add = add;
     wgrad1_kernel<<<net->wg_ctas, kCT, wgrad1_smem(G), s>>>(W);
     // k = C2^T(h2): dh2 = C2(dk); dW2 += wgrad(h2, dk)
-    A.in = net->dk;
+    A.in = N.dk;
     A.w = net->d.k2;
-    A.out = net->dh2;
+    A.out = N.dh2;
     conv16_kernel<E_STORE><<<G.tiles, kCT, conv16_smem(G), s>>>(A);
-    W.dy = net->h2;
-    W.x = net->dk;
+    W.dy = N.h2;
+    W.x = N.dk;
     W.off = kOffW2;
-    W.add = 0;
+    W.add = add;
     wgrad16_kernel<<<net->wg_ctas, kCT, wgrad16_smem(G), s>>>(W);
     // h2 = C2(h1): dW2 += wgrad(dh2, h1); dh1 = C2^T(dh2); da1 = g dh1, dg += a1 dh1
-    W.dy = net->dh2;
-    W.x = net->h1;
+    W.dy = N.dh2;
+    W.x = N.h1;
     W.add = 1;
     wgrad16_kernel<<<net->wg_ctas, kCT, wgrad16_smem(G), s>>>(W);
-    A.in = net->dh2;
+    A.in = N.dh2;
     A.w = net->d.k2t;
-    A.out = net->da1;
-    A.pre = net->a1;
+    A.out = N.da1;
+    A.pre = N.a1;
     A.dg_add = 1;
+    A.dag = N.dag;   // dg is complete: dag = dg g (1 - g)
     conv16_kernel<E_BWD_GATE><<<G.tiles, kCT, conv16_smem(G), s>>>(A);
     // a1 = C1(s_hat): dW1 += wgrad(da1, s_hat)
-    W.dy = net->da1;
-    W.x = net->shat;
+    W.dy = N.da1;
+    W.x = N.shat;
     W.off = kOffW1;
     W.add = 1;
     wgrad1_kernel<<<net->wg_ctas, kCT, wgrad1_smem(G), s>>>(W);
-    // gates: dag = dg g (1 - g); dWg = wgrad(dag, lognu / 8), dbg = sum dag
-    const long long cnt = (long long)act_count(G, kCh);
-    gate_grad_kernel<<<4 * sm_count(net->device), kVT, 0, s>>>(cnt, net->dg, L->gates, net->dag);
-    W.dy = net->dag;
+    // gates: dWg = wgrad(dag, lognu / 8), dbg = sum dag
+    W.dy = N.dag;
     W.x = L->lognu_in;
     W.off = kOffWg;
     W.bias_off = kOffBg;
-    W.add = 0;
+    W.add = add;
     wgrad1_kernel<<<net->wg_ctas, kCT, wgrad1_smem(G), s>>>(W);
-    grad_reduce_kernel<<<(CG_LEARN_PARAMS + kVT - 1) / kVT, kVT, 0, s>>>(net->part, net->wg_ctas, net->d.grad);
+}
+
+// Losses and gradients of the pairs order[0 .. count): added to net->d.grad and
+// net->scal[2] on net->stream, pair k on lane k mod lanes.
+int enqueue_batch(cg_net *net, const cg_learn_set *set, const int64_t *order, int count) {
+    const Geo &G = set->inst[0]->learn->G;
+    const int lanes = (int)std::min<size_t>(net->lanes.size(), (size_t)count);
+    // the gates of every instance among the pairs, once
+    std::vector<const cg_handle *> seen;
+    for (int k = 0; k < count; ++k) {
+        const cg_handle *h = set->inst[set->pair_inst[order[k]]];
+        if (std::find(seen.begin(), seen.end(), h) != seen.end()) continue;
+        seen.push_back(h);
+        launch_gates(h->learn, net, net->stream);
+    }
+    if (!net->fork && cudaEventCreateWithFlags(&net->fork, cudaEventDisableTiming) != cudaSuccess) return CG_ECUDA;
+    if (cudaEventRecord(net->fork, net->stream) != cudaSuccess) return CG_ECUDA;
+    for (int l = 0; l < lanes; ++l)
+        if (cudaStreamWaitEvent(net->lanes[l].stream, net->fork, 0) != cudaSuccess) return CG_ECUDA;
+    for (int k = 0; k < count; ++k) {
+        const int64_t idx = order[k];
+        cg_handle *h = set->inst[set->pair_inst[idx]];
+        enqueue_sample(net, net->lanes[k % lanes], k < lanes, h, set->r + (size_t)idx * G.n, set->e + (size_t)idx * G.n);
+    }
+    GradParts P{};
+    P.lanes = lanes;
+    P.ctas = net->wg_ctas;
+    for (int l = 0; l < lanes; ++l) {
+        if (cudaEventRecord(net->lanes[l].done, net->lanes[l].stream) != cudaSuccess ||
+            cudaStreamWaitEvent(net->stream, net->lanes[l].done, 0) != cudaSuccess)
+            return CG_ECUDA;
+        P.part[l] = net->lanes[l].part;
+        P.scal[l] = net->lanes[l].scal;
+    }
+    grad_reduce_kernel<<<(CG_LEARN_PARAMS + 31) / 32, 32 * kRedGroups, 0, net->stream>>>(P, net->d.grad, net->scal + 2);
+    return cudaGetLastError() == cudaSuccess ? CG_OK : CG_ECUDA;
 }
 
 int check_set(const cg_net *net, const cg_learn_set *set) {
@@ -2303,7 +2451,10 @@ void cg_net_destroy(cg_net *net) {
     if (!net) return;
     DeviceGuard g(net->device);
     if (net->stream) cudaStreamSynchronize(net->stream);
-    for (void *p : net->tallocs) cudaFree(p);
+    for (auto &W : net->lanes)
+        if (W.stream) cudaStreamSynchronize(W.stream);
+    free_train(net);
+    if (net->fork) cudaEventDestroy(net->fork);
     if (net->block) cudaFree(net->block);
     if (net->stream) cudaStreamDestroy(net->stream);
     delete net;
@@ -2473,19 +2624,14 @@ int cg_learn_grad(cg_net *net, const cg_learn_set *set, const int64_t *pairs, in
     DeviceGuard dg(net->device);
     if ((rc = set_smem_limits()) != CG_OK) return rc;
     const Geo &G = set->inst[0]->learn->G;
-    if ((rc = ensure_train(net, G, max_ctas(set))) != CG_OK) return rc;
+    if ((rc = ensure_train(net, G, max_ctas(set), count)) != CG_OK) return rc;
     for (int i = 0; i < set->ninst; ++i)
         if (cudaStreamSynchronize(set->inst[i]->stream) != cudaSuccess) return CG_ECUDA;
     cudaStream_t s = net->stream;
     if (cudaMemsetAsync(net->d.grad, 0, sizeof(float) * CG_LEARN_PARAMS, s) != cudaSuccess ||
         cudaMemsetAsync(net->scal, 0, sizeof(double) * 8, s) != cudaSuccess)
         return CG_ECUDA;
-    for (int32_t k = 0; k < count; ++k) {
-        const int64_t idx = pairs[k];
-        cg_handle *h = set->inst[set->pair_inst[idx]];
-        enqueue_sample(net, h, set->r + (size_t)idx * G.n, set->e + (size_t)idx * G.n);
-    }
-    if (cudaGetLastError() != cudaSuccess) return CG_ECUDA;
+    if ((rc = enqueue_batch(net, set, pairs, count)) != CG_OK) return rc;
     std::vector<float> g(CG_LEARN_PARAMS);
     double sc[8];
     if (cudaMemcpyAsync(g.data(), net->d.grad, sizeof(float) * CG_LEARN_PARAMS, cudaMemcpyDeviceToHost, s) !=
@@ -2513,7 +2659,7 @@ int cg_learn_train(cg_net *net, const cg_learn_set *set, const int64_t *order, i
     DeviceGuard dg(net->device);
     if ((rc = set_smem_limits()) != CG_OK) return rc;
     const Geo &G = set->inst[0]->learn->G;
-    if ((rc = ensure_train(net, G, max_ctas(set))) != CG_OK) return rc;
+    if ((rc = ensure_train(net, G, max_ctas(set), batch)) != CG_OK) return rc;
     for (int i = 0; i < set->ninst; ++i)
         if (cudaStreamSynchronize(set->inst[i]->stream) != cudaSuccess) return CG_ECUDA;
     cudaStream_t s = net->stream;
@@ -2522,11 +2668,7 @@ int cg_learn_train(cg_net *net, const cg_learn_set *set, const int64_t *order, i
         return CG_ECUDA;
     std::vector<double> hist;
     for (int32_t k = 0; k < steps; ++k) {
-        for (int32_t j = 0; j < batch; ++j) {
-            const int64_t idx = order[(int64_t)k * batch + j];
-            cg_handle *h = set->inst[set->pair_inst[idx]];
-            enqueue_sample(net, h, set->r + (size_t)idx * G.n, set->e + (size_t)idx * G.n);
-        }
+        if ((rc = enqueue_batch(net, set, order + (int64_t)k * batch, batch)) != CG_OK) return rc;
         ++net->step;
         const float bc1 = 1.0f - std::pow(0.9f, (float)net->step);
         const float bc2 = 1.0f - std::pow(0.999f, (float)net->step);
