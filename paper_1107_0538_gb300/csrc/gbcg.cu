@@ -1257,7 +1257,7 @@ out:
 }
 
 // y = A x in the SELL-32 layout (stand-alone SpMV).
-__global__ void __launch_bounds__(kSellThreads) sell_spmv_kernel(SellMatrix M, const double *x, double *y) {
+__global__ void __launch_bounds__(kSellThreads, kSellBlocksPerSm) sell_spmv_kernel(SellMatrix M, const double *x, double *y) {
     EpiStore epi{y};
     sell_rows(M, x, epi);
 }

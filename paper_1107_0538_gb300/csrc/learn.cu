@@ -1364,7 +1364,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1) fcg_sell_kernel(FcgSellA
 }
 
 // Plain y = A x for training (no reductions).
-__global__ void __launch_bounds__(kSellThreads) spmv_store_kernel(SellMatrix M, const double *x, double *y) {
+__global__ void __launch_bounds__(kSellThreads, kSellBlocksPerSm) spmv_store_kernel(SellMatrix M, const double *x, double *y) {
     EpiStoreY e{y};
     sell_rows(M, x, e);
 }

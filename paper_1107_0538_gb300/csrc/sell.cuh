@@ -34,7 +34,13 @@ struct SellMatrix {
 };
 
 constexpr int kSellThreads = 256;
-constexpr int kSellBlocksPerSm = 8;
+// Four CTAs an SM, 64 registers a thread: with eight (32 registers) the loads
+// of a batch cannot be in flight together and a system of one or two slices per
+// warp waits for them one after the other.  Eight against four, us per call,
+// three matrices in turn: up to 32^3 10.25 / 6.16, 50^3 20.5 / 14.4, 57^3 20.5 /
+// 17.0, 72^3 28.7 / 26.5, 80^3 and 100^3 32.9 and 57.3 either way.  Batches of 14
+// and 27 with three, two or one CTAs were slower from 40^3 on (100^3 61 to 83).
+constexpr int kSellBlocksPerSm = 4;
 constexpr int kSellUnroll = 9;
 
 // Matrix loads: streaming (evict-first, read once per SpMV) when the matrix
