@@ -188,14 +188,43 @@ __device__ __forceinline__ void combine_segments(const BatchParams &B, int set, 
     }
 }
 
-// Total of one slot for one system: its segments in a fixed order (T = double
-// for the FP64 outer residual, float for the FP32 inner solve).
+// The lanes that share the reads of one pair's totals: a system's segments (one
+// per CTA that holds part of it) are read by L neighbouring lanes, L the power
+// of two that spreads the pairs over the CTA's threads, and joined by a
+// butterfly: with one thread per pair the reads of a system that spans many
+// CTAs would follow each other (one system on 152 CTAs: 105 us per inner
+// iteration, two thirds of it here).  Every CTA adds in the same order.
+__device__ __forceinline__ int pair_lanes(int npairs) {
+    int L = 32;
+    while (L > 1 && npairs * L > kThreads) L >>= 1;
+    return L;
+}
+
 template <class T>
-__device__ __forceinline__ T system_total(const BatchParams &B, int set, int sys, int slot) {
-    T s = T(0);
-    for (int k = B.sys_seg0[sys]; k < B.sys_seg0[sys + 1]; ++k)
-        s += (T)__ldcg(B.segpart + ((size_t)set * B.nseg + k) * kSlots + slot);
-    return s;
+__device__ __forceinline__ T lanes_sum(T v, int L) {
+    for (int m = 1; m < L; m <<= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+    return v;
+}
+
+// Totals of slots sl[0..NS) for one system under the static split (T = double
+// for the FP64 outer residual, float for the FP32 inner solve); sys < 0: none
+// (the lanes take part in the butterfly).  All lanes of the warp call it.
+template <class T, int NS>
+__device__ __forceinline__ void system_totals(const BatchParams &B, int set, int sys, int L, const int (&sl)[NS],
+                                              T (&out)[NS]) {
+#pragma unroll
+    for (int i = 0; i < NS; ++i) out[i] = T(0);
+    if (sys >= 0) {
+        const int k1 = B.sys_seg0[sys + 1];
+#pragma unroll 4
+        for (int k = B.sys_seg0[sys] + ((int)threadIdx.x & (L - 1)); k < k1; k += L) {
+            const double *src = B.segpart + ((size_t)set * B.nseg + k) * kSlots;
+#pragma unroll
+            for (int i = 0; i < NS; ++i) out[i] += (T)__ldcg(src + sl[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) out[i] = lanes_sum(out[i], L);
 }
 
 // Row functions that read their row's vector entries may define
@@ -419,24 +448,28 @@ __device__ __forceinline__ void combine_segments_dyn(const BatchParams &B, int s
     }
 }
 
-// Totals of slots sl[0..NS) for one system under the balanced layout: the
-// system's segments in the pieces it spans, in piece order (zero for a
-// system outside the layout).
+// The same under the balanced layout: the system's segments in the pieces it
+// spans (zero for a system outside the layout).
 template <int NS>
-__device__ __forceinline__ void system_totals_dyn(const BatchParams &B, int set, int total, int sys,
+__device__ __forceinline__ void system_totals_dyn(const BatchParams &B, int set, int total, int sys, int L,
                                                   const int (&sl)[NS], float (&out)[NS]) {
-    const int4 v = B.sinf[(size_t)blockIdx.x * B.nsys + sys];
-    const int G = (int)gridDim.x;
 #pragma unroll
     for (int i = 0; i < NS; ++i) out[i] = 0.0f;
-    for (int c = v.x; c <= v.y; ++c) {
-        // an empty piece (fewer active tiles than CTAs) holds nothing
-        if (v.w && c * total / G == (c + 1) * total / G) continue;
-        const int j = c == v.x ? bchk(v.z, kMaxSegPerCta) : 0;
-        const double *src = B.segdyn + (((size_t)set * G + c) * kMaxSegPerCta + j) * kSlots;
+    if (sys >= 0) {
+        const int4 v = B.sinf[(size_t)blockIdx.x * B.nsys + sys];
+        const int G = (int)gridDim.x;
+#pragma unroll 4
+        for (int c = v.x + ((int)threadIdx.x & (L - 1)); c <= v.y; c += L) {
+            // an empty piece (fewer active tiles than CTAs) holds nothing
+            const bool empty = v.w && (long long)c * total / G == (long long)(c + 1) * total / G;
+            const int j = c == v.x ? bchk(v.z, kMaxSegPerCta) : 0;
+            const double *src = B.segdyn + (((size_t)set * G + c) * kMaxSegPerCta + j) * kSlots;
 #pragma unroll
-        for (int i = 0; i < NS; ++i) out[i] += (float)__ldcg(src + sl[i]);
+            for (int i = 0; i < NS; ++i) out[i] += empty ? 0.0f : (float)__ldcg(src + sl[i]);
+        }
     }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) out[i] = lanes_sum(out[i], L);
 }
 
 template <class VT, class XT, class AT, class Cur, class RowFn, class Acc>
@@ -493,7 +526,6 @@ __device__ __forceinline__ bool batch_pass(const BatchParams &B, const Smem &S, 
             }
             __syncwarp();
             acc_switch(B, acc, cur.seg());
-            const int row = d.r0 + lane;
             if (d.kind == kTileLong) {
                 AT part{};
                 for (int k = d.a + lane; k < d.e; k += 32) part = fma_acc(vals[k], x[bchk(P.colidx[k], P.n)], part);
@@ -666,6 +698,9 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
     int set = 0;
     PairState *st = B.state + (size_t)blockIdx.x * B.nsys * kRhs;
     const int npairs = B.nsys * kRhs;
+    // the pairs' totals and decisions: L lanes per pair, the same pair count per
+    // warp step (every lane of a warp takes part in the butterflies)
+    const int L = pair_lanes(npairs), q0 = (int)threadIdx.x / L, qstep = kThreads / L;
     const VT *vlo;
     if constexpr (sizeof(VT) == 4) vlo = reinterpret_cast<const VT *>(P.vals32);
     else vlo = reinterpret_cast<const VT *>(P.vals16);
@@ -724,14 +759,17 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
         if (!grid_barrier(P, epoch, S)) goto out;
         {
             int inner_any = 0;
-            for (int q = threadIdx.x; q < npairs; q += kThreads) {
-                PairState ps = st[q];
+            for (int q = q0; q - q0 < npairs; q += qstep) {
+                const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
+                PairState ps{};
+                if (in) ps = st[q];
                 const int sys = q / kRhs, r = q % kRhs;
+                const int sl[3] = {r, 4 + r, 8 + r};
+                double tt[3];
+                system_totals<double>(B, set, ps.flags & kOuterActive ? sys : -1, L, sl, tt);
                 ps.flags &= ~kRanInner;
                 if (ps.flags & kOuterActive) {
-                    const double rr = system_total<double>(B, set, sys, r);
-                    const double bb = system_total<double>(B, set, sys, 4 + r);
-                    const double rz = system_total<double>(B, set, sys, 8 + r);
+                    const double rr = tt[0], bb = tt[1], rz = tt[2];
                     if (o == 0) ps.bnorm = sqrt(bb);
                     ps.relres = ps.bnorm > 0.0 ? sqrt(rr) / ps.bnorm : 0.0;
                     if (!finite_bits(rr) || !finite_bits(bb) || !finite_bits(rz)) {
@@ -760,7 +798,8 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         inner_any = 1;
                     }
                 }
-                st[q] = ps;
+                __syncwarp();
+                if (lead) st[q] = ps;
             }
             set ^= 1;
             if (__syncthreads_or(inner_any)) {
@@ -789,19 +828,17 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     else combine_segments(B, set, 4);
                     if (!grid_barrier(P, epoch, S)) goto out;
                     int left_now = 0;
-                    for (int q = threadIdx.x; q < npairs; q += kThreads) {
-                        PairState ps = st[q];
+                    for (int q = q0; q - q0 < npairs; q += qstep) {
+                        const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
+                        PairState ps{};
+                        if (in) ps = st[q];
+                        const int sl[1] = {q % kRhs}, sys = ps.flags & kInnerActive ? q / kRhs : -1;
+                        float o[1];
+                        if (dyn) system_totals_dyn<1>(B, set, bl.total, sys, L, sl, o);
+                        else system_totals<float>(B, set, sys, L, sl, o);
                         ps.alpha = 0.0f;
                         if (ps.flags & kInnerActive) {
-                            float sg;
-                            if (dyn) {
-                                const int sl[1] = {q % kRhs};
-                                float o[1];
-                                system_totals_dyn<1>(B, set, bl.total, q / kRhs, sl, o);
-                                sg = o[0];
-                            } else {
-                                sg = system_total<float>(B, set, q / kRhs, q % kRhs);
-                            }
+                            const float sg = o[0];
                             if (!(sg > 0.0f) || !isfinite(sg)) {
                                 ps.flags &= ~kInnerActive;  // keep d so far
                                 left_now = 1;
@@ -809,7 +846,8 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                                 ps.alpha = (float)ps.rho / sg;
                             }
                         }
-                        st[q] = ps;
+                        __syncwarp();
+                        if (lead) st[q] = ps;
                     }
                     __syncthreads();
                     set ^= 1;
@@ -833,22 +871,17 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     else combine_segments(B, set, 8);
                     if (!grid_barrier(P, epoch, S)) goto out;
                     int left = 0;
-                    for (int q = threadIdx.x; q < npairs; q += kThreads) {
-                        PairState ps = st[q];
+                    for (int q = q0; q - q0 < npairs; q += qstep) {
+                        const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
+                        PairState ps{};
+                        if (in) ps = st[q];
+                        const int r = q % kRhs, sl[2] = {r, 4 + r}, sys = ps.flags & kInnerActive ? q / kRhs : -1;
+                        float o[2];
+                        if (dyn) system_totals_dyn<2>(B, set, bl.total, sys, L, sl, o);
+                        else system_totals<float>(B, set, sys, L, sl, o);
                         ps.beta = 0.0f;
                         if (ps.flags & kInnerActive) {
-                            const int r = q % kRhs;
-                            float rr, rz;
-                            if (dyn) {
-                                const int sl[2] = {r, 4 + r};
-                                float o[2];
-                                system_totals_dyn<2>(B, set, bl.total, q / kRhs, sl, o);
-                                rr = o[0];
-                                rz = o[1];
-                            } else {
-                                rr = system_total<float>(B, set, q / kRhs, r);
-                                rz = system_total<float>(B, set, q / kRhs, 4 + r);
-                            }
+                            const float rr = o[0], rz = o[1];
                             ++ps.iters;
                             if (!isfinite(rr) || !isfinite(rz) || !(rz > 0.0f) || (double)rr <= ps.target2 ||
                                 k >= B.max_inner || ps.iters >= B.maxit) {
@@ -860,7 +893,8 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                                 left = 1;
                             }
                         }
-                        st[q] = ps;
+                        __syncwarp();
+                        if (lead) st[q] = ps;
                     }
                     set ^= 1;
                     if (!__syncthreads_or(left)) break;
