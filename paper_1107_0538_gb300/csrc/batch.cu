@@ -619,75 +619,173 @@ __device__ __forceinline__ void ring_entries(const BatchParams &B, const int *of
     }
 }
 
+// Up to 32 of a warp's tiles of the inner passes, one per lane: the descriptors
+// are read once and stay in registers until the layout changes (a system leaves
+// the inner loop) or the next 32 are due.  Read in the passes, each tile cost a
+// chain of three or four dependent L2 reads (prefix, tile, blob, rows): 6.6k
+// clocks a tile and warp in the SpMM pass.
+struct LaneTiles {
+    int r0, r1;      // rows [r0, r1)
+    int at, width;   // blob (16-byte units), offsets
+    int sys, seg;
+    unsigned int mask;   // lanes that hold a tile
+    int group = -1;      // which 32 of the warp's tiles; -1: none
+};
+
+__device__ __forceinline__ int lane_tile_groups(const BatchParams &B, const Balance &L, bool dyn) {
+    const int w = threadIdx.x >> 5;
+    const int m = dyn ? L.v1 - L.v0 : B.P.cta_tile[blockIdx.x + 1] - B.P.cta_tile[blockIdx.x];
+    return ((m - w + kWarps - 1) / kWarps + 31) / 32;
+}
+
+// Tiles w + kWarps (32 g + lane) of the CTA's piece (balanced) or of its share
+// of the plan's split, there without the systems `active` rejects.
+template <class Active>
+__device__ __forceinline__ void load_lane_tiles(const BatchParams &B, const Balance &L, bool dyn, const Active &active,
+                                                int g, LaneTiles &T) {
+    const int i = (threadIdx.x >> 5) + kWarps * (32 * g + (threadIdx.x & 31));
+    int t = -1;
+    T.r0 = T.r1 = T.at = T.width = T.sys = T.seg = 0;
+    if (dyn) {
+        const int v = L.v0 + i;
+        if (v < L.v1) {
+            const int32_t *pfx = bal_pfx(B), *rk = pfx + B.nsys + 1;
+            int a = L.s0, b = B.nsys;   // the system with pfx[a] <= v < pfx[a + 1]
+            while (b - a > 1) {
+                const int c = (a + b) >> 1;
+                if (pfx[c] <= v) a = c;
+                else b = c;
+            }
+            t = B.sys_tile0[bchk(a, B.nsys)] + (v - pfx[a]);
+            T.sys = a;
+            T.seg = rk[a] - L.k0;
+        }
+    } else {
+        const int u = B.P.cta_tile[blockIdx.x] + i;
+        if (u < B.P.cta_tile[blockIdx.x + 1]) {
+            const int sys = B.tile_sys[u];
+            if (active(sys)) {
+                t = u;
+                T.sys = sys;
+                T.seg = sys - B.cta_sys0[blockIdx.x];
+            }
+        }
+    }
+    if (t >= 0) {
+        const int4 d = __ldg(B.P.tiles + 2 * t);
+        const int2 me = __ldg(B.ring_meta + t);
+        T.r0 = d.x;
+        T.r1 = d.y;
+        T.at = me.x;
+        T.width = me.y;
+    }
+    T.mask = __ballot_sync(0xffffffffu, t >= 0);
+    T.group = g;
+}
+
 // `count`: copies of this warp since the kernel began; copy c goes to buffer
 // c mod ring_bufs and completes phase c / ring_bufs of its mbarrier.  Every
 // copy started in a pass is waited for in it.
-template <class VT, class Cur, class RowFn, class Acc>
+template <class VT, class Active, class RowFn, class Acc>
 __device__ __forceinline__ bool batch_pass_ring(const BatchParams &B, const Smem &S, uint64_t *rbar, uint32_t &count,
-                                                Cur cur, RowFn &rowfn, Acc &acc) {
+                                                const Balance &L, bool dyn, const Active &active, LaneTiles &T,
+                                                RowFn &rowfn, Acc &acc) {
     const Params &P = B.P;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = B.ring_bufs;
     unsigned char *const stage = S.base(w);
     uint64_t *const bar = rbar + w * kRingBufs;
-    bool ok = true;
-    cur.start(w);
-    Cur ahead = cur;
-    uint32_t issued = count;
-    auto issue = [&]() {   // the tile of `ahead` into the next buffer
-        const int2 me = __ldg(B.ring_meta + ahead.tile());
-        const int b = (int)(issued % (uint32_t)nb);
-        // this warp's reads of the buffer before the async-proxy copy into it
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
-        if (lane == 0) {
-            const uint32_t bytes = (uint32_t)batch_ring_bytes(me.y, (int)sizeof(VT));
-            if (bytes == 0) {
-                mbar_arrive(&bar[b]);
-            } else {
-                mbar_arrive_expect_tx(&bar[b], bytes);
-                tma_load_1d(stage + b * B.ring_slot, B.ring_blob + (size_t)me.x * 16, bytes, &bar[b], P.evict_first != 0);
+    const int groups = lane_tile_groups(B, L, dyn);
+    for (int g = 0; g < groups; ++g) {
+        if (T.group != g) load_lane_tiles(B, L, dyn, active, g, T);
+        unsigned int ahead = T.mask;
+        uint32_t issued = count;
+        auto issue = [&]() {   // the next tile of `ahead` into the next buffer
+            const int from = __ffs(ahead) - 1, b = (int)(issued % (uint32_t)nb);
+            ahead &= ahead - 1;
+            // this warp's reads of the buffer before the async-proxy copy into it
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == from) {
+                const uint32_t bytes = (uint32_t)batch_ring_bytes(T.width, (int)sizeof(VT));
+                if (bytes == 0) {
+                    mbar_arrive(&bar[b]);
+                } else {
+                    mbar_arrive_expect_tx(&bar[b], bytes);
+                    tma_load_1d(stage + b * B.ring_slot, B.ring_blob + (size_t)T.at * 16, bytes, &bar[b],
+                                P.evict_first != 0);
+                }
             }
+            __syncwarp();
+            ++issued;
+        };
+        for (int i = 0; i < nb && ahead; ++i) issue();
+        for (unsigned int left = T.mask; left; left &= left - 1) {
+            const int from = __ffs(left) - 1;
+            const int row = __shfl_sync(0xffffffffu, T.r0, from) + lane, end = __shfl_sync(0xffffffffu, T.r1, from);
+            const int sys = __shfl_sync(0xffffffffu, T.sys, from);
+            int k = __shfl_sync(0xffffffffu, T.width, from);
+            if (row < end) batch_prefetch(rowfn, row, 0);
+            const int b = (int)(count % (uint32_t)nb);
+            const bool got = mbar_wait_bounded(&bar[b], (count / (uint32_t)nb) & 1u, P.wait_ns);
+            if (__any_sync(0xffffffffu, !got)) {
+                // the copies still in flight, each with the same limit
+                for (uint32_t c = count + 1; c != issued; ++c)
+                    mbar_wait_bounded(&bar[c % (uint32_t)nb], (c / (uint32_t)nb) & 1u, P.wait_ns);
+                return false;
+            }
+            acc_switch(B, acc, __shfl_sync(0xffffffffu, T.seg, from));
+            const int *offs = reinterpret_cast<const int *>(stage + b * B.ring_slot);
+            const VT *vals = reinterpret_cast<const VT *>(stage + b * B.ring_slot + batch_ring_head(k)) + lane;
+            float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (; k >= 8; k -= 8, offs += 8, vals += 256) ring_entries<8>(B, offs, vals, row, sum);
+            if (k >= 4) {
+                ring_entries<4>(B, offs, vals, row, sum);
+                k -= 4, offs += 4, vals += 128;
+            }
+            if (k == 3) ring_entries<3>(B, offs, vals, row, sum);
+            else if (k == 2) ring_entries<2>(B, offs, vals, row, sum);
+            else if (k == 1) ring_entries<1>(B, offs, vals, row, sum);
+            ++count;
+            if (ahead) issue();
+            if (row < end) rowfn(sys, row, sum, acc);
         }
-        __syncwarp();
-        ++issued;
-        ahead.next();
-    };
-    for (int i = 0; i < nb && ahead.valid(); ++i) issue();
-    for (; cur.valid(); cur.next()) {
-        const int t = cur.tile();
-        const int4 d0 = __ldg(P.tiles + 2 * t);   // rows [x, y)
-        const int2 me = __ldg(B.ring_meta + t);
-        const int row = d0.x + lane;
-        if (row < d0.y) batch_prefetch(rowfn, row, 0);
-        const int b = (int)(count % (uint32_t)nb);
-        const bool got = mbar_wait_bounded(&bar[b], (count / (uint32_t)nb) & 1u, P.wait_ns);
-        if (__any_sync(0xffffffffu, !got)) {
-            ok = false;
-            break;
-        }
-        acc_switch(B, acc, cur.seg());
-        int k = me.y;
-        const int *offs = reinterpret_cast<const int *>(stage + b * B.ring_slot);
-        const VT *vals = reinterpret_cast<const VT *>(stage + b * B.ring_slot + batch_ring_head(k)) + lane;
-        float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (; k >= 8; k -= 8, offs += 8, vals += 256) ring_entries<8>(B, offs, vals, row, sum);
-        if (k >= 4) {
-            ring_entries<4>(B, offs, vals, row, sum);
-            k -= 4, offs += 4, vals += 128;
-        }
-        if (k == 3) ring_entries<3>(B, offs, vals, row, sum);
-        else if (k == 2) ring_entries<2>(B, offs, vals, row, sum);
-        else if (k == 1) ring_entries<1>(B, offs, vals, row, sum);
-        ++count;
-        if (ahead.valid()) issue();
-        if (row < d0.y) rowfn(cur.sys(), row, sum, acc);
     }
-    if (!ok)   // the copies still in flight, each with the same limit
-        for (uint32_t c = count + 1; c != issued; ++c)
-            mbar_wait_bounded(&bar[c % (uint32_t)nb], (c / (uint32_t)nb) & 1u, P.wait_ns);
     if (acc.seg >= 0) flush_acc(B, acc);
     acc.seg = -1;
-    return ok;
+    return true;
+}
+
+// The pass without the matrix over the same tiles; the next tile's rows load
+// before the current one's are done.
+template <class Active, class RowFn, class Acc>
+__device__ __forceinline__ void batch_pass_rows(const BatchParams &B, const Balance &L, bool dyn, const Active &active,
+                                                LaneTiles &T, RowFn &rowfn, Acc &acc) {
+    const int lane = threadIdx.x & 31, groups = lane_tile_groups(B, L, dyn);
+    const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int g = 0; g < groups; ++g) {
+        if (T.group != g) load_lane_tiles(B, L, dyn, active, g, T);
+        int from = __ffs(T.mask) - 1;
+        int row = 0, end = 0;
+        if (T.mask) {
+            row = __shfl_sync(0xffffffffu, T.r0, from) + lane;
+            end = __shfl_sync(0xffffffffu, T.r1, from);
+            if (row < end) batch_prefetch(rowfn, row, 0);
+        }
+        for (unsigned int left = T.mask; left;) {
+            const int at = row, stop = end, sys = __shfl_sync(0xffffffffu, T.sys, from);
+            acc_switch(B, acc, __shfl_sync(0xffffffffu, T.seg, from));
+            left &= left - 1;
+            if (left) {
+                from = __ffs(left) - 1;
+                row = __shfl_sync(0xffffffffu, T.r0, from) + lane;
+                end = __shfl_sync(0xffffffffu, T.r1, from);
+                if (row < end) batch_prefetch(rowfn, row, 0);
+            }
+            if (at < stop) rowfn(sys, at, none, acc);
+        }
+    }
+    if (acc.seg >= 0) flush_acc(B, acc);
+    acc.seg = -1;
 }
 
 // The offsets of a tile's rows (lane k: the k-th smallest) and their number;
@@ -868,6 +966,8 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
     if (threadIdx.x < kWarps * kRingBufs) mbar_init(&rbar[threadIdx.x], 1);
     init_pipeline(S);   // with the barriers' fence and a __syncthreads
     uint32_t rcount = 0;
+    // the inner passes then read no vector with TMA: their barriers need no fence
+    const bool ring = B.ring_blob != nullptr;
     // the block-sum area is free in this kernel: it holds the layout arrays
     int *const bsm = reinterpret_cast<int *>(S.red);
     Balance &bl = *reinterpret_cast<Balance *>(bsm + kBalHdr);
@@ -987,6 +1087,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                 if (B.balance) compute_balance(B, active, bsm);
                 else if (threadIdx.x == 0) bl.dyn = 0;
                 __syncthreads();
+                LaneTiles T;
                 for (int k = 1;; ++k) {
                     const bool dyn = bl.dyn != 0;
                     const int nloc = dyn ? bl.nloc : B.cta_nsys[blockIdx.x];
@@ -998,9 +1099,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         acc.seg = -1;
                         SpmmRow rowfn{B, st};
                         const bool ok =
-                            B.ring_blob
-                                ? (dyn ? batch_pass_ring<VT>(B, S, rbar, rcount, balanced_tiles(B, bl), rowfn, acc)
-                                       : batch_pass_ring<VT>(B, S, rbar, rcount, static_tiles(B, active), rowfn, acc))
+                            ring  ? batch_pass_ring<VT>(B, S, rbar, rcount, bl, dyn, active, T, rowfn, acc)
                             : dyn ? batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, balanced_tiles(B, bl), rowfn, acc)
                                 : batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, static_tiles(B, active), rowfn,
                                                                  acc);
@@ -1008,7 +1107,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     }
                     if (dyn) combine_segments_dyn(B, set, 4, nloc);
                     else combine_segments(B, set, 4);
-                    if (!grid_barrier(P, epoch, S)) goto out;
+                    if (!(ring ? grid_barrier<false>(P, epoch, S) : grid_barrier(P, epoch, S))) goto out;
                     int left_now = 0;
                     for (int q = q0; q - q0 < npairs; q += qstep) {
                         const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
@@ -1040,18 +1139,20 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         WarpAcc<float, 8> acc;
                         acc.seg = -1;
                         UpdateRow rowfn{B, st};
-                        const bool ok =
-                            dyn ? batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
-                                                                 (const float4 *)nullptr, balanced_tiles(B, bl), rowfn,
-                                                                 acc)
-                                : batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
+                        bool ok = true;
+                        if (ring) batch_pass_rows(B, bl, dyn, active, T, rowfn, acc);
+                        else
+                            ok = dyn ? batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
+                                                                      (const float4 *)nullptr, balanced_tiles(B, bl),
+                                                                      rowfn, acc)
+                                     : batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
                                                                  (const float4 *)nullptr, static_tiles(B, active), rowfn,
                                                                  acc);
                         if (!ok) goto out;
                     }
                     if (dyn) combine_segments_dyn(B, set, 8, nloc);
                     else combine_segments(B, set, 8);
-                    if (!grid_barrier(P, epoch, S)) goto out;
+                    if (!(ring ? grid_barrier<false>(P, epoch, S) : grid_barrier(P, epoch, S))) goto out;
                     int left = 0;
                     for (int q = q0; q - q0 < npairs; q += qstep) {
                         const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
@@ -1080,8 +1181,21 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     }
                     set ^= 1;
                     if (!__syncthreads_or(left)) break;
-                    // a pair left the inner loop: its system may have, so re-split
-                    if (B.balance && __syncthreads_or(left_now)) compute_balance(B, active, bsm);
+                    // a pair left the inner loop: where its system did, re-split
+                    if (__syncthreads_or(left_now)) {
+                        if (B.balance) {
+                            const int32_t *rk = bal_pfx(B) + B.nsys + 1;
+                            int changed = 0;
+                            for (int s = threadIdx.x; s < B.nsys; s += kThreads)
+                                changed |= (rk[s + 1] != rk[s]) != active(s);
+                            if (__syncthreads_or(changed)) {
+                                compute_balance(B, active, bsm);
+                                T.group = -1;
+                            }
+                        } else {
+                            T.group = -1;
+                        }
+                    }
                 }
             }
         }
