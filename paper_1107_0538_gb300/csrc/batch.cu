@@ -137,20 +137,28 @@ __device__ __forceinline__ float4 warp_sum_acc(float4 v) {
 // rowfn(tile, row, seg, 0) is called per row.  Each lane keeps kSlots
 // accumulators per segment (acc), flushed to wpart when the warp moves to
 // another segment and at the end.
+struct WarpRows {   // one row per warp, `segs` segments of kSlots sums each
+    double *base;
+    int segs;
+    __device__ __forceinline__ double *row(int w) const { return base + (size_t)w * segs * kSlots; }
+};
+
 template <class T, int NS>
 struct WarpAcc {
     T a[NS > 0 ? NS : 1];
-    int seg;
+    int seg = -1;
+    double *row;   // this warp's row of partial sums, kSlots per segment
+    __device__ __forceinline__ explicit WarpAcc(const WarpRows &R) : row(R.row(threadIdx.x >> 5)) {}
 };
 
 // Warp-sums the lanes' accumulators of the current segment (in T: FP32 for
 // the inner passes, FP64 for the outer residual) and adds them to the warp's
 // own row of wpart (zeroed at the start of each reduction).
 template <class T, int NS>
-__device__ __forceinline__ void flush_acc(const BatchParams &B, WarpAcc<T, NS> &acc) {
+__device__ __forceinline__ void flush_acc(WarpAcc<T, NS> &acc) {
     if (NS == 0) return;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *dst = B.wpart + (((size_t)blockIdx.x * kWarps + w) * kMaxSegPerCta + acc.seg) * kSlots;
+    const int lane = threadIdx.x & 31;
+    double *dst = acc.row + (size_t)acc.seg * kSlots;
 #pragma unroll
     for (int i = 0; i < NS; ++i) {
         T v = acc.a[i];
@@ -161,9 +169,9 @@ __device__ __forceinline__ void flush_acc(const BatchParams &B, WarpAcc<T, NS> &
 }
 
 template <class T, int NS>
-__device__ __forceinline__ void acc_switch(const BatchParams &B, WarpAcc<T, NS> &acc, int seg) {
+__device__ __forceinline__ void acc_switch(WarpAcc<T, NS> &acc, int seg) {
     if (seg != acc.seg) {
-        if (acc.seg >= 0) flush_acc(B, acc);
+        if (acc.seg >= 0) flush_acc(acc);
         acc.seg = seg;
 #pragma unroll
         for (int i = 0; i < (NS > 0 ? NS : 1); ++i) acc.a[i] = T(0);
@@ -171,23 +179,23 @@ __device__ __forceinline__ void acc_switch(const BatchParams &B, WarpAcc<T, NS> 
 }
 
 // Zeroes this warp's rows of wpart for ns segments.
-__device__ __forceinline__ void zero_wpart(const BatchParams &B, int ns) {
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double *row = B.wpart + ((size_t)blockIdx.x * kWarps + w) * kMaxSegPerCta * kSlots;
+__device__ __forceinline__ void zero_wpart(const WarpRows &R, int ns) {
+    const int lane = threadIdx.x & 31;
+    double *row = R.row(threadIdx.x >> 5);
     for (int i = lane; i < ns * kSlots; i += 32) row[i] = 0.0;
     __syncwarp();
 }
 
 // Adds the 16 warp rows of each of this CTA's segments (fixed order) into
 // segpart[set], for the first nslots slots.
-__device__ __forceinline__ void combine_segments(const BatchParams &B, int set, int nslots) {
+__device__ __forceinline__ void combine_segments(const BatchParams &B, const WarpRows &R, int set, int nslots) {
     __syncthreads();
     const int ns = B.cta_nsys[blockIdx.x], seg0 = B.cta_seg0[blockIdx.x];
-    const double *wp = B.wpart + (size_t)blockIdx.x * kWarps * kMaxSegPerCta * kSlots;
     for (int q = threadIdx.x; q < ns * nslots; q += kThreads) {
         const int j = q / nslots, i = q % nslots;
         double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += wp[((size_t)w * kMaxSegPerCta + j) * kSlots + i];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) s += R.row(w)[(size_t)j * kSlots + i];
         B.segpart[((size_t)set * B.nseg + seg0 + j) * kSlots + i] = s;
     }
 }
@@ -300,9 +308,10 @@ __device__ __forceinline__ StaticTiles<Active> static_tiles(const BatchParams &B
 
 // This CTA's prefixes: pfx[s] active tiles and rk[s] active systems before
 // system s (nsys + 1 entries each).
-__device__ __forceinline__ int32_t *bal_pfx(const BatchParams &B) {
-    return B.bal + (size_t)blockIdx.x * 2 * (B.nsys + 1);
-}
+struct BalArrays {
+    int32_t *pfx;
+    int4 *sinf;
+};
 
 // Tiles v0 + w, v0 + w + kWarps, ... < v1 of the active-tile numbering.
 struct BalancedTiles {
@@ -326,8 +335,8 @@ struct BalancedTiles {
         settle();
     }
 };
-__device__ __forceinline__ BalancedTiles balanced_tiles(const BatchParams &B, const Balance &L) {
-    const int32_t *pfx = bal_pfx(B);
+__device__ __forceinline__ BalancedTiles balanced_tiles(const BatchParams &B, const BalArrays &A, const Balance &L) {
+    const int32_t *pfx = A.pfx;
     return BalancedTiles{&B, pfx, pfx + B.nsys + 1, L.v0, L.v1, L.s0, L.k0};
 }
 
@@ -342,11 +351,11 @@ __device__ __forceinline__ int piece_of(int v, int T, int G) {
 // all take the same decision (dyn) and the same layout.  All threads call it;
 // it ends with a __syncthreads.
 template <class Active>
-__device__ void compute_balance(const BatchParams &B, const Active &active, int *bsm) {
+__device__ void compute_balance(const BatchParams &B, const BalArrays &A, const Active &active, int *bsm) {
     Balance &L = *reinterpret_cast<Balance *>(bsm + kBalHdr);
     int *scan = bsm, *k0c = bsm + kBalArr, *k1c = k0c + kMaxBalCtas, *s0c = k1c + kMaxBalCtas;
     const int ns = B.nsys, G = (int)gridDim.x;
-    int32_t *pfx = bal_pfx(B), *rk = pfx + ns + 1;
+    int32_t *pfx = A.pfx, *rk = pfx + ns + 1;
     const int per = (ns + kThreads - 1) / kThreads;
     const int a = min((int)threadIdx.x * per, ns), b = min(a + per, ns);
     int tiles = 0, cnt = 0;
@@ -405,7 +414,7 @@ __device__ void compute_balance(const BatchParams &B, const Active &active, int 
     __syncthreads();
     // each system's pieces: c0 .. c1, its segment j0 in piece c0 (0 in the
     // later ones, which start inside it); with T < G some pieces are empty
-    int4 *sinf = B.sinf + (size_t)blockIdx.x * ns;
+    int4 *sinf = A.sinf;
     for (int s = a; s < b; ++s) {
         const int t0 = pfx[s], t1 = pfx[s + 1];
         int4 v = make_int4(0, -1, 0, 0);
@@ -440,14 +449,15 @@ __device__ void compute_balance(const BatchParams &B, const Active &active, int 
 
 // Adds the 16 warp rows of each of this piece's nloc segments (fixed order)
 // into segdyn[set][c], for the first nslots slots.
-__device__ __forceinline__ void combine_segments_dyn(const BatchParams &B, int set, int nslots, int nloc) {
+__device__ __forceinline__ void combine_segments_dyn(const BatchParams &B, const WarpRows &R, int set, int nslots,
+                                                     int nloc) {
     __syncthreads();
-    const double *wp = B.wpart + (size_t)blockIdx.x * kWarps * kMaxSegPerCta * kSlots;
     double *dst = B.segdyn + ((size_t)set * gridDim.x + blockIdx.x) * kMaxSegPerCta * kSlots;
     for (int q = threadIdx.x; q < nloc * nslots; q += kThreads) {
         const int j = q / nslots, i = q % nslots;
         double s = 0.0;
-        for (int w = 0; w < kWarps; ++w) s += wp[((size_t)w * kMaxSegPerCta + j) * kSlots + i];
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) s += R.row(w)[(size_t)j * kSlots + i];
         dst[(size_t)j * kSlots + i] = s;
     }
 }
@@ -455,12 +465,13 @@ __device__ __forceinline__ void combine_segments_dyn(const BatchParams &B, int s
 // The same under the balanced layout: the system's segments in the pieces it
 // spans (zero for a system outside the layout).
 template <int NS>
-__device__ __forceinline__ void system_totals_dyn(const BatchParams &B, int set, int total, int sys, int L,
+__device__ __forceinline__ void system_totals_dyn(const BatchParams &B, const BalArrays &A, int set, int total, int sys,
+                                                  int L,
                                                   const int (&sl)[NS], float (&out)[NS]) {
 #pragma unroll
     for (int i = 0; i < NS; ++i) out[i] = 0.0f;
     if (sys >= 0) {
-        const int4 v = B.sinf[(size_t)blockIdx.x * B.nsys + sys];
+        const int4 v = A.sinf[sys];
         const int G = (int)gridDim.x;
 #pragma unroll 4
         for (int c = v.x + ((int)threadIdx.x & (L - 1)); c <= v.y; c += L) {
@@ -500,7 +511,7 @@ __device__ __forceinline__ bool batch_pass(const BatchParams &B, const Smem &S, 
                 dn = load_desc(P, nx.tile());
                 if (dn.r0 + lane < dn.r1) batch_prefetch(rowfn, dn.r0 + lane, 0);
             }
-            acc_switch(B, acc, cur.seg());
+            acc_switch(acc, cur.seg());
             const int row = d.r0 + lane;
             if (row < d.r1) rowfn(cur.sys(), row, AT{}, acc);
             d = dn;
@@ -529,7 +540,7 @@ __device__ __forceinline__ bool batch_pass(const BatchParams &B, const Smem &S, 
                 break;
             }
             __syncwarp();
-            acc_switch(B, acc, cur.seg());
+            acc_switch(acc, cur.seg());
             if (d.kind == kTileLong) {
                 AT part{};
                 for (int k = d.a + lane; k < d.e; k += 32) part = fma_acc(vals[k], x[bchk(P.colidx[k], P.n)], part);
@@ -579,7 +590,7 @@ __device__ __forceinline__ bool batch_pass(const BatchParams &B, const Smem &S, 
             cur = nx;
         }
     }
-    if (acc.seg >= 0) flush_acc(B, acc);
+    if (acc.seg >= 0) flush_acc(acc);
     acc.seg = -1;
     return ok;
 }
@@ -592,10 +603,10 @@ __device__ __forceinline__ bool batch_pass(const BatchParams &B, const Smem &S, 
 // 2.1 bytes per entry instead of 6 or 4, no staged window, and small enough for
 // several tiles per warp in the warp's stage.  The staged tiles take the whole
 // stage, so each waits out its own load (7 tiles per warp and pass at 484k
-// rows); here a warp has up to kRingBufs tiles loading ahead, and gathers the
+// rows); here a warp has kRingBufs tiles loading ahead, and gathers the
 // float4 vectors through L1 with 8 entries in flight.  Inner iteration of 16
 // Q1 systems (484k rows, 27 entries a row, FP32): 56.6 us staged, 49.6 so.
-constexpr int kRingBufs = 4;
+constexpr int kRingBufs = 2;
 constexpr int kRingMaxOffs = 32;
 
 __host__ __device__ constexpr int batch_ring_head(int w) { return 16 * ((w + 3) / 4); }
@@ -641,15 +652,15 @@ __device__ __forceinline__ int lane_tile_groups(const BatchParams &B, const Bala
 // Tiles w + kWarps (32 g + lane) of the CTA's piece (balanced) or of its share
 // of the plan's split, there without the systems `active` rejects.
 template <class Active>
-__device__ __forceinline__ void load_lane_tiles(const BatchParams &B, const Balance &L, bool dyn, const Active &active,
-                                                int g, LaneTiles &T) {
+__device__ __forceinline__ void load_lane_tiles(const BatchParams &B, const BalArrays &A, const Balance &L, bool dyn,
+                                                const Active &active, int g, LaneTiles &T) {
     const int i = (threadIdx.x >> 5) + kWarps * (32 * g + (threadIdx.x & 31));
     int t = -1;
     T.r0 = T.r1 = T.at = T.width = T.sys = T.seg = 0;
     if (dyn) {
         const int v = L.v0 + i;
         if (v < L.v1) {
-            const int32_t *pfx = bal_pfx(B), *rk = pfx + B.nsys + 1;
+            const int32_t *pfx = A.pfx, *rk = pfx + B.nsys + 1;
             int a = L.s0, b = B.nsys;   // the system with pfx[a] <= v < pfx[a + 1]
             while (b - a > 1) {
                 const int c = (a + b) >> 1;
@@ -688,15 +699,15 @@ __device__ __forceinline__ void load_lane_tiles(const BatchParams &B, const Bala
 // copy started in a pass is waited for in it.
 template <class VT, class Active, class RowFn, class Acc>
 __device__ __forceinline__ bool batch_pass_ring(const BatchParams &B, const Smem &S, uint64_t *rbar, uint32_t &count,
-                                                const Balance &L, bool dyn, const Active &active, LaneTiles &T,
+                                                const BalArrays &A, const Balance &L, bool dyn, const Active &active, LaneTiles &T,
                                                 RowFn &rowfn, Acc &acc) {
     const Params &P = B.P;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nb = B.ring_bufs;
-    unsigned char *const stage = S.base(w);
+    unsigned char *const stage = S.stage + w * nb * B.ring_slot;
     uint64_t *const bar = rbar + w * kRingBufs;
     const int groups = lane_tile_groups(B, L, dyn);
     for (int g = 0; g < groups; ++g) {
-        if (T.group != g) load_lane_tiles(B, L, dyn, active, g, T);
+        if (T.group != g) load_lane_tiles(B, A, L, dyn, active, g, T);
         unsigned int ahead = T.mask;
         uint32_t issued = count;
         auto issue = [&]() {   // the next tile of `ahead` into the next buffer
@@ -733,7 +744,7 @@ __device__ __forceinline__ bool batch_pass_ring(const BatchParams &B, const Smem
                     mbar_wait_bounded(&bar[c % (uint32_t)nb], (c / (uint32_t)nb) & 1u, P.wait_ns);
                 return false;
             }
-            acc_switch(B, acc, __shfl_sync(0xffffffffu, T.seg, from));
+            acc_switch(acc, __shfl_sync(0xffffffffu, T.seg, from));
             const int *offs = reinterpret_cast<const int *>(stage + b * B.ring_slot);
             const VT *vals = reinterpret_cast<const VT *>(stage + b * B.ring_slot + batch_ring_head(k)) + lane;
             float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -750,7 +761,7 @@ __device__ __forceinline__ bool batch_pass_ring(const BatchParams &B, const Smem
             if (row < end) rowfn(sys, row, sum, acc);
         }
     }
-    if (acc.seg >= 0) flush_acc(B, acc);
+    if (acc.seg >= 0) flush_acc(acc);
     acc.seg = -1;
     return true;
 }
@@ -758,12 +769,12 @@ __device__ __forceinline__ bool batch_pass_ring(const BatchParams &B, const Smem
 // The pass without the matrix over the same tiles; the next tile's rows load
 // before the current one's are done.
 template <class Active, class RowFn, class Acc>
-__device__ __forceinline__ void batch_pass_rows(const BatchParams &B, const Balance &L, bool dyn, const Active &active,
-                                                LaneTiles &T, RowFn &rowfn, Acc &acc) {
+__device__ __forceinline__ void batch_pass_rows(const BatchParams &B, const BalArrays &A, const Balance &L, bool dyn,
+                                                const Active &active, LaneTiles &T, RowFn &rowfn, Acc &acc) {
     const int lane = threadIdx.x & 31, groups = lane_tile_groups(B, L, dyn);
     const float4 none = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (int g = 0; g < groups; ++g) {
-        if (T.group != g) load_lane_tiles(B, L, dyn, active, g, T);
+        if (T.group != g) load_lane_tiles(B, A, L, dyn, active, g, T);
         int from = __ffs(T.mask) - 1;
         int row = 0, end = 0;
         if (T.mask) {
@@ -773,7 +784,7 @@ __device__ __forceinline__ void batch_pass_rows(const BatchParams &B, const Bala
         }
         for (unsigned int left = T.mask; left;) {
             const int at = row, stop = end, sys = __shfl_sync(0xffffffffu, T.sys, from);
-            acc_switch(B, acc, __shfl_sync(0xffffffffu, T.seg, from));
+            acc_switch(acc, __shfl_sync(0xffffffffu, T.seg, from));
             left &= left - 1;
             if (left) {
                 from = __ffs(left) - 1;
@@ -784,7 +795,7 @@ __device__ __forceinline__ void batch_pass_rows(const BatchParams &B, const Bala
             if (at < stop) rowfn(sys, at, none, acc);
         }
     }
-    if (acc.seg >= 0) flush_acc(B, acc);
+    if (acc.seg >= 0) flush_acc(acc);
     acc.seg = -1;
 }
 
@@ -957,17 +968,85 @@ struct UpdateRow {
     }
 };
 
+// b - A x of the outer step with tiles of common offsets: one lane per row, all
+// right-hand sides in one pass over the matrix (FP64, from global memory: six
+// or seven of these passes per solve), rowfn(sys, row, r, (A x)_r) for each.
+template <class Active, class RowFn, class Acc>
+__device__ __forceinline__ void batch_pass_outer(const BatchParams &B, const Active &active, RowFn &rowfn, Acc &acc) {
+    const Params &P = B.P;
+    const int lane = threadIdx.x & 31;
+    auto cur = static_tiles(B, active);
+    for (cur.start(threadIdx.x >> 5); cur.valid(); cur.next()) {
+        const int4 d = __ldg(P.tiles + 2 * cur.tile());
+        const int row = d.x + lane;
+        acc_switch(acc, cur.seg());
+        if (row >= d.y) continue;
+        double ax[kRhs] = {0.0, 0.0, 0.0, 0.0};
+        const int k1 = P.rowptr[row + 1];
+#pragma unroll 4
+        for (int k = P.rowptr[row]; k < k1; ++k) {
+            const double a = P.vals[k];
+            const int c = bchk(P.colidx[k], P.n);
+#pragma unroll
+            for (int r = 0; r < kRhs; ++r) ax[r] = fma(a, B.xw[(size_t)r * B.xstride + c], ax[r]);
+        }
+        rowfn(cur.sys(), row, ax, acc);
+    }
+    if (acc.seg >= 0) flush_acc(acc);
+    acc.seg = -1;
+}
+
+// Shared memory of the kernel over tiles with common offsets: the tile buffers,
+// the area of Smem::red, bcast and ctl, and, as far as they fit, what every
+// reduction reads and writes again: the pair states, the layout arrays and the
+// warps' partial sums of up to kSmemSegs segments.  Tile buffers of two tiles
+// per warp, not the staged kernel's 227 KB: the rest of the SM's 256 KB is L1,
+// where the neighbours of a row are found (inner iteration of 484k rows 41.3 ->
+// 35.5 us; one tile per warp 35.5, three 36.9).
+constexpr int kSmemPairs = 512, kSmemSegs = 8;
+constexpr int kRingFixed = kThreads * 8 + 64 + 64 + kWarps * kSmemSegs * kSlots * 8;
+__host__ __device__ constexpr bool batch_states_fit(int nsys) { return nsys * kRhs <= kSmemPairs; }
+__host__ __device__ constexpr int batch_ring_smem(int bufs, int slot, int nsys) {
+    return kWarps * bufs * slot + kRingFixed +
+           (batch_states_fit(nsys) ? nsys * (kRhs * (int)sizeof(PairState) + 16) + (2 * (nsys + 1) + 3) / 4 * 16 : 0);
+}
+
 // ---------------------------------------------------------------- kernel
-template <class VT>
+template <class VT, bool RING>
 __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const Smem S = carve_smem(smem_raw);
-    __shared__ uint64_t rbar[kWarps * kRingBufs];
-    if (threadIdx.x < kWarps * kRingBufs) mbar_init(&rbar[threadIdx.x], 1);
-    init_pipeline(S);   // with the barriers' fence and a __syncthreads
+    __shared__ uint64_t rbar[RING ? kWarps * kRingBufs : 1];
+    PairState *st = B.state + (size_t)blockIdx.x * B.nsys * kRhs;
+    BalArrays bal{B.bal + (size_t)blockIdx.x * 2 * (B.nsys + 1), B.sinf + (size_t)blockIdx.x * B.nsys};
+    const WarpRows grows{B.wpart + (size_t)blockIdx.x * kWarps * kMaxSegPerCta * kSlots, kMaxSegPerCta};
+    WarpRows srows = grows;
+    Smem S;
+    if constexpr (RING) {
+        unsigned char *at = smem_raw;
+        S.stage = at;
+        at += kWarps * B.ring_bufs * B.ring_slot;
+        S.mbar = nullptr;
+        S.red = reinterpret_cast<double *>(at);
+        S.bcast = S.red + kThreads;
+        S.ctl = reinterpret_cast<int *>(S.bcast + 8);
+        at += kThreads * 8 + 64 + 64;
+        srows = WarpRows{reinterpret_cast<double *>(at), kSmemSegs};
+        at += kWarps * kSmemSegs * kSlots * 8;
+        if (batch_states_fit(B.nsys)) {
+            st = reinterpret_cast<PairState *>(at);
+            at += B.nsys * kRhs * sizeof(PairState);
+            bal.sinf = reinterpret_cast<int4 *>(at);
+            bal.pfx = reinterpret_cast<int32_t *>(at + B.nsys * 16);
+        }
+        if (threadIdx.x < kWarps * kRingBufs) mbar_init(&rbar[threadIdx.x], 1);
+        mbar_init_fence();
+        __syncthreads();
+    } else {
+        S = carve_smem(smem_raw);
+        init_pipeline(S);
+    }
+    auto warp_rows = [&](int segs) { return RING && segs <= kSmemSegs ? srows : grows; };
     uint32_t rcount = 0;
-    // the inner passes then read no vector with TMA: their barriers need no fence
-    const bool ring = B.ring_blob != nullptr;
     // the block-sum area is free in this kernel: it holds the layout arrays
     int *const bsm = reinterpret_cast<int *>(S.red);
     Balance &bl = *reinterpret_cast<Balance *>(bsm + kBalHdr);
@@ -975,7 +1054,6 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
     unsigned int epoch = 0;
     uint32_t count = 0;
     int set = 0;
-    PairState *st = B.state + (size_t)blockIdx.x * B.nsys * kRhs;
     const int npairs = B.nsys * kRhs;
     // the pairs' totals and decisions: L lanes per pair, the same pair count per
     // warp step (every lane of a warp takes part in the butterflies)
@@ -999,43 +1077,56 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
         return a;
     };
 
+    // without staged tiles no vector is read with TMA: the barriers need no fence
     for (int o = 0;; ++o) {
         // ------------------------------------------ outer residual (FP64)
-        zero_wpart(B, B.cta_nsys[blockIdx.x]);
-        for (int r = 0; r < nrhs; ++r) {
-            WarpAcc<double, 12> acc;
-            acc.seg = -1;
-            auto active = [&](int sys) { return (st[sys * kRhs + r].flags & kOuterActive) != 0; };
-            auto rowfn = [&](int sys, int i, double ax, WarpAcc<double, 12> &a) {
-                const double bi = B.B[(size_t)r * P.n + i];
-                const double ri = bi - ax;
-                a.a[r] = fma(ri, ri, a.a[r]);
-                a.a[4 + r] = fma(bi, bi, a.a[4 + r]);
-                const float rf = (float)ri;
-                const float zf = P.precond ? P.dinv32[i] * rf : rf;
-                float4 v = B.r32[i];
-                f4set(v, r, rf);
-                B.r32[i] = v;
-                v = B.p32[i];
-                f4set(v, r, zf);
-                B.p32[i] = v;
-                v = B.pd32[i];
-                f4set(v, r, zf);
-                B.pd32[i] = v;
-                v = B.q32[i];
-                f4set(v, r, 0.0f);
-                B.q32[i] = v;
-                v = B.d32[i];
-                f4set(v, r, 0.0f);
-                B.d32[i] = v;
-                a.a[8 + r] = fma((double)rf, (double)zf, a.a[8 + r]);
+        const WarpRows orows = warp_rows(B.cta_nsys[blockIdx.x]);
+        zero_wpart(orows, B.cta_nsys[blockIdx.x]);
+        auto outer_row = [&](int r, int i, double ax, WarpAcc<double, 12> &a) {
+            const double bi = B.B[(size_t)r * P.n + i];
+            const double ri = bi - ax;
+            a.a[r] = fma(ri, ri, a.a[r]);
+            a.a[4 + r] = fma(bi, bi, a.a[4 + r]);
+            const float rf = (float)ri;
+            const float zf = P.precond ? P.dinv32[i] * rf : rf;
+            float4 v = B.r32[i];
+            f4set(v, r, rf);
+            B.r32[i] = v;
+            v = B.p32[i];
+            f4set(v, r, zf);
+            B.p32[i] = v;
+            v = B.pd32[i];
+            f4set(v, r, zf);
+            B.pd32[i] = v;
+            v = B.q32[i];
+            f4set(v, r, 0.0f);
+            B.q32[i] = v;
+            v = B.d32[i];
+            f4set(v, r, 0.0f);
+            B.d32[i] = v;
+            a.a[8 + r] = fma((double)rf, (double)zf, a.a[8 + r]);
+        };
+        if constexpr (RING) {
+            WarpAcc<double, 12> acc(orows);
+            auto active = [&](int sys) { return any_flag(sys, kOuterActive); };
+            auto rowfn = [&](int sys, int i, const double (&ax)[kRhs], WarpAcc<double, 12> &a) {
+#pragma unroll
+                for (int r = 0; r < kRhs; ++r)
+                    if (r < nrhs && (st[sys * kRhs + r].flags & kOuterActive)) outer_row(r, i, ax[r], a);
             };
-            if (!batch_pass<double, double, double>(B, S, count, P.vals, B.xw + (size_t)r * B.xstride,
-                                                    static_tiles(B, active), rowfn, acc))
-                goto out;
+            batch_pass_outer(B, active, rowfn, acc);
+        } else {
+            for (int r = 0; r < nrhs; ++r) {
+                WarpAcc<double, 12> acc(orows);
+                auto active = [&](int sys) { return (st[sys * kRhs + r].flags & kOuterActive) != 0; };
+                auto rowfn = [&](int, int i, double ax, WarpAcc<double, 12> &a) { outer_row(r, i, ax, a); };
+                if (!batch_pass<double, double, double>(B, S, count, P.vals, B.xw + (size_t)r * B.xstride,
+                                                        static_tiles(B, active), rowfn, acc))
+                    goto out;
+            }
         }
-        combine_segments(B, set, 12);
-        if (!grid_barrier(P, epoch, S)) goto out;
+        combine_segments(B, orows, set, 12);
+        if (!grid_barrier<!RING>(P, epoch, S)) goto out;
         {
             int inner_any = 0;
             for (int q = q0; q - q0 < npairs; q += qstep) {
@@ -1084,7 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
             if (__syncthreads_or(inner_any)) {
                 // ------------------------------------------ inner CG (FP32, 4 rhs)
                 auto active = [&](int sys) { return any_flag(sys, kInnerActive); };
-                if (B.balance) compute_balance(B, active, bsm);
+                if (B.balance) compute_balance(B, bal, active, bsm);
                 else if (threadIdx.x == 0) bl.dyn = 0;
                 __syncthreads();
                 LaneTiles T;
@@ -1093,21 +1184,24 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     const int nloc = dyn ? bl.nloc : B.cta_nsys[blockIdx.x];
                     // p = z + beta p, q = A_lo z + beta q (= A_lo p); p.q
                     // (the SpMM gathers z: A p = A z + beta A p_old)
-                    zero_wpart(B, nloc);
+                    const WarpRows rows = warp_rows(nloc);
+                    zero_wpart(rows, nloc);
                     {
-                        WarpAcc<float, 4> acc;
-                        acc.seg = -1;
+                        WarpAcc<float, 4> acc(rows);
                         SpmmRow rowfn{B, st};
-                        const bool ok =
-                            ring  ? batch_pass_ring<VT>(B, S, rbar, rcount, bl, dyn, active, T, rowfn, acc)
-                            : dyn ? batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, balanced_tiles(B, bl), rowfn, acc)
-                                : batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, static_tiles(B, active), rowfn,
-                                                                 acc);
+                        bool ok;
+                        if constexpr (RING)
+                            ok = batch_pass_ring<VT>(B, S, rbar, rcount, bal, bl, dyn, active, T, rowfn, acc);
+                        else
+                            ok = dyn ? batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, balanced_tiles(B, bal, bl),
+                                                                      rowfn, acc)
+                                     : batch_pass<VT, float4, float4>(B, S, count, vlo, B.p32, static_tiles(B, active),
+                                                                      rowfn, acc);
                         if (!ok) goto out;
                     }
-                    if (dyn) combine_segments_dyn(B, set, 4, nloc);
-                    else combine_segments(B, set, 4);
-                    if (!(ring ? grid_barrier<false>(P, epoch, S) : grid_barrier(P, epoch, S))) goto out;
+                    if (dyn) combine_segments_dyn(B, rows, set, 4, nloc);
+                    else combine_segments(B, rows, set, 4);
+                    if (!grid_barrier<!RING>(P, epoch, S)) goto out;
                     int left_now = 0;
                     for (int q = q0; q - q0 < npairs; q += qstep) {
                         const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
@@ -1115,7 +1209,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         if (in) ps = st[q];
                         const int sl[1] = {q % kRhs}, sys = ps.flags & kInnerActive ? q / kRhs : -1;
                         float o[1];
-                        if (dyn) system_totals_dyn<1>(B, set, bl.total, sys, L, sl, o);
+                        if (dyn) system_totals_dyn<1>(B, bal, set, bl.total, sys, L, sl, o);
                         else system_totals<float>(B, set, sys, L, sl, o);
                         ps.alpha = 0.0f;
                         if (ps.flags & kInnerActive) {
@@ -1134,25 +1228,24 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     set ^= 1;
                     // d += alpha p, r -= alpha q, z = dinv r (gathered by the next SpMM:
                     // every gather of this one is over); r.r, r.z
-                    zero_wpart(B, nloc);
+                    zero_wpart(rows, nloc);
                     {
-                        WarpAcc<float, 8> acc;
-                        acc.seg = -1;
+                        WarpAcc<float, 8> acc(rows);
                         UpdateRow rowfn{B, st};
                         bool ok = true;
-                        if (ring) batch_pass_rows(B, bl, dyn, active, T, rowfn, acc);
+                        if constexpr (RING) batch_pass_rows(B, bal, bl, dyn, active, T, rowfn, acc);
                         else
                             ok = dyn ? batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
-                                                                      (const float4 *)nullptr, balanced_tiles(B, bl),
+                                                                      (const float4 *)nullptr, balanced_tiles(B, bal, bl),
                                                                       rowfn, acc)
                                      : batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr,
                                                                  (const float4 *)nullptr, static_tiles(B, active), rowfn,
                                                                  acc);
                         if (!ok) goto out;
                     }
-                    if (dyn) combine_segments_dyn(B, set, 8, nloc);
-                    else combine_segments(B, set, 8);
-                    if (!(ring ? grid_barrier<false>(P, epoch, S) : grid_barrier(P, epoch, S))) goto out;
+                    if (dyn) combine_segments_dyn(B, rows, set, 8, nloc);
+                    else combine_segments(B, rows, set, 8);
+                    if (!grid_barrier<!RING>(P, epoch, S)) goto out;
                     int left = 0;
                     for (int q = q0; q - q0 < npairs; q += qstep) {
                         const bool in = q < npairs, lead = in && ((int)threadIdx.x & (L - 1)) == 0;
@@ -1160,7 +1253,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         if (in) ps = st[q];
                         const int r = q % kRhs, sl[2] = {r, 4 + r}, sys = ps.flags & kInnerActive ? q / kRhs : -1;
                         float o[2];
-                        if (dyn) system_totals_dyn<2>(B, set, bl.total, sys, L, sl, o);
+                        if (dyn) system_totals_dyn<2>(B, bal, set, bl.total, sys, L, sl, o);
                         else system_totals<float>(B, set, sys, L, sl, o);
                         ps.beta = 0.0f;
                         if (ps.flags & kInnerActive) {
@@ -1184,12 +1277,12 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     // a pair left the inner loop: where its system did, re-split
                     if (__syncthreads_or(left_now)) {
                         if (B.balance) {
-                            const int32_t *rk = bal_pfx(B) + B.nsys + 1;
+                            const int32_t *rk = bal.pfx + B.nsys + 1;
                             int changed = 0;
                             for (int s = threadIdx.x; s < B.nsys; s += kThreads)
                                 changed |= (rk[s + 1] != rk[s]) != active(s);
                             if (__syncthreads_or(changed)) {
-                                compute_balance(B, active, bsm);
+                                compute_balance(B, bal, active, bsm);
                                 T.group = -1;
                             }
                         } else {
@@ -1208,8 +1301,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                 outer_left |= (st[q].flags & kOuterActive) != 0;
             }
             if (__syncthreads_or(ran)) {
-                WarpAcc<float, 0> acc;
-                acc.seg = -1;
+                WarpAcc<float, 0> acc(grows);
                 auto active = [&](int sys) { return any_flag(sys, kRanInner); };
                 auto rowfn = [&](int sys, int i, float4, WarpAcc<float, 0> &) {
                     const float4 d = B.d32[i];
@@ -1226,7 +1318,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                     goto out;
             }
             const bool more = __syncthreads_or(outer_left) != 0;
-            if (!grid_barrier(P, epoch, S)) goto out;
+            if (!grid_barrier<!RING>(P, epoch, S)) goto out;
             if (!more) break;
         }
     }
@@ -1388,6 +1480,12 @@ BatchParams batch_params(const cg_batch *h, const double *Bm, int nrhs, double t
 
 constexpr int kBatchSmem = kSmemBytes;
 
+const void *batch_kernel(int inner_values, bool ring) {
+    if (inner_values == CG_VALUES_BF16)
+        return ring ? (const void *)cg_batch_kernel<__nv_bfloat16, true> : (const void *)cg_batch_kernel<__nv_bfloat16, false>;
+    return ring ? (const void *)cg_batch_kernel<float, true> : (const void *)cg_batch_kernel<float, false>;
+}
+
 // The tiles with common offsets (batch_pass_ring), where every tile has at most
 // kRingMaxOffs of them and they hold at most a quarter more entries than the
 // matrix.
@@ -1419,7 +1517,9 @@ int build_batch_ring(cg_batch *h, const VT *lo) {
     }
     if (4 * entries > 5 * (size_t)h->nnz || at > (size_t)INT32_MAX) return CG_OK;
     h->ring_slot = batch_ring_bytes(wmax, (int)sizeof(VT));
-    h->ring_bufs = std::min(kRingBufs, kStageBytes / h->ring_slot);
+    h->ring_bufs = kRingBufs;
+    static_assert(kWarps * kRingBufs * batch_ring_bytes(kRingMaxOffs, 4) + kRingFixed + kSmemPairs * 80 <= kBatchSmem,
+                  "two tiles per warp fit");
     unsigned char *blob = nullptr;
     if ((rc = bdev_alloc(h, &h->ring_meta, meta.size())) || (rc = bdev_alloc(h, &blob, at * 16)) ||
         (rc = bupload(h->ring_meta, meta)))
@@ -1440,9 +1540,10 @@ int batch_enqueue(cg_batch *h, const double *Bm, double *X, int nrhs, double tol
     if (e == cudaSuccess) {
         BatchParams B = batch_params(h, Bm, nrhs, tol, maxit);
         void *args[] = {&B};
-        const void *kern = h->opts.inner_values == CG_VALUES_BF16 ? (const void *)cg_batch_kernel<__nv_bfloat16>
-                                                                  : (const void *)cg_batch_kernel<float>;
-        e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kThreads), args, (size_t)kBatchSmem, h->stream);
+        const bool ring = B.ring_blob != nullptr;
+        const int smem = ring ? batch_ring_smem(h->ring_bufs, h->ring_slot, h->nsys) : kBatchSmem;
+        e = cudaLaunchCooperativeKernel(batch_kernel(h->opts.inner_values, ring), dim3(h->ctas), dim3(kThreads), args,
+                                        (size_t)smem, h->stream);
     }
     if (e == cudaSuccess && copy_back)
         e = cudaMemcpy2DAsync(X, col, h->xw, pitch, col, (size_t)nrhs, cudaMemcpyDeviceToDevice, h->stream);
@@ -1565,12 +1666,12 @@ int cg_batch_create(const cg_csr *systems, int32_t nsys, const cg_opts *opts_in,
 
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(CG_ECUDA);
-    if (cudaFuncSetAttribute((const void *)cg_batch_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kBatchSmem) != cudaSuccess ||
-        cudaFuncSetAttribute((const void *)cg_batch_kernel<__nv_bfloat16>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kBatchSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_batch_kernel<float>, kThreads, kBatchSmem) !=
-            cudaSuccess ||
+    for (const bool ring : {false, true})
+        if (cudaFuncSetAttribute(batch_kernel(opts.inner_values, ring), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kBatchSmem) != cudaSuccess)
+            return fail(CG_ECUDA);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel(opts.inner_values, false), kThreads,
+                                                      kBatchSmem) != cudaSuccess ||
         per_sm < 1)
         return fail(CG_ECUDA);
     int ctas = opts.grid_ctas > 0 ? std::min(opts.grid_ctas, sms * per_sm) : sms;
