@@ -48,7 +48,7 @@ constexpr int kMaxSegPerCta = 64;
 
 // Per-pair solver state; every CTA keeps its own identical copy.
 struct PairState {
-    double rho;        // inner r.z
+    float rho;         // inner r.z
     double bnorm;      // ||b||
     double relres;     // last outer ||b - A x|| / ||b||
     double target2;    // (inner_tol ||r_outer||)^2
@@ -85,7 +85,7 @@ struct BatchParams {
     int32_t *bal;                // ctas x 2 (nsys + 1): per CTA, active-tile and active-system prefixes
     int4 *sinf;                  // ctas x nsys: per CTA, each active system's first and last piece, its
                                  // segment in the first piece (x, y, z) and whether some piece is empty (w)
-    double *segdyn;              // 2 x ctas x kMaxSegPerCta x kSlots: per-piece segment sums
+    float *segdyn;               // 2 x ctas x kMaxSegPerCta x kSlots: per-piece segment sums
     int32_t balance;             // 1: the inner loop may use the balanced layout
     // tiles with common offsets (nullptr: the staged tiles): see batch_pass_ring
     const int2 *ring_meta;       // per tile: offset of its blob in 16-byte units, width
@@ -186,17 +186,32 @@ __device__ __forceinline__ void zero_wpart(const WarpRows &R, int ns) {
     __syncwarp();
 }
 
+// Sum of the warp rows at (segment, slot), four rows on each of four neighbouring
+// lanes: an FP64 addition occupies a sub-partition's FP64 pipe for 64 clocks, so
+// the warp that adds all 16 rows takes 1k clocks per reduction, so 0.4k.  (With
+// every warp in step, 16 warps share those pipes: 2.4k; only warps with a pair
+// of their own take part.)
+__device__ __forceinline__ double quad_rows_sum(const WarpRows &R, int seg, int slot) {
+    static_assert(kWarps % 4 == 0, "whole rows per lane");
+    const int w0 = (threadIdx.x & 3) * (kWarps / 4);
+    double s = R.row(w0)[(size_t)seg * kSlots + slot];
+#pragma unroll
+    for (int w = 1; w < kWarps / 4; ++w) s += R.row(w0 + w)[(size_t)seg * kSlots + slot];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    return s;
+}
+
 // Adds the 16 warp rows of each of this CTA's segments (fixed order) into
 // segpart[set], for the first nslots slots.
 __device__ __forceinline__ void combine_segments(const BatchParams &B, const WarpRows &R, int set, int nslots) {
     __syncthreads();
     const int ns = B.cta_nsys[blockIdx.x], seg0 = B.cta_seg0[blockIdx.x];
-    for (int q = threadIdx.x; q < ns * nslots; q += kThreads) {
-        const int j = q / nslots, i = q % nslots;
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) s += R.row(w)[(size_t)j * kSlots + i];
-        B.segpart[((size_t)set * B.nseg + seg0 + j) * kSlots + i] = s;
+    for (int q = threadIdx.x / 4; (q & ~7) < ns * nslots; q += kThreads / 4) {
+        const bool in = q < ns * nslots;
+        const int j = in ? q / nslots : 0, i = in ? q % nslots : 0;
+        const double s = quad_rows_sum(R, j, i);
+        if (in && (threadIdx.x & 3) == 0) B.segpart[((size_t)set * B.nseg + seg0 + j) * kSlots + i] = s;
     }
 }
 
@@ -452,13 +467,12 @@ __device__ void compute_balance(const BatchParams &B, const BalArrays &A, const 
 __device__ __forceinline__ void combine_segments_dyn(const BatchParams &B, const WarpRows &R, int set, int nslots,
                                                      int nloc) {
     __syncthreads();
-    double *dst = B.segdyn + ((size_t)set * gridDim.x + blockIdx.x) * kMaxSegPerCta * kSlots;
-    for (int q = threadIdx.x; q < nloc * nslots; q += kThreads) {
-        const int j = q / nslots, i = q % nslots;
-        double s = 0.0;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) s += R.row(w)[(size_t)j * kSlots + i];
-        dst[(size_t)j * kSlots + i] = s;
+    float *dst = B.segdyn + ((size_t)set * gridDim.x + blockIdx.x) * kMaxSegPerCta * kSlots;
+    for (int q = threadIdx.x / 4; (q & ~7) < nloc * nslots; q += kThreads / 4) {
+        const bool in = q < nloc * nslots;
+        const int j = in ? q / nslots : 0, i = in ? q % nslots : 0;
+        const double s = quad_rows_sum(R, j, i);
+        if (in && (threadIdx.x & 3) == 0) dst[(size_t)j * kSlots + i] = (float)s;
     }
 }
 
@@ -478,9 +492,9 @@ __device__ __forceinline__ void system_totals_dyn(const BatchParams &B, const Ba
             // an empty piece (fewer active tiles than CTAs) holds nothing
             const bool empty = v.w && (long long)c * total / G == (long long)(c + 1) * total / G;
             const int j = c == v.x ? bchk(v.z, kMaxSegPerCta) : 0;
-            const double *src = B.segdyn + (((size_t)set * G + c) * kMaxSegPerCta + j) * kSlots;
+            const float *src = B.segdyn + (((size_t)set * G + c) * kMaxSegPerCta + j) * kSlots;
 #pragma unroll
-            for (int i = 0; i < NS; ++i) out[i] += empty ? 0.0f : (float)__ldcg(src + sl[i]);
+            for (int i = 0; i < NS; ++i) out[i] += empty ? 0.0f : __ldcg(src + sl[i]);
         }
     }
 #pragma unroll
@@ -1149,7 +1163,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         ps.status = CG_OK;
                         ps.flags = kRanInner;
                         ps.relres = 0.0;
-                        ps.rho = -1.0;
+                        ps.rho = -1.0f;
                     } else if (rr <= (B.tol * ps.bnorm) * (B.tol * ps.bnorm)) {
                         ps.status = CG_OK;
                         ps.flags = 0;
@@ -1161,7 +1175,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         ps.flags = 0;
                     } else {
                         ps.flags = kOuterActive | kInnerActive | kRanInner;
-                        ps.rho = rz;
+                        ps.rho = (float)rz;
                         ps.beta = 0.0f;   // p_1 = z_0, q_1 = A z_0
                         ps.target2 = B.inner_tol * B.inner_tol * rr;
                         ps.outer = o + 1;
@@ -1218,7 +1232,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                                 ps.flags &= ~kInnerActive;  // keep d so far
                                 left_now = 1;
                             } else {
-                                ps.alpha = (float)ps.rho / sg;
+                                ps.alpha = ps.rho / sg;
                             }
                         }
                         __syncwarp();
@@ -1264,7 +1278,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                                 ps.flags &= ~kInnerActive;
                                 left_now = 1;
                             } else {
-                                ps.beta = rz / (float)ps.rho;
+                                ps.beta = rz / ps.rho;
                                 ps.rho = rz;
                                 left = 1;
                             }
@@ -1309,7 +1323,7 @@ __global__ void __launch_bounds__(kThreads, 1) cg_batch_kernel(BatchParams B) {
                         const PairState &ps = st[sys * kRhs + r];
                         if (!(ps.flags & kRanInner)) continue;
                         double &x = B.xw[(size_t)r * B.xstride + i];
-                        x = ps.rho < 0.0 ? 0.0 : x + (double)f4c(d, r);
+                        x = ps.rho < 0.0f ? 0.0 : x + (double)f4c(d, r);
                     }
                 };
                 if (!batch_pass<VT, float4, float4>(B, S, count, (const VT *)nullptr, (const float4 *)nullptr,
@@ -1359,7 +1373,7 @@ struct cg_batch {
     int32_t *cta_sys0 = nullptr, *cta_nsys = nullptr, *cta_seg0 = nullptr, *sys_seg0 = nullptr;
     int32_t *sys_tile0 = nullptr, *bal = nullptr;
     int4 *sinf = nullptr;
-    double *segdyn = nullptr;
+    float *segdyn = nullptr;
     int4 *tiles_win = nullptr, *tiles_gather = nullptr, *segs = nullptr;
     uint16_t *lcol = nullptr, *vals16 = nullptr;
     double *vals = nullptr, *xw = nullptr, *wpart = nullptr, *segpart = nullptr;
