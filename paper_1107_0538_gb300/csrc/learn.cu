@@ -32,6 +32,7 @@
 // kernel, or by every CTA after the grid barrier (fixed-order sums: bitwise
 // reproducible), and kept in a device state block; kernels return at once
 // after the solve is done.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -281,6 +282,11 @@ __device__ __forceinline__ bool conv_skip(const FcgState *st) {
     return st && (st->done || st->mode != kModeLearned);
 }
 
+// The fields the tensor-core convolution reads (h1, h2 of the solver and the
+// apply) hold channels 0-7 of every position, then channels 8-15, each a padded
+// grid of 16-byte positions: a brick's rows of one half are contiguous boxes.
+__device__ __forceinline__ long long half_field(const Geo &G) { return (G.npad + kSlack) * 8; }
+
 // Gates of a warp's output rows, loaded ahead of the MMA loop: gv[m][hrow][nb]
 // (two channels each), zero for dropped rows.
 template <int EPI>
@@ -317,7 +323,7 @@ __device__ __forceinline__ void store16(const ConvArgs &A, const Brick &B, int w
 #pragma unroll
             for (int nb = 0; nb < 2; ++nb) {
                 const int ch = nb * 8 + 2 * t4;
-                const long long e = pos * kCh + ch;
+                const long long e = EPI == E_GATE ? nb * half_field(A.G) + pos * 8 + 2 * t4 : pos * kCh + ch;
                 float v0 = acc[m][nb][2 * hrow] * oscale, v1 = acc[m][nb][2 * hrow + 1] * oscale;
                 if (EPI == E_SIGMOID) {
                     v0 = 1.0f / (1.0f + __expf(-(v0 + A.bias[ch])));
@@ -399,24 +405,39 @@ __global__ void __launch_bounds__(kCT, 3) conv16_kernel(ConvArgs A) {
 // the stand-alone apply) on the 5th-generation tensor cores.  A CTA owns a
 // brick of 8 (x) x 16 (y) x 4 (z) outputs.  Its input with the halo (10 x 18
 // x 6 positions) is staged channel-split: channels 0-7 of every position in
-// one plane of 16-byte rows, channels 8-15 in a second plane.  The 128
+// one plane of 16-byte rows, channels 8-15 in a second plane.  The field has
+// the same split, so one TMA box copy stages a brick (with 16-byte cp.async
+// from a field of 32-byte positions staging alone took 40 of 63 us at 101^3
+// nodes, whatever the products cost).  The 128
 // outputs of a z-plane of the brick (x fastest, 8 per y) then form an
 // M = 128 operand in the canonical K-major layout without swizzle: 8-row
 // core matrices of consecutive x, 16 bytes per row, y groups one staged row
-// (160 bytes) apart, the two K halves one plane apart.  Tap (dx, dy, dz) is
-// the same operand moved by dx + 10 dy + 180 dz positions, so each of the 27
-// taps is one MMA (M = 128, N = 16, K = 16; BF16 in, FP32 accumulate) into
-// the plane's 16 TMEM columns: 108 MMAs per brick, issued by one thread per
-// plane, completing on an mbarrier.  Warps w and w + 4 read TMEM lanes
-// 32 (w mod 4) .. + 31 (output i = lane index) of alternate planes.
+// (160 bytes) apart, the two K halves one plane apart.  Input plane zi moved by
+// (dx, dy) is such an operand, and it feeds the output planes zi - 2 .. zi (dz =
+// 1, 0, -1), whose 16 TMEM columns each are neighbours: one MMA with N = 48
+// (K = 16; BF16 in, FP32 accumulate) per (zi, dx, dy), fewer columns at the
+// brick's ends.  An MMA this narrow is bound by reading its 4 KB A operand from
+// shared memory (32 clocks); one MMA per tap and output plane (N = 16) read it
+// 108 times per brick, this 57.  Planes ascend, so each output adds its taps in
+// the order dz, dy, dx.  One thread issues them with descriptors that differ by
+// constants; they complete on an mbarrier.  Warps w and w + 4 read TMEM lanes
+// 32 (w mod 4) .. + 31 (output i = lane index) of alternate planes.  The kernel
+// is persistent, two CTAs per SM: its ninth warp loads brick i + 2 and issues the
+// products of brick i + 1 (two staging buffers, two sets of TMEM columns) while
+// the others write brick i.  At 101^3 nodes 37 us (63 before): 30 of them are
+// the products, 64 clocks each (an operand that starts between 128-byte lines is
+// read in two passes); without them 22 to 26.
 constexpr int kTX = 8, kTY = 16, kTZ = 4;
 constexpr int kTSX = kTX + 2, kTSY = kTY + 2, kTSZ = kTZ + 2;
 constexpr int kTStaged = kTSX * kTSY * kTSZ;                  // 1080 positions
 constexpr uint32_t kTPlane = (uint32_t)kTStaged * 16;          // bytes of one channel half
 constexpr uint32_t kTWeights = (uint32_t)kTaps * kCh * kCh * 2;  // 13824 bytes
-constexpr uint32_t kTCols = 64;                                // TMEM columns: 4 planes x 16
+constexpr uint32_t kTXyBytes = 3u * kCh * kCh * 2;             // weights of one (dx, dy)
+constexpr uint32_t kTCols = 128;                               // TMEM columns: 2 bricks x 4 planes x 16
 static_assert(kTX * kTY == 128, "one M = 128 operand per z-plane");
-size_t conv16tc_smem(const Geo &) { return 2 * (size_t)kTPlane + kTWeights + 16; }
+constexpr uint32_t kTBuf = 2 * kTPlane;                         // one staged brick
+constexpr int kTThreads = kCT + 32;
+size_t conv16tc_smem(const Geo &) { return 2 * (size_t)kTBuf + kTWeights + 48; }
 
 // Shared-memory matrix descriptor (SM100 version 1), no swizzle: start, LBO
 // (K-direction core-matrix stride) and SBO (M/N-direction 8-row group
@@ -426,8 +447,10 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
 }
 // Instruction descriptor of kind::f16: FP32 D, BF16 A and B, both K-major,
-// N = 16 (bits 17-22: N / 8), M = 128 (bits 24-28: M / 16).
-constexpr uint32_t kConvIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
+// N (bits 17-22: N / 8), M = 128 (bits 24-28: M / 16).
+__host__ __device__ constexpr uint32_t conv_idesc(uint32_t n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+}
 
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t accumulate) {
@@ -456,130 +479,180 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 
 __device__ __forceinline__ void finish(FcgState *st, int status);
 
+// A brick's staged box: 10 x positions (80 elements of a half), 18 y, 6 z, both
+// halves.  Positions past the padded grid arrive as zeros; they only feed
+// outputs that are dropped.
+__device__ __forceinline__ void load_box(const CUtensorMap &map, void *dst, uint64_t *bar, int x, int y, int z) {
+    mbar_arrive_expect_tx(bar, kTBuf);
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
+        "[%2];" ::"r"(smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(&map)), "r"(smem_u32(bar)), "r"(x * 8), "r"(y), "r"(z), "r"(0)
+        : "memory");
+}
+
+// The products of one staged brick into its TMEM columns (one thread).
+__device__ __forceinline__ void issue_brick(uint32_t tmem, uint64_t ad0, uint64_t bd0, uint64_t *bar) {
+#pragma unroll
+    for (int zi = 0; zi < kTSZ; ++zi) {
+#pragma unroll
+        for (int xy = 0; xy < 9; ++xy) {
+            const uint64_t ad = ad0 + (uint64_t)(xy % 3 + kTSX * (xy / 3 + kTSY * zi));
+            const uint64_t bd = bd0 + (uint64_t)(xy * kTXyBytes / 16);
+            const int p0 = zi < 2 ? 0 : zi - 2;
+            int p1 = zi < kTZ ? zi : kTZ - 1;
+            if (xy == 0 && zi < kTZ) {   // the first product of output plane zi
+                umma_bf16(tmem + (uint32_t)zi * 16, ad, bd + 2 * 16, conv_idesc(16), 0u);
+                --p1;
+            }
+            if (p1 >= p0)
+                umma_bf16(tmem + (uint32_t)p0 * 16, ad, bd + (uint64_t)((2 - zi + p0) * 16),
+                          conv_idesc(16u * (uint32_t)(p1 - p0 + 1)), 1u);
+        }
+    }
+    umma_commit(bar);
+}
+
 template <int EPI>
-__global__ void __launch_bounds__(kCT) conv16tc_kernel(ConvArgs A) {
+__global__ void __launch_bounds__(kTThreads, 2) conv16tc_kernel(ConvArgs A, const __grid_constant__ CUtensorMap in) {
     static_assert(EPI == E_STORE || EPI == E_GATE, "forward epilogues only");
     if (conv_skip(A.st)) return;
     extern __shared__ __align__(128) unsigned char sm[];
     const Geo &G = A.G;
-    unsigned char *sw = sm + 2 * kTPlane;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(sw + kTWeights);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
-    const int tile = blockIdx.x, rest = tile / G.tbx;
-    const int x0 = (tile % G.tbx) * kTX, y0 = (rest % G.tby) * kTY, z0 = (rest / G.tby) * kTZ;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    unsigned char *sw = sm + 2 * kTBuf;
+    // full[b]: brick staged in buffer b; prod[b]: its products are in TMEM set b
+    uint64_t *full = reinterpret_cast<uint64_t *>(sw + kTWeights), *prod = full + 2;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(prod + 2);
+    const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    constexpr int kLoader = kCT / 32;   // the ninth warp
+    const int bricks = (G.ttiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // >= 1
 
-    // input with halo: staged position (xs, ys, zs) is padded node
-    // (x0 + xs, y0 + ys, z0 + zs); rows past the padded grid are zero.  A
-    // warp copies one staged row (10 positions: 320 contiguous bytes) at a
-    // time, lane l < 20 one 16-byte chunk.
-    {
-        const int xs = lane >> 1, h = lane & 1;
-        for (int row = w; row < kTSY * kTSZ; row += kCT / 32) {
-            if (lane >= 2 * kTSX) continue;
-            const int ys = row % kTSY, zs = row / kTSY;
-            const int py = y0 + ys, pz = z0 + zs;
-            unsigned char *dst = sm + h * kTPlane + (uint32_t)(row * kTSX + xs) * 16;
-            if (py < G.py && pz < G.pz)
-                cp_async16(dst, A.in + ((long long)pz * G.plane + (long long)py * G.px + x0 + xs) * kCh + h * 8);
-            else
-                *reinterpret_cast<uint4 *>(dst) = make_uint4(0u, 0u, 0u, 0u);
-        }
-    }
-    // weights of tap t: B = K[t] as 16 (N = output) rows of 16 (K = input)
-    // channels, K halves 256 bytes apart, 8-row groups 128 bytes apart; a
-    // warp copies one tap (32 chunks) at a time
-    for (int t = w; t < kTaps; t += kCT / 32) {
-        const int o = lane >> 1, h = lane & 1;
-        cp_async16(sw + t * 512 + h * 256 + o * 16, A.w + ((size_t)t * kCh + o) * kCh + h * 8);
-    }
-    if (w == 0) {
+    if (w == kLoader) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                      "r"(kTCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (threadIdx.x == 32) {
-        mbar_init(bar, kTZ);   // one commit per issuing warp
-        mbar_init_fence();
-    }
-    // gates of this thread's outputs, loaded while the MMAs run
-    uint4 gq[2][2];
-    const int i = 32 * (w & 3) + lane;   // output (M row, TMEM lane) of this thread
-    const int ox = x0 + (i & 7), oy = y0 + (i >> 3);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int oz = z0 + (w >> 2) + 2 * k;
-        const bool ok = ox < G.nx && oy < G.ny && oz < G.nz;
-        const long long pos = padded_pos(G, ox, oy, oz);
-        if (EPI == E_GATE && ok) {
-            gq[k][0] = __ldg(reinterpret_cast<const uint4 *>(A.gate + pos * kCh));
-            gq[k][1] = __ldg(reinterpret_cast<const uint4 *>(A.gate + pos * kCh + 8));
-        } else {
-            gq[k][0] = gq[k][1] = make_uint4(0u, 0u, 0u, 0u);
+        if (lane == 0) {
+            for (int b = 0; b < 2; ++b) {
+                mbar_init(&full[b], 1);
+                mbar_init(&prod[b], 1);
+            }
+            mbar_init_fence();
         }
     }
+    auto load = [&](int it) {   // one thread
+        const int tile = (int)blockIdx.x + it * (int)gridDim.x, rest = tile / G.tbx, b = it & 1;
+        load_box(in, sm + b * kTBuf, &full[b], (tile % G.tbx) * kTX, (rest % G.tby) * kTY, (rest / G.tby) * kTZ);
+    };
+    // weights of (dx, dy): B = K for dz = 1, 0, -1 as 3 x 16 (N = output) rows of
+    // 16 (K = input) channels, K halves 768 bytes apart, 8-row groups 128 bytes
+    // apart; a warp copies one tap (32 chunks) at a time
+    for (int t = w; t < kTaps; t += kTThreads / 32) {
+        const int o = lane >> 1, h = lane & 1;
+        cp_async16(sw + (t % 9) * kTXyBytes + h * (kTXyBytes / 2) + (2 - t / 9) * 256 + o * 16,
+                   A.w + ((size_t)t * kCh + o) * kCh + h * 8);
+    }
     cp_async_wait_all();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // staged data -> tensor-core reads
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // weights -> tensor-core reads
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    // a thread's tcgen05.mma issue takes ~165 cycles however small the MMA,
-    // against ~10 cycles of tensor work at N = 16: lane 0 of warps 0-3 issue
-    // the 27 taps of one z-plane each, into their own TMEM columns
-    if (lane == 0 && w < kTZ) {
-        const int pl = w;
-        const uint32_t in_base = smem_u32(sm), w_base = smem_u32(sw);
-#pragma unroll 1
-        for (int t = 0; t < kTaps; ++t) {
-            const int s0 = (1 + tap_dx(t)) + kTSX * ((1 + tap_dy(t)) + kTSY * (1 + pl + tap_dz(t)));
-            const uint64_t ad = umma_desc(in_base + (uint32_t)s0 * 16, kTPlane, kTSX * 16);
-            const uint64_t bd = umma_desc(w_base + (uint32_t)t * 512, 256, 128);
-            umma_bf16(tmem + (uint32_t)pl * 16, ad, bd, kConvIdesc, t > 0 ? 1u : 0u);
-        }
-        umma_commit(bar);
+    int failed = 0;
+    auto products = [&](int it) {   // the ninth warp
+        const int b = it & 1;
+        failed = __any_sync(0xffffffffu, !mbar_wait_bounded(&full[b], (uint32_t)(it >> 1) & 1u, A.wait_ns));
+        uint32_t one;   // elected, not lane == 0: the descriptors then stay in uniform registers
+        asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+        if (one && !failed)
+            issue_brick(tmem + (uint32_t)b * 64, umma_desc(smem_u32(sm + b * kTBuf), kTPlane, kTSX * 16),
+                        umma_desc(smem_u32(sw), kTXyBytes / 2, 128), &prod[b]);
+        __syncwarp();
+    };
+    if (w == kLoader) {
+        if (lane == 0)
+            for (int it = 0; it < min(bricks, 2); ++it) load(it);
+        __syncwarp();
+        products(0);
     }
-    bool done = mbar_wait_bounded(bar, 0, A.wait_ns);
-    tc_fence_after();
-    if (done) {
+    const int i = 32 * (w & 3) + lane;   // output (M row, TMEM lane) of this thread
+    int it = 0;
+    for (; it < bricks; ++it) {
+        if (w == kLoader) {
+            // the other buffer's brick; its TMEM columns were read before the last __syncthreads
+            if (it + 1 < bricks && !failed) products(it + 1);
+        } else {
+            const int tile = (int)blockIdx.x + it * (int)gridDim.x, rest = tile / G.tbx;
+            const int ox = (tile % G.tbx) * kTX + (i & 7), oy = (rest % G.tby) * kTY + (i >> 3);
+            const int z0 = (rest / G.tby) * kTZ;
+            // gates of this thread's outputs, loaded while the products run
+            uint4 gq[2][2];
+            long long pos[2];
+            bool ok[2];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int pl = (w >> 2) + 2 * k;
-            uint32_t v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)pl * 16, v);
-            const int oz = z0 + pl;
-            if (ox < G.nx && oy < G.ny && oz < G.nz) {
-                const long long pos = padded_pos(G, ox, oy, oz);
-                uint32_t o[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    float a0 = __uint_as_float(v[2 * j]), a1 = __uint_as_float(v[2 * j + 1]);
-                    if (EPI == E_GATE) {
-                        const uint32_t gw = (&gq[k][j >> 2].x)[j & 3];
-                        const float2 g = unpack_bf16(gw);
-                        a0 *= g.x;
-                        a1 *= g.y;
-                    }
-                    o[j] = pack_bf16(a0, a1);
+            for (int k = 0; k < 2; ++k) {
+                const int oz = z0 + (w >> 2) + 2 * k;
+                ok[k] = ox < G.nx && oy < G.ny && oz < G.nz;
+                pos[k] = padded_pos(G, ox, oy, oz);
+                gq[k][0] = gq[k][1] = make_uint4(0u, 0u, 0u, 0u);
+                if (EPI == E_GATE && ok[k]) {
+                    gq[k][0] = __ldg(reinterpret_cast<const uint4 *>(A.gate + pos[k] * kCh));
+                    gq[k][1] = __ldg(reinterpret_cast<const uint4 *>(A.gate + pos[k] * kCh + 8));
                 }
-                uint4 *dst = reinterpret_cast<uint4 *>(A.out + pos * kCh);
-                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
+            failed = __any_sync(0xffffffffu, !mbar_wait_bounded(&prod[it & 1], (uint32_t)(it >> 1) & 1u, A.wait_ns));
+            tc_fence_after();
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (failed) break;
+                uint32_t v[16];
+                tmem_ld16(tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((it & 1) * 64 + ((w >> 2) + 2 * k) * 16),
+                          v);
+                if (ok[k]) {
+                    uint32_t o[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        float a0 = __uint_as_float(v[2 * j]), a1 = __uint_as_float(v[2 * j + 1]);
+                        if (EPI == E_GATE) {
+                            const uint32_t gw = (&gq[k][j >> 2].x)[j & 3];
+                            const float2 g = unpack_bf16(gw);
+                            a0 *= g.x;
+                            a1 *= g.y;
+                        }
+                        o[j] = pack_bf16(a0, a1);
+                    }
+                    // E_STORE's field is read by this kernel again, E_GATE's by the 16 -> 1 convolution
+                    __nv_bfloat16 *lo = A.out + pos[k] * (EPI == E_STORE ? 8 : kCh);
+                    __nv_bfloat16 *hi = lo + (EPI == E_STORE ? half_field(G) : 8);
+                    *reinterpret_cast<uint4 *>(lo) = make_uint4(o[0], o[1], o[2], o[3]);
+                    *reinterpret_cast<uint4 *>(hi) = make_uint4(o[4], o[5], o[6], o[7]);
+                }
+            }
+            tc_fence_before();
         }
-    } else {
-        // report, then give the MMAs in flight a second bounded wait before
-        // the columns are freed
+        failed = __syncthreads_or(failed);
+        if (failed) break;
+        if (w == kLoader) {
+            tc_fence_after();
+            // brick it's products are complete: its buffer is free
+            if (lane == 0 && it + 2 < bricks) load(it + 2);
+            __syncwarp();
+        }
+    }
+    if (failed) {   // the same in every thread
+        // report, then give the copies and products in flight a second bounded
+        // wait before the columns are freed
         if (threadIdx.x == 0) {
             if (A.st) finish(A.st, CG_ETIMEOUT);
             if (A.err) atomicExch(A.err, CG_ETIMEOUT);
         }
-        done = mbar_wait_bounded(bar, 0, A.wait_ns);
+        for (int u = it; u < min(it + 2, bricks); ++u)
+            if (mbar_wait_bounded(&full[u & 1], (uint32_t)(u >> 1) & 1u, A.wait_ns))
+                mbar_wait_bounded(&prod[u & 1], (uint32_t)(u >> 1) & 1u, A.wait_ns);
     }
     tc_fence_before();
     __syncthreads();
-    if (w == 0) {
+    if (w == kLoader) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTCols) : "memory");
     }
@@ -1774,6 +1847,7 @@ struct LearnCtx {
     int window = 50;
     double factor = 0.9;
     std::vector<void *> allocs;
+    CUtensorMap h1_map, h2_map;      // h1, h2 as boxes (conv16tc_kernel)
     __nv_bfloat16 *lognu_in = nullptr, *gates = nullptr, *h1 = nullptr, *h2 = nullptr, *k1 = nullptr;
     __nv_bfloat16 *s_in = nullptr;   // padded D^-1/2 r (network input)
     int32_t *pidx = nullptr;         // padded position of each node
@@ -1823,6 +1897,38 @@ int convout_grid(const Geo &G) {
     return std::max(1, std::min(G.tiles, resident));
 }
 
+// CTAs of a tensor-core convolution launch: two per SM (its launch bounds and
+// shared memory), each looping over its share of the bricks.
+int conv16tc_grid(const Geo &G) {
+    static const int resident = [] {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        return 2 * sm_count(dev);
+    }();
+    return std::max(1, std::min(G.ttiles, resident));
+}
+
+// The tensor map of a channel-split field: x positions of 8 channels, y, z and
+// the half, staged boxes of 10 x 18 x 6 positions of both halves.
+int field_map(const Geo &G, const __nv_bfloat16 *field, CUtensorMap *map) {
+    using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (found != cudaDriverEntryPointSuccess || !fn) return CG_ECUDA;
+    const cuuint64_t dims[4] = {(cuuint64_t)G.px * 8, (cuuint64_t)G.py, (cuuint64_t)G.pz, 2};
+    const cuuint64_t strides[3] = {(cuuint64_t)G.px * 16, (cuuint64_t)G.plane * 16, (cuuint64_t)(G.npad + kSlack) * 16};
+    const cuuint32_t box[4] = {kTSX * 8, kTSY, kTSZ, 2}, step[4] = {1, 1, 1, 1};
+    const CUresult r = reinterpret_cast<Encode>(fn)(
+        map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<__nv_bfloat16 *>(field), dims, strides, box, step,
+        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? CG_OK : CG_ECUDA;
+}
+
 template <class T>
 int ctx_alloc(std::vector<void *> &allocs, T **p, size_t count, bool zero = true) {
     *p = nullptr;
@@ -1862,7 +1968,6 @@ int set_smem_limits() {
                                      (int)cudaSharedmemCarveoutMaxL1);
     };
     set((const void *)conv16_kernel<E_STORE>);
-    set((const void *)conv16_kernel<E_GATE>);
     set((const void *)conv16_kernel<E_GATE_PRE>);
     set((const void *)conv16_kernel<E_BWD_GATE>);
     set((const void *)conv16tc_kernel<E_STORE>);
@@ -1944,16 +2049,14 @@ void enqueue_body(cg_handle *h, LearnCtx *L, cudaStream_t s) {
     A.out = L->h1;
     conv1_kernel<E_GATE><<<G.tiles, kCT, conv1_smem(G), s>>>(A);
     // h2 = C2(h1)
-    A.in = L->h1;
     A.w = net->d.k2;
     A.out = L->h2;
     A.wait_ns = (unsigned long long)(h->opts.wait_limit_s * 1e9);
-    conv16tc_kernel<E_STORE><<<G.ttiles, kCT, conv16tc_smem(G), s>>>(A);
+    conv16tc_kernel<E_STORE><<<conv16tc_grid(G), kTThreads, conv16tc_smem(G), s>>>(A, L->h1_map);
     // k1 = g * C2^T(h2)
-    A.in = L->h2;
     A.w = net->d.k2t;
     A.out = L->k1;
-    conv16tc_kernel<E_GATE><<<G.ttiles, kCT, conv16tc_smem(G), s>>>(A);
+    conv16tc_kernel<E_GATE><<<conv16tc_grid(G), kTThreads, conv16tc_smem(G), s>>>(A, L->h2_map);
     // z = sigma D^-1/2 C1^T(k1) (or D^-1 r), z.r, z.q, beta
     A.in = L->k1;
     A.w = net->d.k1t;
@@ -2513,7 +2616,8 @@ int cg_set_learned(cg_handle *h, cg_net *net, int32_t ex, int32_t ey, int32_t ez
         (rc = ctx_alloc(A, &L->dsq32, (size_t)G.n)) ||
         (rc = ctx_alloc(A, &L->q, (size_t)G.n)) || (rc = ctx_alloc(A, &L->partials, (size_t)3 * nparts)) ||
         (rc = ctx_alloc(A, &L->sigma, 4)) || (rc = ctx_alloc(A, &L->counter, 4)) || (rc = ctx_alloc(A, &L->st, 1)) ||
-        (rc = ctx_alloc(A, &L->dst, 1)) || (rc = ctx_alloc(A, &L->conv_err, 1)))
+        (rc = ctx_alloc(A, &L->dst, 1)) || (rc = ctx_alloc(A, &L->conv_err, 1)) ||
+        (rc = field_map(G, L->h1, &L->h1_map)) || (rc = field_map(G, L->h2, &L->h2_map)))
         return fail(rc);
     if (cudaMallocHost(&L->st_host, sizeof(FcgState)) != cudaSuccess ||
         cudaMallocHost(&L->flags_host, 2 * sizeof(FcgFlags)) != cudaSuccess ||
@@ -2564,16 +2668,14 @@ int cg_precond_apply(cg_handle *h, const double *r, double *z) {
     A.w = L->net->d.k1in;
     A.out = L->h1;
     conv1_kernel<E_GATE><<<G.tiles, kCT, conv1_smem(G), s>>>(A);
-    A.in = L->h1;
     A.w = L->net->d.k2;
     A.out = L->h2;
     A.wait_ns = (unsigned long long)(h->opts.wait_limit_s * 1e9);
     A.err = L->conv_err;
-    conv16tc_kernel<E_STORE><<<G.ttiles, kCT, conv16tc_smem(G), s>>>(A);
-    A.in = L->h2;
+    conv16tc_kernel<E_STORE><<<conv16tc_grid(G), kTThreads, conv16tc_smem(G), s>>>(A, L->h1_map);
     A.w = L->net->d.k2t;
     A.out = L->k1;
-    conv16tc_kernel<E_GATE><<<G.ttiles, kCT, conv16tc_smem(G), s>>>(A);
+    conv16tc_kernel<E_GATE><<<conv16tc_grid(G), kTThreads, conv16tc_smem(G), s>>>(A, L->h2_map);
     A.in = L->k1;
     A.w = L->net->d.k1t;
     A.z = z;
