@@ -919,11 +919,14 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
             const uint2 v = __ldg(reinterpret_cast<const uint2 *>(A.w) + threadIdx.x);   // 4 BF16 weights
             swt[threadIdx.x] = make_float4(bf16_lo(v.x), bf16_hi(v.x), bf16_lo(v.y), bf16_hi(v.y));
         }
-        // quad Q = thread / 4 owns outputs x = 8 (Q & 1) .. + 7 of brick row
-        // Q / 2 (y = row mod kBY, z = row / kBY); lane j = thread mod 4 adds
-        // input channels 4 j .. 4 j + 3 and finishes outputs 2 j and 2 j + 1
+        // quad Q = thread / 4 owns outputs x = 8 xh .. + 7 of brick row brow (y =
+        // row mod kBY, z = row / kBY), xh = bit 2 of Q, so the four quads of a
+        // half-warp read four rows (disjoint banks: an 8-byte load serves a
+        // half-warp per wavefront; with both halves of one row in it, two);
+        // lane j = thread mod 4 adds input channels 4 j .. 4 j + 3 and finishes
+        // outputs 2 j and 2 j + 1
         const int j4 = threadIdx.x & 3, quad = threadIdx.x >> 2;
-        const int xh = quad & 1, brow = quad >> 1;
+        const int xh = (quad >> 2) & 1, brow = (quad >> 3) * 4 + (quad & 3);
         const int oy = brow % kBY, oz = brow / kBY;
         const float sigma = EPI == E_OUT_LOSS ? 1.0f : (float)(st ? st->sigma : A.sigma[0]);
         // the CTA's bricks b = blockIdx.x, + gridDim.x, ...: brick k is
