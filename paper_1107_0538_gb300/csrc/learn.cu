@@ -117,7 +117,7 @@ size_t conv1_smem(const Geo &) { return kStage1; }
 constexpr int kOutRowBytes = kSX * 32 + 32;
 static_assert(kOutRowBytes % 16 == 0, "16-byte aligned staged rows");
 constexpr size_t kOutStage = (size_t)kSY * kSZ * kOutRowBytes;   // one staged brick
-size_t convout_smem(const Geo &) { return 2 * kOutStage; }          // two: the next brick loads meanwhile
+size_t convout_smem(const Geo &) { return kOutStage; }
 size_t wgrad16_smem(const Geo &) { return kStage16 + kDyTile; }
 size_t wgrad1_smem(const Geo &) { return kStage1 + kDyTile + (size_t)(kCT / 32) * 16 * 32 * 4; }
 
@@ -819,10 +819,12 @@ __device__ __forceinline__ void finish(FcgState *st, int status) {
 // the same bits in every lane).  Input rows are staged 608 bytes apart (18
 // positions of 32 bytes plus 32), so the 32-byte pieces of the 4 rows a warp
 // reads at once fall on disjoint groups of 8 banks: a warp's load takes the
-// minimum two wavefronts (the shared-memory pipe bounds this kernel).  The kernel is persistent: a CTA loops over its share of
-// the bricks with two staging buffers, so the copies of the next brick run
-// while the current one is multiplied, the weights are read once per CTA and
-// each CTA publishes one partial of z.r and z.q.
+// minimum two wavefronts (the shared-memory pipe bounds this kernel).  The
+// kernel is persistent, four CTAs per SM with one staging buffer each: a CTA
+// loads its next brick while it finishes the last one and the other CTAs
+// multiply; the weights are read once per CTA and each CTA publishes one partial
+// of z.r and z.q.  At 101^3 nodes 44.6 us; with two buffers and three CTAs 49.1
+// (2366 bricks are 5.2 rounds of 456 CTAs, 3.9 of 608).
 // Stages a brick's 16-channel input rows with the TMA unit: one 1-D bulk
 // copy per staged row (18 positions, 576 contiguous bytes of the padded
 // grid), completing on bar.  Thread r < kSY kSZ issues row r (or zero-fills
@@ -903,13 +905,13 @@ __device__ __forceinline__ OutNodes out_nodes(const ConvArgs &A, const Brick &B,
 }
 
 template <int EPI>
-__global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
+__global__ void __launch_bounds__(kCT, 4) convout_kernel(ConvArgs A) {
     FcgState *st = A.st;
     if (st && st->done) return;
     extern __shared__ __align__(128) unsigned char sm[];
     __shared__ double sred[2 * 32];
     __shared__ float4 swt[kTaps * 4];   // tap t, channels 4 j .. 4 j + 3 at swt[4 t + j]
-    __shared__ __align__(8) uint64_t sbar[2];   // TMA completion of the two staging buffers
+    __shared__ __align__(8) uint64_t sbar;   // TMA completion of the staged brick
     __shared__ int sflag, sswitch;
     const Geo &G = A.G;
     const bool learned = !st || st->mode == kModeLearned;
@@ -929,35 +931,27 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
         const int xh = (quad >> 2) & 1, brow = (quad >> 3) * 4 + (quad & 3);
         const int oy = brow % kBY, oz = brow / kBY;
         const float sigma = EPI == E_OUT_LOSS ? 1.0f : (float)(st ? st->sigma : A.sigma[0]);
-        // the CTA's bricks b = blockIdx.x, + gridDim.x, ...: brick k is
-        // multiplied from buffer k mod 2 while brick k + 1 is staged into the
-        // other one, and the epilogue operands of a lane's two nodes are
-        // loaded one brick ahead
+        // the CTA's bricks b = blockIdx.x, + gridDim.x, ...: brick k + 1 is
+        // staged as soon as brick k is multiplied, and the epilogue operands
+        // of a lane's two nodes are loaded one brick ahead
         const int nb = G.tiles;
         int b = blockIdx.x;
         if (threadIdx.x == 0) {
-            mbar_init(&sbar[0], 1);
-            mbar_init(&sbar[1], 1);
+            mbar_init(&sbar, 1);
             mbar_init_fence();
         }
         __syncthreads();
-        if (b < nb) stage16_rows_tma(G, brick_of(G, b), A.in, sm, &sbar[0]);
+        if (b < nb) stage16_rows_tma(G, brick_of(G, b), A.in, sm, &sbar);
         OutNodes nd = out_nodes<EPI>(A, brick_of(G, b), xh, oy, oz, j4, b < nb);
         for (int k = 0; b < nb; ++k, b += gridDim.x) {
-            const unsigned char *cur = sm + (size_t)(k & 1) * kOutStage;
             const int bn = b + gridDim.x;
-            if (bn < nb) stage16_rows_tma(G, brick_of(G, bn), A.in, sm + (size_t)((k + 1) & 1) * kOutStage,
-                                          &sbar[(k + 1) & 1]);
-            // brick b has landed (use k / 2 of its buffer's barrier); brick bn
-            // may still be in flight
-            if (!mbar_wait_bounded(&sbar[k & 1], (uint32_t)((k >> 1) & 1), A.wait_ns)) {
+            if (!mbar_wait_bounded(&sbar, (uint32_t)(k & 1), A.wait_ns)) {
                 // report, then give the copies in flight a second bounded wait
                 if (threadIdx.x == 0) {
                     if (st) finish(st, CG_ETIMEOUT);
                     if (A.err) atomicExch(A.err, CG_ETIMEOUT);
                 }
-                mbar_wait_bounded(&sbar[k & 1], (uint32_t)((k >> 1) & 1), A.wait_ns);
-                if (bn < nb) mbar_wait_bounded(&sbar[(k + 1) & 1], (uint32_t)(((k + 1) >> 1) & 1), A.wait_ns);
+                mbar_wait_bounded(&sbar, (uint32_t)(k & 1), A.wait_ns);
                 return;
             }
             __syncthreads();   // the zero-filled rows (plain stores) too
@@ -966,7 +960,7 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
             uint64_t acc2[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc2[i] = 0ull;
-            const unsigned char *in0 = cur + (size_t)(xh * 8) * 32 + j4 * 8;
+            const unsigned char *in0 = sm + (size_t)(xh * 8) * 32 + j4 * 8;
             const ulonglong2 *wt = reinterpret_cast<const ulonglong2 *>(swt) + j4;
 #pragma unroll
             for (int g9 = 0; g9 < 9; ++g9) {
@@ -984,6 +978,8 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
                     if (j >= 2) acc2[j - 2] = ffma2(wp.y, a23, ffma2(wp.x, a01, acc2[j - 2]));
                 }
             }
+            __syncthreads();   // the buffer is read: the next brick loads while this one is finished
+            if (bn < nb) stage16_rows_tma(G, brick_of(G, bn), A.in, sm, &sbar);
             float acc[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -1020,7 +1016,6 @@ __global__ void __launch_bounds__(kCT) convout_kernel(ConvArgs A) {
                 }
             }
             nd = out_nodes<EPI>(A, brick_of(G, bn), xh, oy, oz, j4, bn < nb);
-            __syncthreads();   // buffer k mod 2 is staged again for brick k + 2
         }
     } else {
         const int n = G.n;
