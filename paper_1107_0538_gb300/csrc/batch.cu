@@ -1779,10 +1779,17 @@ int cg_batch_create(const cg_csr *systems, int32_t nsys, const cg_opts *opts_in,
         for (int32_t i = 0; i < n; ++i) di[i] = 1.0f / inner.diag[i];
         if ((rc = bupload(h->dinv32, di))) return fail(rc);
     }
+    const size_t mark = h->allocs.size();
     rc = opts.inner_values == CG_VALUES_FP32
              ? build_batch_ring<float>(h, h->vals32)
              : build_batch_ring<__nv_bfloat16>(h, reinterpret_cast<const __nv_bfloat16 *>(h->vals16));
-    if (rc != CG_OK) return fail(rc);
+    if (rc == CG_ENOMEM) {   // the batch keeps its staged tiles
+        cudaGetLastError();
+        for (; h->allocs.size() > mark; h->allocs.pop_back()) cudaFree(h->allocs.back());
+        h->ring_meta = nullptr;
+    } else if (rc != CG_OK) {
+        return fail(rc);
+    }
     *out = h;
     return CG_OK;
 }

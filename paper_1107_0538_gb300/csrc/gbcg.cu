@@ -1381,6 +1381,23 @@ int fixed_scales(cg_handle *h, bool *ok) {
     return CG_OK;
 }
 
+// Builds a further copy of the matrix; without memory for it the handle keeps
+// the kernels that need none.
+template <class F>
+int optional_copy(cg_handle *h, F build) {
+    const size_t mark = h->allocs.size();
+    const int64_t bytes = h->device_bytes;
+    const int rc = build();
+    if (rc != CG_ENOMEM) return rc;
+    cudaGetLastError();
+    for (; h->allocs.size() > mark; h->allocs.pop_back()) cudaFree(h->allocs.back());
+    h->device_bytes = bytes;
+    h->fixed_c = nullptr;
+    h->fixed_vals = nullptr;
+    h->ring_meta = nullptr;
+    return CG_OK;
+}
+
 // The fixed-point copy of the handle's SELL-32 matrix, for the slice and
 // cluster kernels.
 int build_fixed(cg_handle *h, size_t entries) {
@@ -2000,18 +2017,25 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         // (48.7), 57x44x61 11.1 (18.1), 50^3 9.7 (13.8), 20^3 9.1 (13.9).
         int max_slices = 0;
         for (size_t c = 0; c + 1 < scut.size(); ++c) max_slices = std::max(max_slices, scut[c + 1] - scut[c]);
-        if (h->sell_solve && !mixed && (rc = build_fixed(h, tot)) != CG_OK) return fail(rc);
+        if (h->sell_solve && !mixed && (rc = optional_copy(h, [&] { return build_fixed(h, tot); })) != CG_OK)
+            return fail(rc);
         if (h->sell_mem && !mixed) {
-            bool ok = false;
             const void *k[] = {(const void *)cg_ring_kernel<false>, (const void *)cg_ring_kernel<true>};
-            if ((rc = fixed_scales(h, &ok)) != CG_OK) return fail(rc);
-            if (ok && (rc = build_ring<int2>(h, k, 2, tot, max_slices, l2)) != CG_OK) return fail(rc);
+            rc = optional_copy(h, [&] {
+                bool ok = false;
+                const int r = fixed_scales(h, &ok);
+                return r == CG_OK && ok ? build_ring<int2>(h, k, 2, tot, max_slices, l2) : r;
+            });
+            if (rc != CG_OK) return fail(rc);
         } else if ((h->sell_solve || h->sell_mem) && mixed) {
             const void *k32[] = {(const void *)cg_irring_kernel<float>, (const void *)lo_spmv_ring_kernel<float>};
             const void *k16[] = {(const void *)cg_irring_kernel<__nv_bfloat16>,
                                  (const void *)lo_spmv_ring_kernel<__nv_bfloat16>};
-            rc = opts.inner_values == CG_VALUES_FP32 ? build_ring<float>(h, k32, 2, tot, max_slices, l2)
-                                                     : build_ring<__nv_bfloat16>(h, k16, 2, tot, max_slices, l2);
+            rc = optional_copy(h, [&] {
+                return opts.inner_values == CG_VALUES_FP32
+                           ? build_ring<float>(h, k32, 2, tot, max_slices, l2)
+                           : build_ring<__nv_bfloat16>(h, k16, 2, tot, max_slices, l2);
+            });
             if (rc != CG_OK) return fail(rc);
         }
         // refinement of matrices without common offsets, on the SELL copies for
