@@ -30,13 +30,17 @@
 // it: a process that resets a device must not call this entry point on it
 // again.
 //
-// It is the recurrence of the SELL-32 solve kernels (two grid barriers per
-// iteration: q = A r + beta q, p = r + beta p, then x and r), with their
-// fixed-order sums, thread-0 scalars and bounded barriers, and a row-per-thread
-// SpMV straight from the caller's CSR arrays instead of the SELL-32 copy that
-// cg_create builds.  Per iteration, against the three-barrier form with two
-// entries in flight per row: 50^3 17.1 us (22.6), 60x61x59 25.1 (29.5),
-// 37x41x29 13.0 (15.4), 20^3 11.7 (14.0).
+// It is textbook CG (q = A p, then x and r, then p: three grid barriers per
+// iteration), with the fixed-order sums, thread-0 scalars and bounded barriers
+// of the SELL-32 solve kernels, and a row-per-thread SpMV straight from the
+// caller's CSR arrays instead of the SELL-32 copy that cg_create builds.  The
+// product loads nine entries of a row before their FMAs; x += alpha p runs while
+// thread 0 waits for the barrier of r.r.  Per iteration, against two entries in
+// flight and 512 threads: 50^3 18.2 us (22.6), 60x61x59 25.9 (29.5), 37x41x29 13.7
+// (15.4), 20^3 12.6 (14.0).  A third barrier could be saved with q = A r + beta q
+// (17.1, 25.1, 13.0 and 11.7 us), but that q collects the rounding of all
+// iterations before it: after 116 iterations at 37x41x29 to 60^3 the iterates were 10 to
+// 300 times further from exact ones.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -194,14 +198,13 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1) cg_noalloc_kernel(Noallo
     int status = CG_OK, iters = 0;
     double rr = 0.0, bb = 0.0, rho = 0.0, bnorm = 0.0, tol2bb = 0.0;
 
-    // setup: r = b - A x, p = r, q = 0; r.r, b.b (and any malformed row)
+    // setup: r = b - A x, p = r; r.r, b.b (and any malformed row)
     double v[3] = {0.0, 0.0, 0.0};
     for (int i = row_lo + tid; i < row_hi; i += kT) {
         const double bi = A.b[i];
         const double ri = bi - noalloc_row<true>(A, i, A.x, nnz, bad);
         P.r[i] = ri;
         P.pd[i] = ri;
-        P.q[i] = 0.0;
         v[0] = fma(ri, ri, v[0]);
         v[1] = fma(bi, bi, v[1]);
     }
@@ -235,19 +238,15 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1) cg_noalloc_kernel(Noallo
     }
     if (ctl[0]) {
         if (tid == 0) status = CG_ENOCONV;
-        double beta = 0.0;   // p_1 = r_0, q_1 = A r_0
         for (int k = 1; k <= P.maxit; ++k) {
-            // q = A r + beta q (= A p), p = r + beta p; p . q
+            // q = A p, p . q
             double v1[1] = {0.0};
             for (int i = row_lo + tid; i - (tid & 31) < row_hi; i += kT) {
-                const double az = two ? noalloc_rows2(A, i - (tid & 31), row_hi, P.r)
-                                      : (i < row_hi ? noalloc_row<false>(A, i, P.r, nnz, bad) : 0.0);
+                const double qi = two ? noalloc_rows2(A, i - (tid & 31), row_hi, P.pd)
+                                      : (i < row_hi ? noalloc_row<false>(A, i, P.pd, nnz, bad) : 0.0);
                 if (i >= row_hi) break;
-                const double qi = fma(beta, P.q[i], az);
-                const double pi = fma(beta, P.pd[i], P.r[i]);
                 P.q[i] = qi;
-                P.pd[i] = pi;
-                v1[0] = fma(pi, qi, v1[0]);
+                v1[0] = fma(P.pd[i], qi, v1[0]);
             }
             block_sum_1k<1>(v1, red, quarter);
             publish_partials<1>(P, set, v1);
@@ -266,7 +265,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1) cg_noalloc_kernel(Noallo
             __syncthreads();
             if (!ctl[0]) break;
             const double alpha = bcast[0];
-            // r -= alpha q (every gather of it is over); r.r
+            // r -= alpha q; r.r
             double v2[1] = {0.0};
             for (int i = row_lo + tid; i < row_hi; i += kT) {
                 const double ri = fma(-alpha, P.q[i], P.r[i]);
@@ -300,7 +299,10 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1) cg_noalloc_kernel(Noallo
             }
             __syncthreads();
             if (!ctl[0]) break;
-            beta = bcast[1];
+            // p = r + beta p (every gather of it is over), published for the next product
+            const double beta = bcast[1];
+            for (int i = row_lo + tid; i < row_hi; i += kT) P.pd[i] = fma(beta, P.pd[i], P.r[i]);
+            if (!grid_barrier<false>(P, epoch, S)) return;
         }
     }
     if (blockIdx.x == 0 && tid == 0) {
