@@ -49,6 +49,7 @@
 #include <mutex>
 
 #include "gbcg.h"
+#include "rowwalk.h"
 #include "sellsolve.cuh"
 
 using namespace gbcg;
@@ -109,13 +110,13 @@ __device__ __forceinline__ double noalloc_row(const NoallocArgs &A, int i, const
         return 0.0;
     }
     double s = 0.0;
-    for (int k = k0; k < k1; k += kNoallocUnroll) {
+    for (RowWalk<kNoallocUnroll> e(k0, k1); e.more(); e.next()) {
         double vr[kNoallocUnroll], xr[kNoallocUnroll];
 #pragma unroll
         for (int u = 0; u < kNoallocUnroll; ++u) {
-            const bool in = k + u < k1;
-            vr[u] = in ? __ldg(A.vals + k + u) : 0.0;
-            const int c = in ? __ldg(A.colidx + k + u) : i;
+            const bool in = e.has(u);
+            vr[u] = in ? __ldg(A.vals + e.k + u) : 0.0;
+            const int c = in ? __ldg(A.colidx + e.k + u) : i;
             if (CHECK) {
                 const bool ok = (unsigned)c < (unsigned)A.n;
                 bad |= !ok;
@@ -126,7 +127,7 @@ __device__ __forceinline__ double noalloc_row(const NoallocArgs &A, int i, const
         }
 #pragma unroll
         for (int u = 0; u < kNoallocUnroll; ++u)
-            if (k + u < k1) s = fma(vr[u], xr[u], s);
+            if (e.has(u)) s = fma(vr[u], xr[u], s);
     }
     return s;
 }
@@ -143,32 +144,28 @@ __device__ __forceinline__ double noalloc_row(const NoallocArgs &A, int i, const
 // 48000 (316 per CTA), where latency counts, 14.0 and 12.6.
 __device__ __forceinline__ double noalloc_rows2(const NoallocArgs &A, int base, int row_hi, const double *v) {
     const int lane = threadIdx.x & 31;
-    int k[2], k1[2];
     double s[2] = {0.0, 0.0};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int row = base + 16 * h + (lane >> 1);
+    auto row_walk = [&](int row) {
         const bool in = row < row_hi;
-        k[h] = in ? __ldg(A.rowptr + row) + (lane & 1) : 0;
-        k1[h] = in ? __ldg(A.rowptr + row + 1) : 0;
-    }
-    while (__any_sync(0xffffffffu, k[0] < k1[0] || k[1] < k1[1])) {
+        return RowWalk<2 * kNoallocUnroll2>(in ? __ldg(A.rowptr + row) : 0, in ? __ldg(A.rowptr + row + 1) : 0, lane & 1);
+    };
+    RowWalk<2 * kNoallocUnroll2> e[2] = {row_walk(base + (lane >> 1)), row_walk(base + 16 + (lane >> 1))};
+    while (__any_sync(0xffffffffu, e[0].more() || e[1].more())) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             double vr[kNoallocUnroll2], xr[kNoallocUnroll2];
 #pragma unroll
             for (int u = 0; u < kNoallocUnroll2; ++u) {
-                const int e = k[h] + 2 * u;
                 vr[u] = xr[u] = 0.0;
-                if (e < k1[h]) {
-                    vr[u] = __ldg(A.vals + e);
-                    xr[u] = __ldca(v + __ldg(A.colidx + e));
+                if (e[h].has(2 * u)) {
+                    vr[u] = __ldg(A.vals + e[h].k + 2 * u);
+                    xr[u] = __ldca(v + __ldg(A.colidx + e[h].k + 2 * u));
                 }
             }
 #pragma unroll
             for (int u = 0; u < kNoallocUnroll2; ++u)
-                if (k[h] + 2 * u < k1[h]) s[h] = fma(vr[u], xr[u], s[h]);
-            k[h] += 2 * kNoallocUnroll2;
+                if (e[h].has(2 * u)) s[h] = fma(vr[u], xr[u], s[h]);
+            e[h].next();
         }
     }
     const int src = 2 * (lane & 15);
