@@ -105,6 +105,7 @@ KERNEL_SOURCES = {
     "cg_sell_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "cg_sellmem_kernel": ["gbcg.cu", "sell.cuh", "fixed.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "sell_spmv_kernel": ["gbcg.cu", "sell.cuh", "plan.h"],
+    "cg_cluster_kernel": ["gbcg.cu", "cluster.cuh", "fixed.cuh", "sell.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "cg_ring_kernel": ["gbcg.cu", "ring.cuh", "fixed.cuh", "sell.cuh", "sellsolve.cuh", "plan.h"] + _COMMON,
     "cg_irring_kernel": ["gbcg.cu", "ring.cuh", "sell.cuh", "sellsolve.cuh", "plan.h", "lowprec.h"] + _COMMON,
     "cg_ir_kernel": ["gbcg.cu", "plan.h", "lowprec.h"] + _COMMON,
@@ -587,13 +588,13 @@ def measure_forms_100cube(flush, fp64_tflops: float, count: int = 2) -> dict:
             if it is not None:
                 tried[f"{it:g}"] = round(v_ms, 3)
             if best is None or v_ms < best[0]:
-                best = (v_ms, res_v[-1][1], x.cpu().numpy(), vs.plan(), it)
+                best = (v_ms, res_v[-1][1], x.cpu().numpy(), vs.kernel(), it)
             vs.close()
-        v_ms, info_v, xv, plan_v, it_best = best
+        v_ms, info_v, xv, kernel_v, it_best = best
         if name == "fp64_cg":
             x_fp64, ms_fp64 = xv.copy(), v_ms
             # FP64-ALU roofline of the solve kernel (Table I's flop count)
-            kern = "cg_ring_kernel" if plan_v["slice_solve"] == 2 else "cg_solve_kernel"
+            kern = kernel_v.split("/")[0]
             kern_s = statistics.mean(i.kernel_ms for _, i in res_v) / 1e3
             flops = info_v.iters * flops_per_iteration(big.A.n, big.A.nnz, False)
             tr = ncu_traffic(kern)
@@ -772,9 +773,7 @@ def run_gbcg(args) -> None:
     kern_s = statistics.mean(kern_ms) / 1e3
     achieved_tflops = iters * fpi / kern_s / 1e12
     achieved_gbs = iters * bpi / kern_s / 1e9
-    # the persistent solve kernel the plan picked: one SELL-32 slice per warp
-    # (systems up to 31 slices per CTA) or the tiled kernel
-    solve_kernel = "cg_sell_kernel" if solver.plan()["slice_solve"] else "cg_solve_kernel"
+    solve_kernel = solver.kernel().split("/")[0]   # the persistent kernel the handle picked
     tr = ncu_traffic(solve_kernel)
     fp64 = fp64_peak(stream)
     nominal = fp64["sms"] * 2 * 2 * (clk.summary()["sm_max_mhz"] or 2070.0) * 1e6 / 1e12

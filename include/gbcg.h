@@ -149,12 +149,10 @@ typedef struct {
                                 vectors_in_memory                                 */
     int32_t window_tiles;    /* tiles whose gathers read a staged x-window        */
     int64_t device_bytes;    /* device memory the handle owns                     */
-    int32_t slice_solve;     /* FP64 solves run: 1 the SELL-32 kernel with one
-                                32-row slice per warp and rows in registers; 2
-                                the SELL-32 kernel with the vectors in memory
-                                (reg_rows 0); 0 that kernel too when reg_rows is
-                                not 0, else the tiled kernel described by the
-                                fields above                                     */
+    int32_t slice_solve;     /* how the SELL-32 slices are shared out: 1 at most one
+                                32-row slice per warp; 2 more, and reg_rows is 0;
+                                0 more, and reg_rows is not 0, or vectors_in_memory.
+                                It names no kernel: cg_kernel_name does          */
     int32_t inner_solve;     /* handles with inner_values FP32/BF16: 1 when the
                                 refinement runs with one 32-row slice per warp;
                                 0 for larger systems and when it runs on the staged
@@ -230,6 +228,19 @@ int cg_spmv_inner(cg_handle *h, const float *x, float *y);
 
 /* Fills *plan with the handle's launch plan.  CG_EINVAL on NULL arguments. */
 int cg_get_plan(const cg_handle *h, cg_plan *plan);
+
+/*
+ * The kernel that the handle's solves run, as text that lives as long as the
+ * library: "cg_cluster_kernel" (small systems, one thread-block cluster),
+ * "cg_sell_kernel" (one 32-row slice per warp), "cg_ring_kernel" (matrix through a
+ * shared-memory ring), "cg_sellmem_kernel" or "cg_solve_kernel" (row tiles), each
+ * followed by "/int" where A z is summed in exact integers or "/fp64" where by FP64
+ * FMAs; for handles with inner_values FP32/BF16 "cg_irring_kernel",
+ * "cg_irsell_kernel" or "cg_ir_kernel" (row tiles); for CG_PRECOND_LEARNED "fcg_sell_kernel"
+ * or "fcg_spmv_kernel", the one that multiplies with A in flexible CG, and ""
+ * before cg_set_learned.  "" for NULL.
+ */
+const char *cg_kernel_name(const cg_handle *h);
 
 /* Frees everything the handle owns (after synchronizing its stream).
  * cg_destroy(NULL) is a no-op; a handle must not be destroyed twice. */
@@ -353,6 +364,12 @@ int cg_batch_tune(cg_batch *h, const double *B, double *X, int32_t nrhs, double 
  * ignored.  CG_EINVAL otherwise.  Takes effect at the next enqueue.
  */
 int cg_batch_set_tuning(cg_batch *h, const cg_batch_tuning *choice);
+
+/* The form of cg_batch_kernel that the handle's solves run with its present
+ * tuning: "cg_batch_kernel/offsets" (tiles stored by their rows' common column
+ * offsets) or "cg_batch_kernel/staged" (tiles staged through shared memory).
+ * "" for NULL. */
+const char *cg_batch_kernel_name(const cg_batch *h);
 
 /* Frees the batch handle (NULL is a no-op). */
 void cg_batch_destroy(cg_batch *h);

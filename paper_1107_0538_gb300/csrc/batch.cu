@@ -1430,6 +1430,10 @@ void batch_free(cg_batch *h) {
     delete h;
 }
 
+// Whether the handle's solves run on the tiles with common offsets: the tuned
+// kinds other than one lane per row on windows stay staged tiles.
+bool batch_ring(const cg_batch *h) { return h->ring_blob && !h->use_gather && h->lanes_per_row == 1; }
+
 BatchParams batch_params(const cg_batch *h, const double *Bm, int nrhs, double tol, int maxit) {
     BatchParams B{};
     Params &P = B.P;
@@ -1483,8 +1487,7 @@ BatchParams batch_params(const cg_batch *h, const double *Bm, int nrhs, double t
     B.sinf = h->sinf;
     B.segdyn = h->segdyn;
     B.balance = (h->ctas <= kMaxBalCtas && !h->static_split) ? 1 : 0;
-    // the tuned kinds other than one lane per row on windows stay staged tiles
-    const bool ring = h->ring_blob && !h->use_gather && h->lanes_per_row == 1;
+    const bool ring = batch_ring(h);
     B.ring_meta = h->ring_meta;
     B.ring_blob = ring ? h->ring_blob : nullptr;
     B.ring_slot = h->ring_slot;
@@ -1893,6 +1896,11 @@ int cg_batch_set_tuning(cg_batch *h, const cg_batch_tuning *choice) {
     h->lanes_per_row = choice->lanes_per_row;
     h->static_split = choice->static_split;
     return CG_OK;
+}
+
+const char *cg_batch_kernel_name(const cg_batch *h) {
+    if (!h) return "";
+    return batch_ring(h) ? "cg_batch_kernel/offsets" : "cg_batch_kernel/staged";
 }
 
 void cg_batch_destroy(cg_batch *h) { batch_free(h); }

@@ -1571,6 +1571,17 @@ cudaLaunchConfig_t cluster_config(const cg_handle *h, cudaLaunchAttribute *at) {
     return cfg;
 }
 
+// The kernel of a handle's solves: the one decision that enqueue_solve and
+// cg_kernel_name share.
+enum class SolvePath { cluster, ring, irring, sell, sellmem, irsell, tiled, tiled_ir };
+SolvePath solve_path(const cg_handle *h) {
+    const bool mixed = h->opts.inner_values != CG_VALUES_FP64;
+    if (h->cluster_ctas > 0) return SolvePath::cluster;
+    if (h->ring_blob) return mixed ? SolvePath::irring : SolvePath::ring;
+    if (mixed) return h->sell_lo ? SolvePath::irsell : SolvePath::tiled_ir;
+    return h->sell_solve ? SolvePath::sell : h->sell_mem ? SolvePath::sellmem : SolvePath::tiled;
+}
+
 // Enqueues one solve on the handle's stream (no synchronization).
 int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t maxit, int precond) {
     Params P = base_params(h);
@@ -1584,7 +1595,8 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
     if (e == cudaSuccess) e = cudaMemsetAsync(h->st, 0, sizeof(DevStatus), h->stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev0, h->stream);
     if (e == cudaSuccess) {
-        if (h->cluster_ctas > 0) {
+        const SolvePath path = solve_path(h);
+        if (path == SolvePath::cluster) {
             const SellMatrix M = sell_of(h);
             const FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
             const ClusterArgs L{h->cluster_cut, h->cluster_win, h->cluster_entries, h->cluster_window};
@@ -1592,7 +1604,7 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
             const cudaLaunchConfig_t cfg = cluster_config(h, &at);
             e = precond ? cudaLaunchKernelEx(&cfg, cg_cluster_kernel<true>, P, M, F, L)
                         : cudaLaunchKernelEx(&cfg, cg_cluster_kernel<false>, P, M, F, L);
-        } else if (h->ring_blob) {
+        } else if (path == SolvePath::ring || path == SolvePath::irring) {
             SellMatrix M = sell_of(h);
             RingMatrix R = ring_of(h);
             const int32_t *cut = h->sell_cut;
@@ -1600,23 +1612,24 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
             int u = h->fixed_u;
             void *z = h->ring_z;
             void *args64[] = {&P, &M, &R, &c, &u, &z, &cut}, *args_ir[] = {&P, &M, &R, &z, &cut};
-            const bool fp64 = h->opts.inner_values == CG_VALUES_FP64;
+            const bool fp64 = path == SolvePath::ring;
             const void *kern = fp64 ? (precond ? (const void *)cg_ring_kernel<true> : (const void *)cg_ring_kernel<false>)
                                : h->opts.inner_values == CG_VALUES_FP32
                                    ? (const void *)cg_irring_kernel<float>
                                    : (const void *)cg_irring_kernel<__nv_bfloat16>;
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), fp64 ? args64 : args_ir,
                                             ring_smem(h), h->stream);
-        } else if ((h->sell_solve || h->sell_mem) && h->opts.inner_values == CG_VALUES_FP64) {
+        } else if (path == SolvePath::sell || path == SolvePath::sellmem) {
             SellMatrix M = sell_of(h);
             FixedMatrix F{h->fixed_vals, h->sell_c16, h->fixed_c, h->fixed_u};
             const int32_t *cut = h->sell_cut;
             void *args_slice[] = {&P, &M, &F, &cut}, *args_mem[] = {&P, &M, &cut};
-            void **args = h->sell_solve ? args_slice : args_mem;
+            const bool slice = path == SolvePath::sell;
+            void **args = slice ? args_slice : args_mem;
             const bool pre = precond != 0, fx = h->fixed_vals != nullptr;
-            const void *kern = h->sell_solve ? sell_kernel_for(pre, fx) : sellmem_kernel_for(pre, fx);
+            const void *kern = slice ? sell_kernel_for(pre, fx) : sellmem_kernel_for(pre, fx);
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), args, 0, h->stream);
-        } else if (h->sell_lo && h->opts.inner_values != CG_VALUES_FP64) {
+        } else if (path == SolvePath::irsell) {
             SellMatrix M = sell_of(h);
             const int32_t *cut = h->sell_cut;
             const void *vlo = h->sell_lo;
@@ -2290,6 +2303,22 @@ int cg_get_plan(const cg_handle *h, cg_plan *plan) {
     p.inner_solve = h->sell_lo || (h->ring_blob && h->sell_solve && h->opts.inner_values != CG_VALUES_FP64) ? 1 : 0;
     *plan = p;
     return CG_OK;
+}
+
+const char *cg_kernel_name(const cg_handle *h) {
+    if (!h) return "";
+    if (h->opts.precond == CG_PRECOND_LEARNED) return learn_kernel_name(h);
+    switch (solve_path(h)) {
+        case SolvePath::cluster: return "cg_cluster_kernel/int";
+        case SolvePath::ring: return "cg_ring_kernel/int";
+        case SolvePath::irring: return "cg_irring_kernel";
+        case SolvePath::sell: return h->fixed_vals ? "cg_sell_kernel/int" : "cg_sell_kernel/fp64";
+        case SolvePath::sellmem: return "cg_sellmem_kernel/fp64";
+        case SolvePath::irsell: return "cg_irsell_kernel";
+        case SolvePath::tiled_ir: return "cg_ir_kernel";
+        case SolvePath::tiled: break;
+    }
+    return "cg_solve_kernel/fp64";
 }
 
 void cg_destroy(cg_handle *h) { free_handle(h); }

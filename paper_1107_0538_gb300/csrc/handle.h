@@ -130,6 +130,8 @@ int enqueue_fp64_solve(cg_handle *h, const double *b, double *x, double tol, int
 int enqueue_spmv(cg_handle *h, const double *x, double *y);
 // Flexible CG with the learned preconditioner (learn.cu).
 int learn_solve(cg_handle *h, const double *b, double *x, double tol, int32_t maxit, cg_info *info);
+// The kernel that multiplies with A in flexible CG, "" without a net (learn.cu).
+const char *learn_kernel_name(const cg_handle *h);
 // Frees the learned-preconditioner workspace of a handle (learn.cu).
 void learn_free(cg_handle *h);
 // Index faults counted by the bounds-check build in batch.cu and learn.cu

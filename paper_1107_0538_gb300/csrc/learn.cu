@@ -2383,6 +2383,11 @@ int max_ctas(const cg_learn_set *set) {
 
 long long gbcg::bounds_faults_learn() { return read_bounds_faults(); }
 
+const char *gbcg::learn_kernel_name(const cg_handle *h) {
+    if (!h->learn) return "";
+    return h->learn->fused ? "fcg_sell_kernel" : "fcg_spmv_kernel";
+}
+
 void gbcg::learn_free(cg_handle *h) {
     if (h && h->learn) {
         free_ctx(h->learn);

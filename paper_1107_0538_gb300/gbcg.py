@@ -29,7 +29,7 @@ CG_VALUES_FP64, CG_VALUES_FP32, CG_VALUES_BF16 = 0, 1, 2
 
 # Every entry point of include/gbcg.h (checked against the header by the tests).
 EXPORTS = ("cg_version", "cg_opts_default", "cg_create", "cg_solve", "cg_solve_host",
-           "cg_spmv", "cg_spmv_inner", "cg_get_plan", "cg_destroy", "cg_strerror", "cg_bounds_faults", "cg_fp64_peak",
+           "cg_spmv", "cg_spmv_inner", "cg_get_plan", "cg_kernel_name", "cg_batch_kernel_name", "cg_destroy", "cg_strerror", "cg_bounds_faults", "cg_fp64_peak",
            "cg_solve_noalloc",
            "cg_batch_create", "cg_batch_enqueue", "cg_batch_results", "cg_batch_solve",
            "cg_batch_tune", "cg_batch_set_tuning", "cg_batch_destroy", "cg_net_create", "cg_net_get_params",
@@ -128,6 +128,9 @@ def lib() -> ctypes.CDLL:
             L.cg_spmv_inner.restype = ctypes.c_int
             L.cg_get_plan.argtypes = [vp, ctypes.POINTER(cg_plan)]
             L.cg_get_plan.restype = ctypes.c_int
+            for name in ("cg_kernel_name", "cg_batch_kernel_name"):
+                getattr(L, name).argtypes = [vp]
+                getattr(L, name).restype = ctypes.c_char_p
             L.cg_destroy.argtypes = [vp]
             L.cg_destroy.restype = None
             L.cg_strerror.argtypes = [ctypes.c_int]
@@ -229,6 +232,14 @@ def cg_get_plan(h: int) -> cg_plan:
     if rc:
         raise GbcgError(rc, "cg_get_plan")
     return p
+
+
+def cg_kernel_name(h: int | None) -> str:
+    return lib().cg_kernel_name(ctypes.c_void_p(h or 0)).decode()
+
+
+def cg_batch_kernel_name(h: int | None) -> str:
+    return lib().cg_batch_kernel_name(ctypes.c_void_p(h or 0)).decode()
 
 
 def cg_destroy(h: int | None) -> None:
@@ -337,6 +348,10 @@ class Solver:
     def plan(self) -> dict:
         return cg_get_plan(self.h).as_dict()
 
+    def kernel(self) -> str:
+        """The kernel its solves run (``cg_kernel_name``)."""
+        return cg_kernel_name(self.h)
+
     def close(self) -> None:
         if getattr(self, "h", None):
             cg_destroy(self.h)
@@ -442,6 +457,9 @@ class BatchSolver:
 
     def results(self, nrhs: int):
         return cg_batch_results(self.h, self.nsys, nrhs)
+
+    def kernel(self) -> str:
+        return cg_batch_kernel_name(self.h)
 
     def tune(self, B, X, tol: float):
         return cg_batch_tune(self.h, B.data_ptr(), X.data_ptr(), B.shape[0], tol)

@@ -1,0 +1,131 @@
+"""Which kernel a handle's solves run (cg_kernel_name, cg_batch_kernel_name), on
+both sides of the limits by which it is picked.  Every kernel falls back to
+another correct one, so the tests that compare solutions would not notice a
+kernel that is never picked; the matrices they use are named here with the
+kernel they mean to reach."""
+import numpy as np
+import pytest
+
+import test_fixed
+import test_gpu_batch_ring
+import test_gpu_cluster
+import test_gpu_ring
+from paper_1107_0538_gb300 import gbcg, problems
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FP32, BF16 = dict(inner_values=gbcg.CG_VALUES_FP32), dict(inner_values=gbcg.CG_VALUES_BF16)
+MEM = dict(vectors_in_memory=True)
+fixed, ring, cluster, batch = test_fixed.CASES, test_gpu_ring.CASES, test_gpu_cluster.CASES, test_gpu_batch_ring.CASES
+
+
+@pytest.fixture(scope="module", autouse=True)
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return torch.device("cuda:0")
+
+
+def box(ex, ey, ez):
+    return test_gpu_ring.box(ex, ey, ez)
+
+
+def scaled_rows(spread):
+    """Band matrix whose diagonal spans a factor of spread (a power of two), in two steps."""
+    A = test_fixed.banded(600, 7, 8)
+    s = np.where(np.arange(A.n) < 300, 1.0, spread ** 0.5)
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    d = A.to_dense().diagonal()
+    v = A.vals / np.sqrt(d[rows] * d[A.colidx]) * 1.5   # diagonal 1.5: its exponent is away from a rounding edge
+    return problems.CSR(A.n, A.rowptr, A.colidx, v * s[rows] * s[A.colidx])
+
+
+def row_sum(total):
+    """Diagonal 1 and 30 equal off-diagonals in the inner rows, |row| summing to total there."""
+    A = test_fixed.banded(600, 31, 9)
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    return problems.CSR(A.n, A.rowptr, A.colidx, np.where(rows == A.colidx, 1.0, -(total - 1.0) / 30.0))
+
+
+def negative_diagonal():
+    A = test_fixed.banded(600, 7, 8)
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    return problems.CSR(A.n, A.rowptr, A.colidx, np.where((rows == 17) & (A.colidx == 17), -A.vals, A.vals))
+
+
+# name: (matrix, options, kernel)
+CASES = {
+    # one cluster, the slices of the grid, the ring, by size
+    "box8": (lambda: box(8, 8, 8), {}, "cg_cluster_kernel/int"),
+    "box8_jacobi": (lambda: box(8, 8, 8), dict(precond=1), "cg_cluster_kernel/int"),
+    "box20": (lambda: box(20, 20, 20), {}, "cg_cluster_kernel/int"),
+    "box24": (cluster["24cube"], {}, "cg_sell_kernel/int"),
+    "box50": (lambda: box(50, 50, 50), {}, "cg_sell_kernel/int"),
+    "chip": (ring["chip"][0], {}, "cg_ring_kernel/int"),
+    "box60": (lambda: box(60, 60, 60), dict(precond=1), "cg_ring_kernel/int"),
+    # windows of a cluster's CTAs that fit, and that do not
+    "513_rows": (cluster["17_slices"], {}, "cg_cluster_kernel/int"),
+    "flat": (cluster["flat_box"], {}, "cg_cluster_kernel/int"),
+    # a given CTA count asks for the grid
+    "box8_grid": (lambda: box(8, 8, 8), dict(grid_ctas=152), "cg_sell_kernel/int"),
+    "two_ctas": (ring["two_ctas"][0], dict(grid_ctas=2), "cg_ring_kernel/int"),
+    "one_cta": (ring["one_cta"][0], dict(grid_ctas=1), "cg_ring_kernel/int"),
+    # limits of the integer product
+    "width33": (fixed["width33"][0], dict(grid_ctas=152), "cg_sell_kernel/fp64"),
+    "width33_ring": (fixed["width33"][0], dict(grid_ctas=1), "cg_sellmem_kernel/fp64"),
+    "far32767": (fixed["far32767"][0], {}, "cg_sell_kernel/int"),
+    "far32768": (fixed["far32768"][0], {}, "cg_sell_kernel/fp64"),
+    "scaled": (fixed["scaled"][0], dict(grid_ctas=152), "cg_sell_kernel/int"),
+    "scaled_wide": (fixed["scaled_wide"][0], dict(grid_ctas=152), "cg_sell_kernel/fp64"),
+    "spread24": (lambda: scaled_rows(2.0 ** 24), dict(grid_ctas=152), "cg_sell_kernel/int"),
+    "spread26": (lambda: scaled_rows(2.0 ** 26), dict(grid_ctas=152), "cg_sell_kernel/fp64"),
+    "sum64.1": (lambda: row_sum(64.1), dict(grid_ctas=152), "cg_sell_kernel/fp64"),
+    "negative": (negative_diagonal, {}, "cg_sell_kernel/fp64"),
+    # repeated columns and too many offsets leave the ring
+    "repeats": (ring["repeats"][0], dict(grid_ctas=2), "cg_sellmem_kernel/fp64"),
+    "memory": (lambda: box(8, 8, 8), MEM, "cg_solve_kernel/fp64"),
+    # refinement
+    "fp32": (lambda: box(8, 8, 8), FP32, "cg_irring_kernel"),
+    "bf16": (lambda: box(8, 8, 8), dict(precond=1, **BF16), "cg_irring_kernel"),
+    "fp32_mid": (ring["chip"][0], FP32, "cg_irring_kernel"),
+    "fp32_repeats": (lambda: test_gpu_ring.with_repeats(box(8, 8, 8)), FP32, "cg_irsell_kernel"),
+    "bf16_width33": (fixed["width33"][0], BF16, "cg_irsell_kernel"),
+    "fp32_repeats_two_ctas": (ring["repeats"][0], dict(grid_ctas=2, **FP32), "cg_ir_kernel"),
+    "fp32_memory": (lambda: box(8, 8, 8), dict(**FP32, **MEM), "cg_ir_kernel"),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_solve_kernel(name):
+    make, kw, want = CASES[name]
+    with gbcg.Solver(make(), **kw) as s:
+        assert s.kernel() == want
+
+
+@pytest.mark.parametrize("name,want", [("ragged", "offsets"), ("many_tiles", "offsets"), ("31_offsets", "offsets"),
+                                       ("33_offsets", "staged"), ("repeats", "staged")])
+@pytest.mark.parametrize("values", [gbcg.CG_VALUES_FP32, gbcg.CG_VALUES_BF16], ids=["fp32", "bf16"])
+def test_batch_kernel(name, want, values):
+    with gbcg.BatchSolver(batch[name](), inner_values=values, precond=1) as bs:
+        assert bs.kernel() == "cg_batch_kernel/" + want
+        for gather, lanes, static in ((1, 1, 0), (0, 2, 0), (0, 4, 1)):
+            bs.set_tuning(1e-3, gather, lanes, static)
+            assert bs.kernel() == "cg_batch_kernel/staged"
+        bs.set_tuning(1e-3, 0, 1, 1)
+        assert bs.kernel() == "cg_batch_kernel/" + want
+
+
+def test_learned_kernel():
+    inst = problems.learn_instance(8, 20001)
+    net = gbcg.Net(problems.learn_init_params())
+    for kw, want in (({}, "fcg_sell_kernel"), (MEM, "fcg_spmv_kernel")):
+        with gbcg.Solver(inst.A, precond=gbcg.CG_PRECOND_LEARNED, **kw) as s:
+            assert s.kernel() == ""
+            s.set_learned(net, inst.grid, inst.lognu.astype(np.float32))
+            assert s.kernel() == want
+    net.close()
+
+
+def test_no_handle():
+    assert gbcg.cg_kernel_name(None) == "" and gbcg.cg_batch_kernel_name(None) == ""
