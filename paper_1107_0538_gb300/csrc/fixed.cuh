@@ -16,7 +16,7 @@
 //            whole vector; Z_j = z1 2^30 + z0, |z0| <= 2^29
 //   row      (A z)_i = 2^(c_i - u - S) sum_j A_ij Z_j
 // The products with a0 are at most 2^58 each and those with a1 at most 2^29
-// times a row sum of 2^33, so a row of up to kFixedMaxWidth = 31 entries stays
+// times a row sum of 2^33, so a row of up to kFixedMaxWidth = 31 nonzeros stays
 // below 2^63 in each of the four 64-bit accumulators: the sum is exact.  The
 // scaling by the diagonal's roots makes every entry of an SPD matrix at most
 // about 1 in these units, at material interfaces too.
@@ -34,7 +34,7 @@
 // 47e-13).  With A_ij cut at 57 bits they were up to 100 times further: its
 // rounding is the same in every iteration.
 //
-// A matrix with a row of more than 31 entries, a column more than 32767 rows
+// A matrix with a row of more than 31 nonzeros, a column more than 32767 rows
 // away, a diagonal entry that is not positive, a row whose entries sum to more
 // than 64 in the scaled units, or a diagonal outside 2^+-200 or spread over
 // more than a factor of 2^24 (where the one shift of the whole vector would

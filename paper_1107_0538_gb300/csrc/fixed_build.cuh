@@ -17,14 +17,17 @@ __global__ void __launch_bounds__(256) fixed_scale_kernel(SellMatrix M, int8_t *
     const long long a = M.ptr[t];
     const int w = (int)((M.ptr[t + 1] - a) >> 5);
     double d = 0.0;
+    int m = 0;   // products that can be other than zero: the slice's width also counts padding
     for (int k = 0; k < w; ++k) {
         const long long i = a + 32LL * k + lane;
         const int col = M.cols16 ? row + M.cols16[i] : M.cols32[i];
-        if (col == row) d += M.vals[i];   // padding adds zeros
+        const double v = M.vals[i];
+        if (col == row) d += v;
+        m += v != 0.0;
     }
     const int e = (int)((unsigned long long)__double_as_longlong(d) >> 52);   // with the sign bit
     const int ci = (e - 1023 + 1) >> 1;
-    if (w > kFixedMaxWidth || e == 0 || e >= 2047 || ci > kFixedMaxC || ci < -kFixedMaxC) {
+    if (m > kFixedMaxWidth || e == 0 || e >= 2047 || ci > kFixedMaxC || ci < -kFixedMaxC) {
         atomicOr(flags, 1u);
         c[row] = 0;
         return;

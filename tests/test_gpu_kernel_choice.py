@@ -71,7 +71,9 @@ CASES = {
     "box8_grid": (lambda: box(8, 8, 8), dict(grid_ctas=152), "cg_sell_kernel/int"),
     "two_ctas": (ring["two_ctas"][0], dict(grid_ctas=2), "cg_ring_kernel/int"),
     "one_cta": (ring["one_cta"][0], dict(grid_ctas=1), "cg_ring_kernel/int"),
+    "ten_ctas": (lambda: box(20, 20, 20), dict(grid_ctas=10), "cg_sell_kernel/int"),
     # limits of the integer product
+    "width31": (fixed["width31"][0], dict(grid_ctas=152), "cg_sell_kernel/int"),
     "width33": (fixed["width33"][0], dict(grid_ctas=152), "cg_sell_kernel/fp64"),
     "width33_ring": (fixed["width33"][0], dict(grid_ctas=1), "cg_sellmem_kernel/fp64"),
     "far32767": (fixed["far32767"][0], {}, "cg_sell_kernel/int"),
@@ -80,6 +82,7 @@ CASES = {
     "scaled_wide": (fixed["scaled_wide"][0], dict(grid_ctas=152), "cg_sell_kernel/fp64"),
     "spread24": (lambda: scaled_rows(2.0 ** 24), dict(grid_ctas=152), "cg_sell_kernel/int"),
     "spread26": (lambda: scaled_rows(2.0 ** 26), dict(grid_ctas=152), "cg_sell_kernel/fp64"),
+    "sum63.9": (lambda: row_sum(63.9), dict(grid_ctas=152), "cg_sell_kernel/int"),
     "sum64.1": (lambda: row_sum(64.1), dict(grid_ctas=152), "cg_sell_kernel/fp64"),
     "negative": (negative_diagonal, {}, "cg_sell_kernel/fp64"),
     # repeated columns and too many offsets leave the ring
