@@ -98,8 +98,10 @@ typedef struct {
     int32_t vectors_in_memory; /* 0 (default): FP64 solves run the SELL-32 kernels,
                                 which keep the vectors of systems with at most one
                                 32-row slice per warp in registers for the whole
-                                solve; 1: the tiled kernel, every vector in device
-                                memory                                            */
+                                solve, or, for long rows in systems of up to four
+                                rows per thread, the tiled kernel with its rows in
+                                registers; 1: the tiled kernel, every vector in
+                                device memory                                    */
     int32_t inner_values;    /* CG_VALUES_*; default CG_VALUES_FP64.  FP32/BF16
                                 turn the solve into iterative refinement: the
                                 outer loop keeps x and r = b - A x in FP64 with
@@ -144,9 +146,10 @@ typedef struct {
     int32_t smem_bytes;      /* dynamic shared memory per CTA                     */
     int32_t lanes_per_row;   /* threads that share one row in the SpMV            */
     int32_t l2_evict_first;  /* 1 when the matrix stream is marked evict-first    */
-    int32_t reg_rows;        /* rows per thread if each thread of the tiled plan
-                                held its rows in registers: 1, 2 or 4; 0: more, or
-                                vectors_in_memory                                 */
+    int32_t reg_rows;        /* rows per thread of the tiled plan, rounded up to 1,
+                                2 or 4: cg_solve_kernel then holds their vectors in
+                                registers (for systems that it solves); 0: more than
+                                4, or vectors_in_memory                          */
     int32_t window_tiles;    /* tiles whose gathers read a staged x-window        */
     int64_t device_bytes;    /* device memory the handle owns                     */
     int32_t slice_solve;     /* how the SELL-32 slices are shared out: 1 at most one

@@ -526,11 +526,13 @@ __device__ __forceinline__ bool warp_tile(const Params &P, const Smem &S, Pipe &
 // Row sums of this CTA's rows: epi.row(i, sum_k vals[k] * x[colidx[k]], j)
 // is called once per row by the thread that owns it; VT is the stored value
 // type, XT the vector element type (x 16-byte aligned), AT the accumulation
-// type.  `one_pass` stops the pipeline at the end of the pass; otherwise the
-// next pass's first tile is left in flight (matrix part only, same value
-// type).  Returns false in every thread of the CTA if a TMA wait ran out (the
-// error is recorded).
-template <class VT, class XT, class AT, class Epi>
+// type.  RPT > 0 unrolls the warp's tile loop (at most RPT tiles per warp)
+// so that j is a compile-time index into register-resident row state;
+// RPT = 0 loops at run time.  `one_pass` stops the pipeline at the end of
+// the pass; otherwise the next pass's first tile is left in flight (matrix
+// part only, same value type).  Returns false in every thread of the CTA if
+// a TMA wait ran out (the error is recorded).
+template <class VT, class XT, class AT, int RPT = 0, class Epi>
 __device__ __forceinline__ bool spmv_tiles(const Params &P, const Smem &S, Pipe &pp, const VT *vals,
                                            const XT *x, Epi &epi, bool one_pass = false) {
     const int t0 = P.cta_tile[blockIdx.x], t1 = P.cta_tile[blockIdx.x + 1];
@@ -548,8 +550,16 @@ __device__ __forceinline__ bool spmv_tiles(const Params &P, const Smem &S, Pipe 
             ++pp.win_issued;
         }
         issue_next<VT, XT>(P, S, pp, t0, m, limit, pass_end, vals, x);
-        for (int j = 0; j < m && !failed; ++j)
-            failed = !warp_tile<VT, XT, AT>(P, S, pp, t0, m, limit, pass_end, vals, x, epi, j);
+        if (RPT > 0) {
+#pragma unroll
+            for (int j = 0; j < (RPT > 0 ? RPT : 1); ++j) {
+                if (j < m && !failed)
+                    failed = !warp_tile<VT, XT, AT>(P, S, pp, t0, m, limit, pass_end, vals, x, epi, j);
+            }
+        } else {
+            for (int j = 0; j < m && !failed; ++j)
+                failed = !warp_tile<VT, XT, AT>(P, S, pp, t0, m, limit, pass_end, vals, x, epi, j);
+        }
     }
     if (__syncthreads_or(failed)) {
         if (threadIdx.x == 0) set_error(P.st, CG_ETIMEOUT, 2);

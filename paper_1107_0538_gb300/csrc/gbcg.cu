@@ -49,6 +49,19 @@ static_assert(sizeof(I4) == sizeof(int4), "tile descriptor layout");
 
 namespace {
 
+// ------------------------------------------------------------ row state
+// With RPT > 0 every thread keeps the vector entries of the rows it owns
+// (lane l of warp w owns row r0 + l of each of the warp's tiles) in
+// registers for the whole solve: x, r, z, p, q and 1/diag never round-trip
+// through memory; only p is published (the SpMV gathers it) and x is written
+// at the end.  RPT = 0 keeps every vector in global memory.
+template <int RPT>
+struct RegRows {
+    int row[RPT > 0 ? RPT : 1];
+    double x[RPT > 0 ? RPT : 1], r[RPT > 0 ? RPT : 1], z[RPT > 0 ? RPT : 1];
+    double p[RPT > 0 ? RPT : 1], q[RPT > 0 ? RPT : 1], dinv[RPT > 0 ? RPT : 1];
+};
+
 // ------------------------------------------------------------ epilogues
 struct EpiSetup {       // r = b - A x0, z = M^-1 r (gathered), p = z, q = 0; sums r.r, r.z, b.b
     const double *b;
@@ -78,6 +91,28 @@ struct EpiSetup {       // r = b - A x0, z = M^-1 r (gathered), p = z, q = 0; su
     }
 };
 
+template <int RPT>
+struct RegSetup {       // the same, into registers (p is also published)
+    RegRows<RPT> &R;
+    const double *b;
+    double *p;
+    int precond;
+    double rr = 0.0, rz = 0.0, bb = 0.0;
+    __device__ __forceinline__ void row(int i, double ax, int j) {
+        const double bi = b[i];
+        const double ri = bi - ax;
+        const double zi = precond ? R.dinv[j] * ri : ri;
+        R.r[j] = ri;
+        R.z[j] = zi;
+        R.p[j] = zi;
+        R.q[j] = 0.0;
+        p[i] = zi;
+        rr = fma(ri, ri, rr);
+        rz = fma(ri, zi, rz);
+        bb = fma(bi, bi, bb);
+    }
+};
+
 struct EpiIter {        // p = z + beta p, q = A z + beta q; sum p . q
     double *q;
     double *pd;
@@ -95,6 +130,20 @@ struct EpiIter {        // p = z + beta p, q = A z + beta q; sum p . q
         const double pi = fma(beta, pi_, zi_);
         q[i] = qi;
         pd[i] = pi;
+        pq = fma(pi, qi, pq);
+    }
+};
+
+template <int RPT>
+struct RegIter {
+    RegRows<RPT> &R;
+    double beta;
+    double pq = 0.0;
+    __device__ __forceinline__ void row(int, double az, int j) {
+        const double qi = fma(beta, R.q[j], az);
+        const double pi = fma(beta, R.p[j], R.z[j]);
+        R.q[j] = qi;
+        R.p[j] = pi;
         pq = fma(pi, qi, pq);
     }
 };
@@ -125,6 +174,7 @@ constexpr int kCtlShift = 4;     // fixed-point shift of the published z
 // Scalar recurrences (alpha, beta, the stop test) run in thread 0 only: on
 // GB300 an FP64 divide or square root executed by every warp would cost the
 // FP64 pipe as much as a tile of the SpMV.
+template <int RPT>
 __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const Smem S = carve_smem(smem_raw);
@@ -140,13 +190,41 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
     // thread 0's scalar state
     int status = CG_OK, iters = 0;
     double rr = 0.0, bb = 0.0, true_rr = -1.0, rho = 0.0, bnorm = 0.0;
+    RegRows<RPT> R;
+    if constexpr (RPT > 0) {
+        const int t0 = P.cta_tile[blockIdx.x], nt = P.cta_tile[blockIdx.x + 1] - t0;
+        const int w = tid >> 5, lane = tid & 31;
+#pragma unroll
+        for (int j = 0; j < RPT; ++j) {
+            R.row[j] = -1;
+            R.x[j] = 0.0;
+            R.dinv[j] = 1.0;
+            const int t = w + kWarps * j;
+            if (t < nt) {
+                const TileDesc d = load_desc(P, t0 + t);
+                const int row = d.r0 + lane;
+                if (row < d.r1) {
+                    R.row[j] = row;
+                    R.x[j] = P.x[row];
+                    if (P.precond) R.dinv[j] = P.dinv[row];
+                }
+            }
+        }
+    }
+
     // ---- setup: r0 = b - A x0, z0 = M^-1 r0, p0 = z0; r.r, r.z, b.b
     bool run;
     {
         double v[3];
-        EpiSetup epi{P.b, P.r, P.z, p, P.pd, P.q, P.dinv, P.precond};
-        if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, epi)) goto out;
-        v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
+        if constexpr (RPT > 0) {
+            RegSetup<RPT> epi{R, P.b, p, P.precond};
+            if (!spmv_tiles<double, double, double, RPT>(P, S, pipe, P.vals, P.x, epi)) goto out;
+            v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
+        } else {
+            EpiSetup epi{P.b, P.r, P.z, p, P.pd, P.q, P.dinv, P.precond};
+            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, epi)) goto out;
+            v[0] = epi.rr; v[1] = epi.rz; v[2] = epi.bb;
+        }
         block_sum<3>(v, S);
         publish_partials<3>(P, set, v);
         if (!grid_barrier(P, epoch, S)) goto out;
@@ -178,8 +256,14 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         }
         __syncthreads();
         run = S.ctl[kCtlRun] != 0;
-        if (S.ctl[kCtlZeroB])  // b = 0: the solution is x = 0
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) P.x[i] = 0.0;
+        if (S.ctl[kCtlZeroB]) {  // b = 0: the solution is x = 0
+            if constexpr (RPT > 0) {
+#pragma unroll
+                for (int j = 0; j < RPT; ++j) R.x[j] = 0.0;
+            } else {
+                for (int i = row_lo + tid; i < row_hi; i += kThreads) P.x[i] = 0.0;
+            }
+        }
     }
 
     // ---- the CG loop
@@ -188,9 +272,17 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         double beta = 0.0;  // p_1 = z_0 and q_1 = A z_0
         for (int k = 1; k <= P.maxit; ++k) {
             // phase A: p = z + beta p, q = A z + beta q (= A p), p . q
-            EpiIter ei{P.q, P.pd, p, beta};
-            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, p, ei)) goto out;
-            double v1[1] = {ei.pq};
+            double pq;
+            if constexpr (RPT > 0) {
+                RegIter<RPT> ei{R, beta};
+                if (!spmv_tiles<double, double, double, RPT>(P, S, pipe, P.vals, p, ei)) goto out;
+                pq = ei.pq;
+            } else {
+                EpiIter ei{P.q, P.pd, p, beta};
+                if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, p, ei)) goto out;
+                pq = ei.pq;
+            }
+            double v1[1] = {pq};
             block_sum<1>(v1, S);
             publish_partials<1>(P, set, v1);
             if (!grid_barrier(P, epoch, S)) goto out;
@@ -213,18 +305,37 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
             // phase B: x += alpha p, r -= alpha q, z = dinv r (published for
             // the next SpMV: every gather of phase A is over); r.r, r.z
             double prr = 0.0, prz = 0.0;
-            for (int i = row_lo + tid; i < row_hi; i += kThreads) {
-                const double pi = P.pd[i], qi = P.q[i], xi = P.x[i], ri0 = P.r[i];
-                P.x[i] = fma(alpha, pi, xi);
-                const double ri = fma(-alpha, qi, ri0);
-                P.r[i] = ri;
-                prr = fma(ri, ri, prr);
-                double zi = ri;
-                if (P.precond) {
-                    zi = P.dinv[i] * ri;
-                    prz = fma(ri, zi, prz);
+            if constexpr (RPT > 0) {
+#pragma unroll
+                for (int j = 0; j < RPT; ++j) {
+                    if (R.row[j] >= 0) {
+                        R.x[j] = fma(alpha, R.p[j], R.x[j]);
+                        const double ri = fma(-alpha, R.q[j], R.r[j]);
+                        R.r[j] = ri;
+                        prr = fma(ri, ri, prr);
+                        double zi = ri;
+                        if (P.precond) {
+                            zi = R.dinv[j] * ri;
+                            prz = fma(ri, zi, prz);
+                        }
+                        R.z[j] = zi;
+                        p[R.row[j]] = zi;
+                    }
                 }
-                p[i] = zi;
+            } else {
+                for (int i = row_lo + tid; i < row_hi; i += kThreads) {
+                    const double pi = P.pd[i], qi = P.q[i], xi = P.x[i], ri0 = P.r[i];
+                    P.x[i] = fma(alpha, pi, xi);
+                    const double ri = fma(-alpha, qi, ri0);
+                    P.r[i] = ri;
+                    prr = fma(ri, ri, prr);
+                    double zi = ri;
+                    if (P.precond) {
+                        zi = P.dinv[i] * ri;
+                        prz = fma(ri, zi, prz);
+                    }
+                    p[i] = zi;
+                }
             }
             double t2[2];
             if (P.precond) {
@@ -266,15 +377,23 @@ __global__ void __launch_bounds__(kThreads, 1) cg_solve_kernel(Params P) {
         }
     }
 
-    // ---- the true residual ||b - A x||
+    // ---- publish x (register mode), then the true residual ||b - A x||
+    if constexpr (RPT > 0) {
+#pragma unroll
+        for (int j = 0; j < RPT; ++j)
+            if (R.row[j] >= 0) P.x[R.row[j]] = R.x[j];
+    }
     {
         if (tid == 0) S.ctl[kCtlTrue] = (P.true_res && status != CG_ENAN && bb != 0.0) ? 1 : 0;
         __syncthreads();
         const bool want_true = S.ctl[kCtlTrue] != 0;
         if (tid == 0 && P.true_res && status != CG_ENAN && bb == 0.0) true_rr = 0.0;
         if (want_true) {
+            if constexpr (RPT > 0) {
+                if (!grid_barrier(P, epoch, S)) goto out;  // every x entry is written
+            }
             EpiTrue et{P.b};
-            if (!spmv_tiles<double, double, double>(P, S, pipe, P.vals, P.x, et)) goto out;
+            if (!spmv_tiles<double, double, double, RPT>(P, S, pipe, P.vals, P.x, et)) goto out;
             double v[1] = {et.acc};
             block_sum<1>(v, S);
             publish_partials<1>(P, set, v);
@@ -1350,6 +1469,10 @@ bool prepare_solve_kernels(const void *(*kernel_for)(bool, bool), bool *resident
 }
 
 constexpr int kRptChoices[] = {1, 2, 4};   // cg_plan.reg_rows
+using SolveKernel = void (*)(Params);
+// The tiled kernel with up to four rows of a thread in registers, or none:
+// systems of one or two rows per thread run the slice kernel.
+SolveKernel solve_kernel_for(int rpt) { return rpt > 0 ? cg_solve_kernel<4> : cg_solve_kernel<0>; }
 
 }  // namespace
 
@@ -1639,7 +1762,7 @@ int enqueue_solve(cg_handle *h, const double *b, double *x, double tol, int32_t 
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kSellSolveThreads), args, 0, h->stream);
         } else {
             void *args[] = {&P};
-            const void *kern = (const void *)cg_solve_kernel;
+            const void *kern = (const void *)solve_kernel_for(h->rpt);
             if (h->opts.inner_values == CG_VALUES_FP32) kern = (const void *)cg_ir_kernel<float>;
             if (h->opts.inner_values == CG_VALUES_BF16) kern = (const void *)cg_ir_kernel<__nv_bfloat16>;
             e = cudaLaunchCooperativeKernel(kern, dim3(h->ctas), dim3(kThreads),
@@ -1869,8 +1992,10 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
     h->max_tile_nnz = max_tile;
     int sms = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return fail(CG_ECUDA);
-    if (cudaFuncSetAttribute((const void *)cg_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) !=
-            cudaSuccess ||
+    if (cudaFuncSetAttribute((const void *)cg_solve_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute((const void *)cg_solve_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmemBytes) != cudaSuccess ||
         cudaFuncSetAttribute((const void *)sell_spmv_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxL1) != cudaSuccess ||
         cudaFuncSetAttribute((const void *)cg_ir_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1882,7 +2007,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         cudaFuncSetAttribute((const void *)lo_spmv_tiles_kernel<__nv_bfloat16>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess)
         return fail(CG_ECUDA);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_solve_kernel, kThreads, kSmemBytes) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_kernel_for(4), kThreads, kSmemBytes) !=
             cudaSuccess ||
         per_sm < 1)
         return fail(CG_ECUDA);
@@ -1993,9 +2118,9 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
             }
         }
         // larger systems: the SELL-32 kernel with the vectors in memory, slices
-        // in contiguous ranges per CTA (at n = 161820, Jacobi-PCG: 22.2 us per
-        // iteration, 18.6 with the fixed-point product, where the tiled kernel
-        // with its rows in registers took 26.0)
+        // in contiguous ranges per CTA (a Q1 box of 161820 rows, Jacobi-PCG: 22.2 us
+        // per iteration, where the tiled kernel with its rows in registers took
+        // 26.0; long rows: see below)
         if (!h->sell_solve && !opts.vectors_in_memory && n > 0) {
             const std::vector<int32_t> mcut = split_slices(sh.ptr, ctas, h->sell_slices, kSliceVecCost);
             bool resident = false;
@@ -2040,6 +2165,11 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                 return r == CG_OK && ok ? build_ring<int2>(h, k, 2, tot, max_slices, l2) : r;
             });
             if (rc != CG_OK) return fail(rc);
+            // long rows without a ring: the tiled kernel, its rows in registers
+            if (!h->ring_blob && h->rpt > 0 && sell_walks_long_rows(sh.ptr, nnz, opts.precond != CG_PRECOND_NONE, l2)) {
+                h->sell_mem = 0;
+                h->sell_cut = nullptr;   // flexible CG too
+            }
         } else if ((h->sell_solve || h->sell_mem) && mixed) {
             const void *k32[] = {(const void *)cg_irring_kernel<float>, (const void *)lo_spmv_ring_kernel<float>};
             const void *k16[] = {(const void *)cg_irring_kernel<__nv_bfloat16>,

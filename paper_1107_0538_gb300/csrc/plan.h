@@ -477,6 +477,26 @@ inline SellHost build_sell(int32_t n, const std::vector<int32_t> &rowptr, const 
     return S;
 }
 
+// Whether long rows make SELL-32 with the vectors in memory the slower choice
+// for a system of at most four rows per thread, whose other choice is the tiled
+// kernel (it gives a long row to 32 lanes and pads nothing).  One warp walks all
+// of a wide slice while the others wait at the grid barrier; with the Jacobi
+// vectors, padding also costs where it takes the matrix past half of the L2.
+// us per iteration, SELL-32 / tiled with rows in registers:
+//   widest slice, rows of 26 entries (161820): 87 wide 24.5 / 26.2, Jacobi 26.6 /
+//   27.8; 147 32.3 / 30.8, 35.0 / 32.4; 527 81.3 / 61.4, 89.3 / 62.9; 9027 1280 / 43;
+//   rows of 5 entries (160000): 65 20.8 / 22.8, 125 29.1 / 27.8; 245 45.1 / 36.6;
+//   rows of 6 (300000): 125 33.3 / 34.6, Jacobi 36.3 / 36.2
+//   padding, Jacobi: 1.81 times the entries, 16 MB 16.9 / 22.0; 1.37 times, 60 MB
+//   25.8 / 29.7; 1.60 times, 70 MB 50.1 / 39.6; 1.67 times, 85 MB 36.5 / 33.7 (plain 28.9 /
+//   32.1); 1.85 times, 147 MB 59.7 / 58.7 (plain 53.8 / 57.2)
+inline bool sell_walks_long_rows(const std::vector<long long> &ptr, int64_t nnz, bool precond, int64_t l2_bytes) {
+    long long widest = 0;   // entries of the widest slice
+    for (size_t t = 0; t + 1 < ptr.size(); ++t) widest = std::max(widest, ptr[t + 1] - ptr[t]);
+    const double padded = (double)ptr.back();
+    return widest > 32 * 120 || (precond && padded > 1.5 * (double)nnz && 10.0 * padded > 0.5 * (double)l2_bytes);
+}
+
 // Plan of the one-cluster solve (cluster.cuh): contiguous slice ranges for up
 // to kClusterMaxCtas CTAs, a warp per slice and one control warp each, and the
 // window of rows every CTA's columns lie in.  Shared memory per CTA: 8 + 2

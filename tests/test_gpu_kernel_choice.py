@@ -6,6 +6,7 @@ kernel they mean to reach."""
 import numpy as np
 import pytest
 
+import oracle
 import test_fixed
 import test_gpu_batch_ring
 import test_gpu_cluster
@@ -54,6 +55,20 @@ def negative_diagonal():
     return problems.CSR(A.n, A.rowptr, A.colidx, np.where((rows == 17) & (A.colidx == 17), -A.vals, A.vals))
 
 
+def with_hub(A, m):
+    """A with row 777 coupled to m further rows, spread over the matrix, weakly enough to stay definite."""
+    rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
+    others = np.setdiff1d(np.linspace(0, A.n - 1, m + 40).astype(int), A.colidx[A.rowptr[777]:A.rowptr[778]])[:m]
+    w = np.full(m, 1e-9)
+    hub = np.full(m, 777)
+    key = np.concatenate([rows.astype(np.int64) * A.n + A.colidx, hub * A.n + others, others * A.n + hub])
+    order = np.argsort(key, kind="stable")
+    key = key[order]
+    assert np.all(np.diff(key) > 0)
+    rowptr = np.searchsorted(key, np.arange(A.n + 1, dtype=np.int64) * A.n).astype(np.int32)
+    return problems.CSR(A.n, rowptr, (key % A.n).astype(np.int32), np.concatenate([A.vals, w, w])[order])
+
+
 # name: (matrix, options, kernel)
 CASES = {
     # one cluster, the slices of the grid, the ring, by size
@@ -88,6 +103,11 @@ CASES = {
     # repeated columns and too many offsets leave the ring
     "repeats": (ring["repeats"][0], dict(grid_ctas=2), "cg_sellmem_kernel/fp64"),
     "memory": (lambda: box(8, 8, 8), MEM, "cg_solve_kernel/fp64"),
+    # a long row, which one warp of a SELL-32 slice would walk alone
+    "mid_hub120": (lambda: with_hub(box(53, 54, 55), 102), {}, "cg_sellmem_kernel/fp64"),
+    "mid_hub121": (lambda: with_hub(box(53, 54, 55), 103), {}, "cg_solve_kernel/fp64"),
+    "mid_hub2000": (lambda: with_hub(box(53, 54, 55), 2000), dict(precond=1), "cg_solve_kernel/fp64"),
+    "large_hub2000": (lambda: with_hub(box(20, 20, 20), 2000), dict(grid_ctas=1), "cg_sellmem_kernel/fp64"),
     # refinement
     "fp32": (lambda: box(8, 8, 8), FP32, "cg_irring_kernel"),
     "bf16": (lambda: box(8, 8, 8), dict(precond=1, **BF16), "cg_irring_kernel"),
@@ -104,6 +124,27 @@ def test_solve_kernel(name):
     make, kw, want = CASES[name]
     with gbcg.Solver(make(), **kw) as s:
         assert s.kernel() == want
+
+
+@pytest.mark.parametrize("precond", [0, 1])
+@pytest.mark.parametrize("edges,ctas", [((53, 54, 55), 0), ((20, 20, 20), 6), ((9, 9, 30), 3)],
+                         ids=["chip", "six_ctas", "three_ctas"])
+def test_long_row_iterates(dev, edges, ctas, precond):
+    """The tiled kernel with a thread's rows in registers, one row of 800 entries: 1e-10 from the oracle at a fixed iteration count, the bar of the
+    FP64 kernels, and a full solve's own and true residual."""
+    A = with_hub(box(*edges), 800)
+    b = problems.rhs_uniform(A.n, 31)
+    with gbcg.Solver(A, precond=precond, grid_ctas=ctas) as s:
+        assert s.kernel() == "cg_solve_kernel/fp64" and s.plan()["reg_rows"] > 0
+        for k in (1, 2, 40):
+            ref = oracle.cg(A, b, tol=0.0, maxit=k, precond=precond)
+            xt = torch.zeros(A.n, dtype=torch.float64, device=dev)
+            info = s.solve(torch.from_numpy(b).to(dev), xt, tol=0.0, maxit=k)
+            assert info.iters == k and np.linalg.norm(xt.cpu().numpy() - ref["x"]) <= 1e-10 * np.linalg.norm(ref["x"])
+        xt.zero_()
+        info = s.solve(torch.from_numpy(b).to(dev), xt, tol=1e-9)
+        true = np.linalg.norm(b - oracle.spmv(A, xt.cpu().numpy())) / np.linalg.norm(b)
+        assert info.status == gbcg.CG_OK and info.relres <= 1e-9 and true <= 1.05e-9
 
 
 @pytest.mark.parametrize("name,want", [("ragged", "offsets"), ("many_tiles", "offsets"), ("31_offsets", "offsets"),
