@@ -197,6 +197,19 @@ __device__ __forceinline__ void ring_fma(LoAcc &a, int k, const __nv_bfloat16 *v
     a.s[k & 1] = fmaf(__uint_as_float(b << 16), z, a.s[k & 1]);
 }
 
+// The same for y = A_lo x with a caller's x: a row without the slice's offset
+// holds +0 there (and no stored entry is +0, ring_build.cuh), and adds nothing
+// even where x is infinite or NaN.  The solve needs no such test: it ends at the
+// first sum that is not finite.
+struct LoAccStored : LoAcc {};
+template <class VT>
+__device__ __forceinline__ void ring_fma(LoAccStored &a, int k, const VT *v, float z) {
+    bool stored;
+    if constexpr (sizeof(VT) == 4) stored = __float_as_uint(*v) != 0u;
+    else stored = *reinterpret_cast<const unsigned short *>(v) != 0;
+    if (stored) ring_fma(static_cast<LoAcc &>(a), k, v, z);
+}
+
 // Adds the N entries at offs, vals: all gathers in flight, then the products.
 template <int N, class VT, class ZT, class Acc>
 __device__ __forceinline__ void ring_batch(const RingMatrix &R, const int *offs, const VT *vals, unsigned int rowb,
@@ -542,7 +555,7 @@ out:
 // ------------------------------------------------- mixed precision
 // The refinement of cg_irsell_kernel with its inner matrix in the ring: outer
 // residual and x in FP64 on the SELL-32 copy, inner CG in FP32 on the
-// low-precision slices (diagonal slots zero, the compensated diagonal kept
+// low-precision slices (diagonal slots -0, the compensated diagonal kept
 // apart).  zf: the inner z, padded.
 template <class VT>
 __global__ void __launch_bounds__(kSellSolveThreads, 1)
@@ -811,7 +824,7 @@ __global__ void __launch_bounds__(kSellSolveThreads, 1)
             if (lane == 0) set_error(P.st, CG_ETIMEOUT, 2);
             break;
         }
-        LoAcc acc;
+        LoAccStored acc;
         ring_sum<16, VT>(R, slot, __ldg(R.meta + t).y, row < P.n ? row : P.n - 1, zf, acc);
         const float s = acc.s[0] + acc.s[1];
         ring.release(j);

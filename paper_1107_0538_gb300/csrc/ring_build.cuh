@@ -58,7 +58,8 @@ __global__ void __launch_bounds__(256) ring_count_kernel(SellMatrix M, int32_t *
 }
 
 // Values of the slices: fixed-point integers (VT = int2), or the off-diagonals
-// rounded to nearest-even in VT (float, BF16 bits), zero on the diagonal.
+// rounded to nearest-even in VT (float, BF16 bits) and zero on the diagonal,
+// where every zero is -0: +0 marks an offset that the row does not have.
 template <class VT>
 __device__ __forceinline__ VT ring_convert(double v, int row, int off, const int8_t *c, int u);
 template <>
@@ -67,11 +68,13 @@ __device__ __forceinline__ int2 ring_convert<int2>(double v, int row, int off, c
 }
 template <>
 __device__ __forceinline__ float ring_convert<float>(double v, int, int off, const int8_t *, int) {
-    return off == 0 ? 0.0f : __double2float_rn(v);
+    const float f = off == 0 ? 0.0f : __double2float_rn(v);
+    return f == 0.0f ? -0.0f : f;
 }
 template <>
 __device__ __forceinline__ __nv_bfloat16 ring_convert<__nv_bfloat16>(double v, int, int off, const int8_t *, int) {
-    return __double2bfloat16(off == 0 ? 0.0 : v);
+    const __nv_bfloat16 f = __double2bfloat16(off == 0 ? 0.0 : v);
+    return __bfloat162float(f) == 0.0f ? __ushort_as_bfloat16(0x8000) : f;
 }
 __device__ __forceinline__ void ring_zero(int2 &v) { v = make_int2(0, 0); }
 __device__ __forceinline__ void ring_zero(float &v) { v = 0.0f; }
