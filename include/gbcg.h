@@ -507,7 +507,11 @@ typedef struct {
  * s = D^-1/2 r, sigma = rms(s), u the network output for s / sigma before
  * the final D^-1/2 scaling, e_hat = D^1/2 e / sigma; *loss receives the
  * mean over the pairs and grad (host, CG_LEARN_PARAMS floats, may be NULL)
- * its gradient.  Synchronous.
+ * its gradient.  The same call gives the same bits.  The net keeps a workspace
+ * for this grid until it trains on another or is destroyed: up to four copies of the
+ * fields of one pair (about 450 bytes per node and 19 MB each) where the device
+ * has memory for them, one at least; their number does not change the result.
+ * Synchronous.
  */
 int cg_learn_grad(cg_net *net, const cg_learn_set *set, const int64_t *pairs, int32_t count, double *loss,
                   float *grad);

@@ -21,7 +21,7 @@ ROOT = os.path.dirname(_HERE)
 SOURCES = [os.path.join(_HERE, "csrc", f) for f in ("gbcg.cu", "noalloc.cu", "batch.cu", "learn.cu")]
 DEPS = SOURCES + [os.path.join(_HERE, "csrc", f) for f in ("cg_device.cuh", "layout.h", "plan.h", "lowprec.h",
                                                            "handle.h", "cluster.cuh", "fixed.cuh", "fixed_build.cuh", "ring.cuh",
-                                                           "ring_build.cuh", "rowwalk.h", "sell.cuh", "sellsolve.cuh",
+                                                           "ring_build.cuh", "rowwalk.h", "sell.cuh", "sellsolve.cuh", "trainplan.h",
                                                            "check.cuh")] + [
     os.path.join(ROOT, "include", "gbcg.h")]
 OUT = os.path.join(_HERE, "libgbcg.so")

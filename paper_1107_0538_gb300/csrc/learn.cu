@@ -50,6 +50,7 @@
 #include "handle.h"
 #include "lowprec.h"
 #include "sellsolve.cuh"
+#include "trainplan.h"
 
 using namespace gbcg;
 
@@ -1687,39 +1688,47 @@ __global__ void __launch_bounds__(kCT) wgrad1_kernel(WgArgs W) {
     }
 }
 
-// The partial gradients of a mini-batch: one array of CTAs per lane.
-constexpr int kTrainLanes = 4;
+// The partial gradients of up to kTrainSlots slots of a mini-batch
+// (trainplan.h): one array of CTAs per lane.
 struct GradParts {
-    const float *part[kTrainLanes];
-    double *scal[kTrainLanes];   // the lanes' scalars; [2]: loss sum
+    const float *part[kTrainSlots];
+    double *scal[kTrainSlots];   // the lanes' scalars; [2]: loss sum
     int lanes, ctas;
 };
 
-// grad += sum over lanes and CTAs of the parts, in a fixed order: thread (g, j)
-// of a block adds every kRedGroups-th CTA's entry j, then the groups are added
-// in order.  The 16 x 16 weight's entries are [t][o][c] in the parts.  The
-// lanes' loss sums go to loss[0] and are cleared.
+// grad += each lane's sum over its CTAs, lane by lane, all in a fixed order:
+// thread (g, j) of a block adds every kRedGroups-th CTA's entry j, then a warp
+// per lane adds the groups in order.  The 16 x 16 weight's entries are [t][o][c]
+// in the parts.  The lanes' loss sums go to loss[0] and are cleared.
 constexpr int kRedGroups = 32;
 __global__ void __launch_bounds__(32 * kRedGroups) grad_reduce_kernel(GradParts P, float *grad, double *loss) {
-    __shared__ float sum[kRedGroups][32];
+    __shared__ float sum[kTrainSlots][kRedGroups][32];
+    __shared__ float total[kTrainSlots][32];
     const int jl = threadIdx.x & 31, g = threadIdx.x >> 5, j = blockIdx.x * 32 + jl;
-    float s = 0.0f;
-    if (j < CG_LEARN_PARAMS)
-        for (int l = 0; l < P.lanes; ++l)
+    for (int l = 0; l < P.lanes; ++l) {
+        float s = 0.0f;
+        if (j < CG_LEARN_PARAMS)
 #pragma unroll 8
             for (int c = g; c < P.ctas; c += kRedGroups) s += P.part[l][(size_t)c * CG_LEARN_PARAMS + j];
-    sum[g][jl] = s;
+        sum[l][g][jl] = s;
+    }
+    __syncthreads();
+    if (g < P.lanes) {
+        float t = sum[g][0][jl];
+#pragma unroll
+        for (int k = 1; k < kRedGroups; ++k) t += sum[g][k][jl];
+        total[g][jl] = t;
+    }
     __syncthreads();
     if (g == 0 && j < CG_LEARN_PARAMS) {
-        float t = sum[0][jl];
-#pragma unroll
-        for (int k = 1; k < kRedGroups; ++k) t += sum[k][jl];
         int dst = j;
         if (j >= kOffW2 && j < kOffWg) {
             const int tap = (j - kOffW2) / (kCh * kCh), oc = (j - kOffW2) % (kCh * kCh);
             dst = kOffW2 + oc * kTaps + tap;
         }
-        grad[dst] += t;
+        float t = grad[dst];
+        for (int l = 0; l < P.lanes; ++l) t += total[l][jl];
+        grad[dst] = t;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0)
         for (int l = 0; l < P.lanes; ++l) {
@@ -1813,8 +1822,8 @@ struct cg_net {
     void *block = nullptr;
     long long step = 0;
     // training workspace (allocated on first use, for one grid): up to
-    // kTrainLanes lanes, each with its own stream, work on the pairs of a
-    // mini-batch in turn, because the kernels of one pair leave SMs idle
+    // kTrainSlots lanes, each with its own stream, work on the pairs of a
+    // mini-batch (trainplan.h), because the kernels of one pair leave SMs idle
     // (at 50^3 a convolution is 364 CTAs where 456 to 608 fit)
     struct TrainLane {
         cudaStream_t stream = nullptr;
@@ -2197,7 +2206,7 @@ int ensure_train(cg_net *net, const Geo &G, int ninst_ctas, int batch) {
         if (rc != CG_OK) return rc;
         net->have_train = true;
     }
-    const size_t want = (size_t)std::min(kTrainLanes, std::max(batch, 1));
+    const size_t want = (size_t)std::min(kTrainSlots, std::max(batch, 1));
     while (net->lanes.size() < want) {
         net->lanes.emplace_back();
         const int rc = alloc_lane(net, G, ninst_ctas, net->lanes.back());
@@ -2322,10 +2331,9 @@ void enqueue_sample(cg_net *net, cg_net::TrainLane &N, bool first, cg_handle *h,
 }
 
 // Losses and gradients of the pairs order[0 .. count): added to net->d.grad and
-// net->scal[2] on net->stream, pair k on lane k mod lanes.
+// net->scal[2] on net->stream.
 int enqueue_batch(cg_net *net, const cg_learn_set *set, const int64_t *order, int count) {
     const Geo &G = set->inst[0]->learn->G;
-    const int lanes = (int)std::min<size_t>(net->lanes.size(), (size_t)count);
     // the gates of every instance among the pairs, once
     std::vector<const cg_handle *> seen;
     for (int k = 0; k < count; ++k) {
@@ -2335,25 +2343,29 @@ int enqueue_batch(cg_net *net, const cg_learn_set *set, const int64_t *order, in
         launch_gates(h->learn, net, net->stream);
     }
     if (!net->fork && cudaEventCreateWithFlags(&net->fork, cudaEventDisableTiming) != cudaSuccess) return CG_ECUDA;
-    if (cudaEventRecord(net->fork, net->stream) != cudaSuccess) return CG_ECUDA;
-    for (int l = 0; l < lanes; ++l)
-        if (cudaStreamWaitEvent(net->lanes[l].stream, net->fork, 0) != cudaSuccess) return CG_ECUDA;
-    for (int k = 0; k < count; ++k) {
-        const int64_t idx = order[k];
-        cg_handle *h = set->inst[set->pair_inst[idx]];
-        enqueue_sample(net, net->lanes[k % lanes], k < lanes, h, set->r + (size_t)idx * G.n, set->e + (size_t)idx * G.n);
+    for (const TrainRound &R : plan_training(count, (int)net->lanes.size())) {
+        // after the gates, and after the round before has been added up
+        if (cudaEventRecord(net->fork, net->stream) != cudaSuccess) return CG_ECUDA;
+        for (int l = 0; l < R.lanes; ++l)
+            if (cudaStreamWaitEvent(net->lanes[l].stream, net->fork, 0) != cudaSuccess) return CG_ECUDA;
+        for (const TrainPair &t : R.pairs) {
+            const int64_t idx = order[t.pair];
+            cg_handle *h = set->inst[set->pair_inst[idx]];
+            enqueue_sample(net, net->lanes[t.lane], t.first, h, set->r + (size_t)idx * G.n, set->e + (size_t)idx * G.n);
+        }
+        GradParts P{};
+        P.lanes = R.lanes;
+        P.ctas = net->wg_ctas;
+        for (int l = 0; l < R.lanes; ++l) {
+            if (cudaEventRecord(net->lanes[l].done, net->lanes[l].stream) != cudaSuccess ||
+                cudaStreamWaitEvent(net->stream, net->lanes[l].done, 0) != cudaSuccess)
+                return CG_ECUDA;
+            P.part[l] = net->lanes[l].part;
+            P.scal[l] = net->lanes[l].scal;
+        }
+        grad_reduce_kernel<<<(CG_LEARN_PARAMS + 31) / 32, 32 * kRedGroups, 0, net->stream>>>(P, net->d.grad,
+                                                                                           net->scal + 2);
     }
-    GradParts P{};
-    P.lanes = lanes;
-    P.ctas = net->wg_ctas;
-    for (int l = 0; l < lanes; ++l) {
-        if (cudaEventRecord(net->lanes[l].done, net->lanes[l].stream) != cudaSuccess ||
-            cudaStreamWaitEvent(net->stream, net->lanes[l].done, 0) != cudaSuccess)
-            return CG_ECUDA;
-        P.part[l] = net->lanes[l].part;
-        P.scal[l] = net->lanes[l].scal;
-    }
-    grad_reduce_kernel<<<(CG_LEARN_PARAMS + 31) / 32, 32 * kRedGroups, 0, net->stream>>>(P, net->d.grad, net->scal + 2);
     return cudaGetLastError() == cudaSuccess ? CG_OK : CG_ECUDA;
 }
 
