@@ -640,7 +640,10 @@ __device__ __forceinline__ void ring_entries(const BatchParams &B, const int *of
     for (int u = 0; u < N; ++u) {
         // a row without the offset adds nothing, whatever another system holds there
         const float v = (float)vals[32 * u];
-        if (v != 0.0f) sum = fma_acc(v, zr[u], sum);
+        if (v != 0.0f) {
+            bchk(row + o[u], B.P.n);   // the index before it was clamped
+            sum = fma_acc(v, zr[u], sum);
+        }
     }
 }
 

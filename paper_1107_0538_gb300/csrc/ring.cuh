@@ -210,6 +210,11 @@ __device__ __forceinline__ void ring_fma(LoAccStored &a, int k, const VT *v, flo
     if (stored) ring_fma(static_cast<LoAcc &>(a), k, v, z);
 }
 
+// Whether a slice's value is other than zero.
+__device__ __forceinline__ bool ring_adds(int2 v) { return v.x != 0 || v.y != 0; }
+__device__ __forceinline__ bool ring_adds(float v) { return v != 0.0f; }
+__device__ __forceinline__ bool ring_adds(__nv_bfloat16 v) { return __bfloat162float(v) != 0.0f; }
+
 // Adds the N entries at offs, vals: all gathers in flight, then the products.
 template <int N, class VT, class ZT, class Acc>
 __device__ __forceinline__ void ring_batch(const RingMatrix &R, const int *offs, const VT *vals, unsigned int rowb,
@@ -220,6 +225,10 @@ __device__ __forceinline__ void ring_batch(const RingMatrix &R, const int *offs,
     ZT zr[N];
 #pragma unroll
     for (int u = 0; u < N; ++u) zr[u] = ring_gather(R, z, rowb + (unsigned int)o[u]);
+#ifdef GBCG_BOUNDS_CHECK
+    for (int u = 0; u < N; ++u)   // an entry that adds something reads a row's value, not the margin
+        if (ring_adds(vals[32 * u])) bchk((int)((rowb + (unsigned int)o[u]) / sizeof(ZT)) - R.pad, R.n);
+#endif
 #pragma unroll
     for (int u = 0; u < N; ++u) ring_fma(acc, u, vals + 32 * u, zr[u]);
 }
