@@ -12,7 +12,7 @@ namespace gbcg {
 constexpr int kSellSolveThreads = 1024;
 constexpr int kSellUnrollMem = 18;   // loads in flight per row where rows are not held in registers
 
-// a / b to the last bit or two, for the scalars of an iteration: Newton's step
+// a / b or its neighbour in the last place, for the scalars of an iteration: Newton's step
 // for the reciprocal from a single-precision seed y (error 2^-22), folded into
 // the quotient, and one correction with the exact remainder (Markstein, "Computation
 // of elementary functions on the IBM RISC System/6000", 1990): five FP64
