@@ -40,6 +40,12 @@ constexpr int kSellThreads = 256;
 // three matrices in turn: up to 32^3 10.25 / 6.16, 50^3 20.5 / 14.4, 57^3 20.5 /
 // 17.0, 72^3 28.7 / 26.5, 80^3 and 100^3 32.9 and 57.3 either way.  Batches of 14
 // and 27 with three, two or one CTAs were slower from 40^3 on (100^3 61 to 83).
+// Half as many warps only pay with a row's rest in one batch too: entry by
+// entry, short rows fell behind the eight CTAs.  Eight / four, entry by entry / four,
+// one batch, us per call in a row: 3 entries a row, 1.2M rows 14.5 / 20.7 / 14.8 (2.4M
+// 23.1 / 36.6 / 25.5); 5-point 2000^2 49.5 / 57.8 / 51.6; 7-point 90^3 16.8 / 20.5 / 16.6;
+// 21 entries, 1.2M rows 55.9 / 58.2 / 53.5; Q1 72^3 29.0 / 26.2 / 24.9, 100^3 59.5 / 57.5 /
+// 55.6.  (Reading the next slice's place ahead: 2400000 x 3 24.9, but Q1 100^3 56.4.)
 constexpr int kSellBlocksPerSm = 4;
 constexpr int kSellUnroll = 9;
 
@@ -50,11 +56,52 @@ __device__ __forceinline__ T mload(const T *p, bool stream) {
     return stream ? __ldcs(p) : __ldcg(p);
 }
 
+// Entries k .. k + N - 1 of lane's row, all their loads in flight before the
+// FMAs: even ones into s0, odd ones into s1, or (TAIL) all into s0, in order.
+template <int N, bool TAIL, class Col>
+__device__ __forceinline__ void sell_batch(const SellMatrix &M, const double *vv, const Col *cc, int base, int k,
+                                           const double *__restrict__ x, double &s0, double &s1) {
+    const bool st = M.stream != 0;
+    double vr[N], xr[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        vr[u] = mload(vv + (k + u) * 32, st);
+        xr[u] = __ldg(x + bchk(base + (int)mload(cc + (k + u) * 32, st), M.n));
+    }
+#pragma unroll
+    for (int u = 0; u < N; ++u) {
+        if (!TAIL && (u & 1)) s1 = fma(vr[u], xr[u], s1);
+        else s0 = fma(vr[u], xr[u], s0);
+    }
+}
+
+// Lane's row of a slice of width w in batches of kSellUnroll, the rest in one
+// batch of its size (the branches are the warp's).
+template <class Col>
+__device__ __forceinline__ double sell_row(const SellMatrix &M, const double *vv, const Col *cc, int base, int w,
+                                           const double *__restrict__ x) {
+    double s0 = 0.0, s1 = 0.0;
+    int k = 0;
+    for (; k + kSellUnroll <= w; k += kSellUnroll) sell_batch<kSellUnroll, false>(M, vv, cc, base, k, x, s0, s1);
+    static_assert(kSellUnroll == 9, "cases below");
+    switch (w - k) {
+        case 8: sell_batch<8, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 7: sell_batch<7, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 6: sell_batch<6, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 5: sell_batch<5, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 4: sell_batch<4, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 3: sell_batch<3, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 2: sell_batch<2, true>(M, vv, cc, base, k, x, s0, s1); break;
+        case 1: sell_batch<1, true>(M, vv, cc, base, k, x, s0, s1); break;
+        default: break;
+    }
+    return s0 + s1;
+}
+
 // Row sums of the slices owned by this warp (grid-stride over slices):
 // epi.row(i, sum) for every row i < n.
 template <class Epi>
 __device__ __forceinline__ void sell_rows(const SellMatrix &M, const double *__restrict__ x, Epi &epi) {
-    const bool st = M.stream != 0;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -62,43 +109,9 @@ __device__ __forceinline__ void sell_rows(const SellMatrix &M, const double *__r
         const long long a = M.ptr[t];
         const int w = (int)((M.ptr[t + 1] - a) >> 5);
         const int row = t * 32 + lane;
-        const double *vv = M.vals + a + lane;
-        double s0 = 0.0, s1 = 0.0;
-        int k = 0;
-        if (M.cols16) {
-            const int16_t *cc = M.cols16 + a + lane;
-            for (; k + kSellUnroll <= w; k += kSellUnroll) {
-                double vr[kSellUnroll], xr[kSellUnroll];
-#pragma unroll
-                for (int u = 0; u < kSellUnroll; ++u) {
-                    vr[u] = mload(vv + (k + u) * 32, st);
-                    xr[u] = __ldg(x + bchk(row + (int)mload(cc + (k + u) * 32, st), M.n));
-                }
-#pragma unroll
-                for (int u = 0; u < kSellUnroll; ++u) {
-                    if (u & 1) s1 = fma(vr[u], xr[u], s1);
-                    else s0 = fma(vr[u], xr[u], s0);
-                }
-            }
-            for (; k < w; ++k) s0 = fma(mload(vv + k * 32, st), __ldg(x + bchk(row + (int)mload(cc + k * 32, st), M.n)), s0);
-        } else {
-            const int32_t *cc = M.cols32 + a + lane;
-            for (; k + kSellUnroll <= w; k += kSellUnroll) {
-                double vr[kSellUnroll], xr[kSellUnroll];
-#pragma unroll
-                for (int u = 0; u < kSellUnroll; ++u) {
-                    vr[u] = mload(vv + (k + u) * 32, st);
-                    xr[u] = __ldg(x + bchk(mload(cc + (k + u) * 32, st), M.n));
-                }
-#pragma unroll
-                for (int u = 0; u < kSellUnroll; ++u) {
-                    if (u & 1) s1 = fma(vr[u], xr[u], s1);
-                    else s0 = fma(vr[u], xr[u], s0);
-                }
-            }
-            for (; k < w; ++k) s0 = fma(mload(vv + k * 32, st), __ldg(x + bchk(mload(cc + k * 32, st), M.n)), s0);
-        }
-        if (row < M.n) epi.row(row, s0 + s1, 0);
+        const double sum = M.cols16 ? sell_row(M, M.vals + a + lane, M.cols16 + a + lane, row, w, x)
+                                    : sell_row(M, M.vals + a + lane, M.cols32 + a + lane, 0, w, x);
+        if (row < M.n) epi.row(row, sum, 0);
     }
 }
 
