@@ -1796,7 +1796,7 @@ int finish_solve(cg_handle *h, cg_info *info) {
 }
 
 // Sets up the one-cluster solve where the system fits it and the device can
-// run a cluster of that size.
+// run a cluster of that size (its fixed-point matrix is built after it).
 int plan_cluster_solve(cg_handle *h, const SellHost &sh) {
     const void *kern[] = {(const void *)cg_cluster_kernel<false>, (const void *)cg_cluster_kernel<true>};
     cudaFuncAttributes fa{};
@@ -2155,8 +2155,18 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
         // (48.7), 57x44x61 11.1 (18.1), 50^3 9.7 (13.8), 20^3 9.1 (13.9).
         int max_slices = 0;
         for (size_t c = 0; c + 1 < scut.size(); ++c) max_slices = std::max(max_slices, scut[c + 1] - scut[c]);
-        if (h->sell_solve && !mixed && (rc = optional_copy(h, [&] { return build_fixed(h, tot); })) != CG_OK)
-            return fail(rc);
+        const bool jacobi = opts.precond != CG_PRECOND_NONE;
+        if (h->sell_solve && !mixed) {
+            // small systems: the whole solve inside one cluster (a caller that sets
+            // the CTA count, or tests the grid barrier, gets the grid); it needs the
+            // integers, which short rows on the grid do not pay for
+            if (opts.grid_ctas == 0 && opts.debug_phantom_arrivals == 0 && (rc = plan_cluster_solve(h, sh)) != CG_OK)
+                return fail(rc);
+            if ((h->cluster_ctas > 0 || !short_rows_for_fixed((int64_t)tot, n, ctas, jacobi)) &&
+                (rc = optional_copy(h, [&] { return build_fixed(h, tot); })) != CG_OK)
+                return fail(rc);
+            if (!h->fixed_vals) h->cluster_ctas = 0;
+        }
         if (h->sell_mem && !mixed) {
             const void *k[] = {(const void *)cg_ring_kernel<false>, (const void *)cg_ring_kernel<true>};
             rc = optional_copy(h, [&] {
@@ -2166,7 +2176,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
             });
             if (rc != CG_OK) return fail(rc);
             // long rows without a ring: the tiled kernel, its rows in registers
-            if (!h->ring_blob && h->rpt > 0 && sell_walks_long_rows(sh.ptr, nnz, opts.precond != CG_PRECOND_NONE, l2)) {
+            if (!h->ring_blob && h->rpt > 0 && sell_walks_long_rows(sh.ptr, nnz, jacobi, l2)) {
                 h->sell_mem = 0;
                 h->sell_cut = nullptr;   // flexible CG too
             }
@@ -2226,11 +2236,6 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
                 if (el != cudaSuccess) return fail(cuda_fail(el));
             }
         }
-        // small systems: the whole solve inside one cluster (a caller that sets
-        // the CTA count, or tests the grid barrier, gets the grid)
-        if (h->sell_solve && h->fixed_vals && opts.grid_ctas == 0 && opts.debug_phantom_arrivals == 0 &&
-            (rc = plan_cluster_solve(h, sh)) != CG_OK)
-            return fail(rc);
     }
     if (cudaMallocHost(&h->st_host, sizeof(DevStatus)) != cudaSuccess) return fail(CG_ENOMEM);
     if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess)

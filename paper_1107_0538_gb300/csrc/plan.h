@@ -477,6 +477,18 @@ inline SellHost build_sell(int32_t n, const std::vector<int32_t> &rowptr, const 
     return S;
 }
 
+// Whether rows are too short for the integer product (fixed.cuh) in the slice
+// kernel: publishing z as integers with their bound and turning the sums back
+// costs a row as much as several FP64 FMAs.  us per iteration, integers / FP64
+// product, entries a row: 3 (150000 rows) 10.7 / 10.0, Jacobi 12.8 / 11.5; 7 10.9 / 10.7,
+// 13.0 / 12.4 (7-point 52^3 11.0 / 10.4, 12.9 / 11.9); 9 11.1 / 11.2, 13.0 / 12.8; 11 11.4 /
+// 12.2, 13.2 / 13.4; 27 13.8 / 16.0, 15.3 / 17.5.  Up to 400 rows per CTA (60000 on
+// 152) latency hides it: 3 to 9 entries within 2% either way.  The cluster kernel
+// gains from the integers at every width.
+inline bool short_rows_for_fixed(int64_t entries, int32_t n, int ctas, bool jacobi) {
+    return n > 400 * (int64_t)ctas && entries < (jacobi ? 10 : 8) * (int64_t)n;
+}
+
 // Whether long rows make SELL-32 with the vectors in memory the slower choice
 // for a system of at most four rows per thread, whose other choice is the tiled
 // kernel (it gives a long row to 32 lanes and pads nothing).  One warp walks all

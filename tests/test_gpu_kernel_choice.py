@@ -55,6 +55,24 @@ def negative_diagonal():
     return problems.CSR(A.n, A.rowptr, A.colidx, np.where((rows == 17) & (A.colidx == 17), -A.vals, A.vals))
 
 
+def points(*dims):
+    """Weighted Laplacian of a grid (5 or 7 points), shifted."""
+    idx = np.arange(int(np.prod(dims))).reshape(dims)
+    i, j = [], []
+    for ax in range(len(dims)):
+        a = np.moveaxis(idx, ax, 0)
+        i.append(a[:-1].ravel())
+        j.append(a[1:].ravel())
+    i, j = np.concatenate(i), np.concatenate(j)
+    w = np.random.default_rng(1).uniform(0.5, 1.0, i.size)
+    n = idx.size
+    d = 1e-2 + np.bincount(i, w, n) + np.bincount(j, w, n)
+    key = np.concatenate([i * n + j, j * n + i, np.arange(n) * (n + 1)])
+    order = np.argsort(key)
+    rowptr = np.searchsorted(key[order], np.arange(n + 1, dtype=np.int64) * n).astype(np.int32)
+    return problems.CSR(n, rowptr, (key[order] % n).astype(np.int32), np.concatenate([-w, -w, d])[order])
+
+
 def with_hub(A, m):
     """A with row 777 coupled to m further rows, spread over the matrix, weakly enough to stay definite."""
     rows = np.repeat(np.arange(A.n), np.diff(A.rowptr))
@@ -87,6 +105,15 @@ CASES = {
     "two_ctas": (ring["two_ctas"][0], dict(grid_ctas=2), "cg_ring_kernel/int"),
     "one_cta": (ring["one_cta"][0], dict(grid_ctas=1), "cg_ring_kernel/int"),
     "ten_ctas": (lambda: box(20, 20, 20), dict(grid_ctas=10), "cg_sell_kernel/int"),
+    # short rows: integers only where they make the cluster possible
+    "7point20": (lambda: points(20, 20, 20), {}, "cg_cluster_kernel/int"),
+    "7point40": (lambda: points(40, 40, 40), {}, "cg_sell_kernel/fp64"),
+    "7point38": (lambda: points(38, 38, 38), {}, "cg_sell_kernel/int"),     # 361 rows per CTA
+    "width7": (lambda: test_fixed.banded(3000, 7, 1), dict(grid_ctas=4), "cg_sell_kernel/fp64"),
+    "width7_8_ctas": (lambda: test_fixed.banded(3000, 7, 1), dict(grid_ctas=8), "cg_sell_kernel/int"),
+    "width9": (lambda: test_fixed.banded(3000, 9, 1), dict(grid_ctas=4), "cg_sell_kernel/int"),
+    "width9_jacobi": (lambda: test_fixed.banded(3000, 9, 1), dict(grid_ctas=4, precond=1), "cg_sell_kernel/fp64"),
+    "width11_jacobi": (lambda: test_fixed.banded(3000, 11, 1), dict(grid_ctas=4, precond=1), "cg_sell_kernel/int"),
     # limits of the integer product
     "width31": (fixed["width31"][0], dict(grid_ctas=152), "cg_sell_kernel/int"),
     "width33": (fixed["width33"][0], dict(grid_ctas=152), "cg_sell_kernel/fp64"),
