@@ -2171,6 +2171,7 @@ int cg_create(const cg_csr *A, const cg_opts *opts_in, void *stream, cg_handle *
             const void *k[] = {(const void *)cg_ring_kernel<false>, (const void *)cg_ring_kernel<true>};
             rc = optional_copy(h, [&] {
                 bool ok = false;
+                if (short_rows_for_ring((int64_t)tot, n, jacobi)) return (int)CG_OK;
                 const int r = fixed_scales(h, &ok);
                 return r == CG_OK && ok ? build_ring<int2>(h, k, 2, tot, max_slices, l2) : r;
             });

@@ -489,6 +489,15 @@ inline bool short_rows_for_fixed(int64_t entries, int32_t n, int ctas, bool jaco
     return n > 400 * (int64_t)ctas && entries < (jacobi ? 10 : 8) * (int64_t)n;
 }
 
+// Whether a Jacobi solve's rows are too short for the ring (ring.cuh), whose
+// alternative is SELL-32 with the vectors in memory and the FP64 product.  us per
+// iteration, ring / SELL-32, entries a row: 3 (340000 rows) 19.5 / 17.8, (600000) 24.5 /
+// 21.8, (1.2M) 38.6 / 39.6, (2.4M) 84.8 / 81.9; 5 (300000) 17.5 / 17.0, (600000) 25.2 / 24.0,
+// 5-point 550^2 18.6 / 17.0, 2000^2 141.6 / 136.9; 7 (600000) 25.9 / 28.7, 7-point 67^3
+// 19.4 / 19.1, 100^3 38.7 / 43.9.  Without the preconditioner the ring is as fast or faster
+// from 3 entries on (600000 rows 19.7 / 19.0, 1.2M 30.7 / 34.9).
+inline bool short_rows_for_ring(int64_t entries, int32_t n, bool jacobi) { return jacobi && entries < 6 * (int64_t)n; }
+
 // Whether long rows make SELL-32 with the vectors in memory the slower choice
 // for a system of at most four rows per thread, whose other choice is the tiled
 // kernel (it gives a long row to 32 lanes and pads nothing).  One warp walks all

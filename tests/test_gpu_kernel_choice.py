@@ -102,6 +102,9 @@ CASES = {
     "flat": (cluster["flat_box"], {}, "cg_cluster_kernel/int"),
     # a given CTA count asks for the grid
     "box8_grid": (lambda: box(8, 8, 8), dict(grid_ctas=152), "cg_sell_kernel/int"),
+    "5point": (lambda: points(90, 90), dict(grid_ctas=4), "cg_ring_kernel/int"),
+    "5point_jacobi": (lambda: points(90, 90), dict(grid_ctas=4, precond=1), "cg_sellmem_kernel/fp64"),
+    "7point_jacobi": (lambda: points(20, 20, 20), dict(grid_ctas=4, precond=1), "cg_ring_kernel/int"),
     "two_ctas": (ring["two_ctas"][0], dict(grid_ctas=2), "cg_ring_kernel/int"),
     "one_cta": (ring["one_cta"][0], dict(grid_ctas=1), "cg_ring_kernel/int"),
     "ten_ctas": (lambda: box(20, 20, 20), dict(grid_ctas=10), "cg_sell_kernel/int"),
